@@ -99,10 +99,6 @@ size_t layout_workspace(Workspace &w, char *base) {
   w.ale = (int *)take(sizeof(int) * N);
   w.scal = (double *)take(sizeof(double) * 4);
   w.scal_i = (int *)take(sizeof(int) * 4);
-  w.rowpart = tables ? (double *)take(sizeof(double) * NB * TILE * 4) : nullptr;
-  w.colpart = tables ? (double *)take(sizeof(double) * NB * TILE * 4) : nullptr;
-  w.rowcnt = tables ? (int *)take(sizeof(int) * NT) : nullptr;
-  w.colcnt = tables ? (int *)take(sizeof(int) * NT) : nullptr;
   w.status = (int *)take(sizeof(int) * 4);
   w.bk = w.blocks ? (unsigned long long *)take(sizeof(unsigned long long) * 4 * NT * TILE2) : nullptr;
   w.be = w.blocks ? (int *)take(sizeof(int) * 4 * NT * TILE2) : nullptr;

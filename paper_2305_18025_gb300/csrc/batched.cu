@@ -45,7 +45,7 @@ int evaluate_batched(bpimd_ctx *ctx, const double *pos, double *V_B, double *F) 
                             mode == BPIMD_MIXED32, V_B, s) != cudaSuccess)
     return BPIMD_ERR_CUDA;
   mark(2);
-  if (launch_prob_forces_batched(ctx->d_ws, ctx->d_blk_tab, ctx->n_blk_tab, ctx->d_off, mode, pos, F,
+  if (launch_prob_forces_batched(ctx->d_ws, ctx->d_item_tab, ctx->n_item_tab, ctx->d_off, mode, pos, F,
                                  ctx->tune_prob_bpsm, s) != cudaSuccess)
     return BPIMD_ERR_CUDA;
   mark(3);
@@ -85,7 +85,7 @@ int bpimd_create_batched(bpimd_ctx **out, const bpimd_config *cfg, int32_t R, co
   ctx->h_ws.resize(R);
   ctx->h_off.resize(R);
   // host tables
-  std::vector<int2> bead_tab, blk_tab;
+  std::vector<int2> bead_tab, blk_tab, item_tab;
   std::vector<int> order(R);
   long long off = 0;
   size_t wbytes = 0;
@@ -115,6 +115,15 @@ int bpimd_create_batched(bpimd_ctx **out, const bpimd_config *cfg, int32_t R, co
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return N[a] > N[b]; });
   ctx->h_order = order;
+  // longest partner lists first: items 2k, 2k+1 of a replica have NT - k tiles of partners
+  for (int len = ctx->h_ws[order[0]].NT; len > 0; --len)
+    for (int r : order) {
+      const int k = ctx->h_ws[r].NT - len;
+      if (k < 0) break;  // order is by decreasing N
+      item_tab.push_back(make_int2(r, 2 * k));
+      item_tab.push_back(make_int2(r, 2 * k + 1));
+    }
+  ctx->n_item_tab = (int)item_tab.size();
   ctx->n_bead_tab = (int)bead_tab.size();
   ctx->n_blk_tab = (int)blk_tab.size();
   // one allocation: workspaces, shared status word, tables
@@ -123,7 +132,8 @@ int bpimd_create_batched(bpimd_ctx **out, const bpimd_config *cfg, int32_t R, co
   const size_t o_dws = o_status + 256;
   const size_t o_bead = o_dws + align256(sizeof(Workspace) * R);
   const size_t o_blk = o_bead + align256(sizeof(int2) * bead_tab.size());
-  const size_t o_order = o_blk + align256(sizeof(int2) * blk_tab.size());
+  const size_t o_item = o_blk + align256(sizeof(int2) * blk_tab.size());
+  const size_t o_order = o_item + align256(sizeof(int2) * item_tab.size());
   const size_t o_off = o_order + align256(sizeof(int) * R);
   const size_t bytes = o_off + align256(sizeof(long long) * R);
   if (cudaMalloc(&ctx->dev_block, bytes) != cudaSuccess) {
@@ -146,6 +156,7 @@ int bpimd_create_batched(bpimd_ctx **out, const bpimd_config *cfg, int32_t R, co
   ctx->d_ws = (Workspace *)(base + o_dws);
   ctx->d_bead_tab = (int2 *)(base + o_bead);
   ctx->d_blk_tab = (int2 *)(base + o_blk);
+  ctx->d_item_tab = (int2 *)(base + o_item);
   ctx->d_order = (int *)(base + o_order);
   ctx->d_off = (long long *)(base + o_off);
   cudaStream_t s = ctx->stream;
@@ -156,6 +167,8 @@ int bpimd_create_batched(bpimd_ctx **out, const bpimd_config *cfg, int32_t R, co
                             cudaMemcpyHostToDevice, s) == cudaSuccess &&
             cudaMemcpyAsync(ctx->d_blk_tab, blk_tab.data(), sizeof(int2) * blk_tab.size(), cudaMemcpyHostToDevice,
                             s) == cudaSuccess &&
+            cudaMemcpyAsync(ctx->d_item_tab, item_tab.data(), sizeof(int2) * item_tab.size(),
+                            cudaMemcpyHostToDevice, s) == cudaSuccess &&
             cudaMemcpyAsync(ctx->d_order, order.data(), sizeof(int) * R, cudaMemcpyHostToDevice, s) == cudaSuccess &&
             cudaMemcpyAsync(ctx->d_off, ctx->h_off.data(), sizeof(long long) * R, cudaMemcpyHostToDevice, s) ==
                 cudaSuccess &&

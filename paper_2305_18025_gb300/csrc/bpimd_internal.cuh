@@ -170,11 +170,6 @@ struct Workspace {
   void *alm; int *ale;
   // scalars: [0] V_B, [1] invZ mantissa, [2] reserved ; int [0] invZ exponent
   double *scal; int *scal_i;
-  // force partial sums: rowpart/colpart [NB][TILE][4]
-  double *rowpart, *colpart;
-  // per row / column tile: number of finished blocks of the probability pass
-  // (the last block of a tile forms its forces and resets the count to 0)
-  int *rowcnt, *colcnt;
   int *status;          // device status word
   // blocked recursions (cluster kernel): per recursion and row tile, the
   // c-scaled coupling block Dc to the previous tile's unknowns and the tile
@@ -281,8 +276,8 @@ cudaError_t launch_spring_expectation_batched(const Workspace *ws, const int2 *t
 cudaError_t launch_diag_potentials(const Workspace &w, double *Vf, double *Vb, cudaStream_t s);
 
 // Replica batches: ws[r] is replica r's workspace (device array); block tables
-// hold (replica, particle block) for the bead pass and (replica, g block) for
-// the pair factors and the probability pass; off[r] is the element offset of
+// hold (replica, particle block) for the bead pass, (replica, g block) for the
+// pair factors and (replica, row or column tile item) for the exterior forces; off[r] is the element offset of
 // replica r in the packed position/force arrays; order lists replicas by
 // decreasing N.
 // bead pass (bead_tab: (replica, first particle)) and pair factors (blk_tab:

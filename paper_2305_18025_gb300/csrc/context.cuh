@@ -38,7 +38,8 @@ struct bpimd_ctx {
   std::vector<long long> h_off;           // element offset of each replica
   bpimd::Workspace *d_ws;                 // device copies of h_ws
   int2 *d_bead_tab, *d_blk_tab;           // (replica, particle block), (replica, g block)
-  int n_bead_tab, n_blk_tab;
+  int2 *d_item_tab;                       // (replica, tile item of the exterior forces), longest first
+  int n_bead_tab, n_blk_tab, n_item_tab;
   int *d_order;                           // replicas by decreasing N
   std::vector<int> h_order;               // the same order on the host
   int n_big;                              // replicas above BATCH_MAX_N (first in the order)

@@ -3,23 +3,14 @@
 //   Pr[l -> u] (u <= l) = y_{u-1} g(u,l) mu_l / (N y_N)     (Eq. close-cycle-probability)
 //   Pr[l -> l+1]        = 1 - y_l B_{l+1} / (N y_N)          (Eq. direct-link-probability)
 //   Pr[l -> u]          = 0 for u > l+1                      (Lemma zero-connection-probability)
-// The N x N matrix is never stored: each 32x32 block of the lower triangle is
-// generated from the stored pair factors g and reduced on the spot into
-//   row l    : sum_u Pr[l->u],  sum_u Pr[l->u] (r_l^P - r_u^1)    (bead P of l)
-//   column u : sum_l Pr[l->u],  sum_l Pr[l->u] (r_u^1 - r_l^P)    (bead 1 of u)
-// partial sums per block.  Each block then counts itself in its row tile and
-// its column tile (an atomic counter per tile); the block that completes a
-// tile adds that tile's partials in a fixed block order (so the result does
-// not depend on which block finishes last), adds the direct-link term and
+// The N x N matrix is never stored: the pass goes by tiles of 32 particles and
 // forms (Eq. force-on-1-sum-neighbors, Eq. force-on-P-sum-neighbors)
 //   F_l^P = -m w_P^2 [ (sum_u Pr[l->u]) (r_l^P - r_l^{P-1}) + sum_u Pr[l->u] (r_l^P - r_u^1) ]
 //   F_l^1 = -m w_P^2 [ (sum_l' Pr[l'->l]) (r_l^1 - r_l^2) + sum_l' Pr[l'->l] (r_l^1 - r_l'^P) ]
 // i.e. the per-neighbour sums of the paper distributed over their terms.
-// Precision forms: FP64 in float64 throughout.  MIXED (prob_block_mixed):
-// Pr from 64-bit integer mantissa products, products with the float32 bead
-// differences and all sums as compensated float32 pairs.  MIXED32: bead
-// differences from float32 high/low parts, block-local products and sums in
-// float32, the combination across blocks with float32 TwoSum compensation.
+// Precision forms: bead differences in float64 (FP64) or float32 (mixed
+// forms, from the high/low parts or the fixed-point copies); products and sums
+// on 64-bit integer mantissas, the direct links and the results in float64.
 #include <type_traits>
 
 #include "bpimd_internal.cuh"
@@ -47,24 +38,6 @@ __device__ __forceinline__ xd mu_of(const Workspace &w, int b) {
   return xd{w.ybm[r], w.ybe[r]};
 }
 
-// Sum of float32 block partials, in the given order, to float64 accuracy on
-// the float32 pipe: Knuth's TwoSum splits every addition into its rounded sum
-// and exact rounding error, and the errors are carried alongside (float64
-// additions would queue on the SM's slow float64 pipe: 16 per thread here).
-struct fsum2 {
-  float s = 0.0f, c = 0.0f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = s + v, bp = t - s;
-    c += (s - (t - bp)) + (v - bp);
-    s = t;
-  }
-  __device__ __forceinline__ void add2(float h, float l) {  // an unevaluated sum h + l
-    add(h);
-    c += l;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-
 // 2^e as a double for e in the normal range (0 below it), built from the bits.
 __device__ __forceinline__ double pow2_normal(int e) {
   return e < -1022 ? 0.0 : __longlong_as_double((long long)(min(e, 1023) + 1023) << 52);
@@ -84,616 +57,401 @@ __device__ __forceinline__ double img(const Workspace &w, double d) {
   return PBC ? d - w.L * rint(d * w.invL) : d;
 }
 
-// Bead P of the 32 particles of row tile t: sum the row partials of blocks
-// (t, 0..t) in that order, add the direct link, form F_l^P.  Run by the last
-// block of the tile to finish; all 256 threads call it.  The finishing warp's
-// loads are issued before the partial sums.
-// Kinds of block partials: float64, float32, or an unevaluated float32 pair
-// (high, low) written by the MIXED pass.
-constexpr int PK_F64 = 0, PK_F32 = 1, PK_FF = 2;
+// ------------------------------------------- exterior forces by whole tiles
+// Item 2k is row tile NT-1-k (bead P of its 32 particles b, against every
+// source a <= b), item 2k+1 column tile k (bead 1 of its 32 particles a,
+// against every b >= a): decreasing sizes.  A lane owns one particle; the
+// partners are dealt out in chunks over the item's cluster (CL CTAs) and
+// staged in shared memory, a warp taking an eighth of a chunk.  With mu_b and
+// 1/(N y_N) taken out of a row's sum, and y_a and 1/(N y_N) out of a column's,
+//   row b    : mu_b / (N y_N) sum_a y_a g(a,b) (r_b^P - r_a^1)
+//   column a : y_a / (N y_N) sum_b mu_b g(a,b) (r_b^P - r_a^1)
+// a pair is one product and three products with the difference's components.
+//   Mixed forms: unevaluated float32 pairs (products by FMA, sums by TwoSum:
+//   2^-46 relative) on the float32 pipe; the powers of two of all factors,
+//   the taken-out ones included, scale the pair, so a term is at most 2.
+//   FP64: 64-bit integer mantissas, signed 64-bit sums with one running
+//   exponent a lane (2^-60 of the largest term of a group of four); GB300's
+//   float64 pipe retires ~1.7 lanes a clock, so it forms the differences only.
+// The sums of the probabilities themselves are not needed: by the recursions'
+// own equations sum_u Pr[l->u] + Pr[l->l+1] = 1, and so for the columns.
+// Partial sums meet in shared memory, then in the cluster's first CTA, in a
+// fixed order: nothing O(N^2) is written, and there are no atomics.
+// Each pair is formed twice (row and column), which costs less than the
+// transposed reduction, the global partial sums, the fence and the counters
+// of a pass that forms it once.
+struct PSum {  // FP64: sum_c = v[c] 2^(E - 61)
+  long long v[3];
+  int E;
+};
 
-template <int PK, bool PBC>
-__device__ void finalize_rows(const Workspace &w, int t, const double *__restrict__ pos, double *__restrict__ F,
-                              double (*fin)[9]) {
-  const int q = threadIdx.x & 3, jj = (threadIdx.x >> 2) & 31, half = threadIdx.x >> 7;
-  const int p = t * TILE + threadIdx.x;
-  const bool mine = threadIdx.x < TILE && p < w.N;
-  double M = 0.0, rp[3] = {0, 0, 0}, n1[3] = {0, 0, 0}, nb[3] = {0, 0, 0};
-  if (mine) {
-    const double *r = w.RP + 4 * (size_t)p, *nbP = pos + ((size_t)p * w.P + (w.P - 2)) * 3;  // bead P-1 (1-based)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) { rp[c] = r[c]; nb[c] = nbP[c]; }
-    if (p + 1 < w.N) {
-      const double *n = w.R1 + 4 * (size_t)(p + 1);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) n1[c] = n[c];
-    }
-  }
-  const size_t base = (size_t)t * (t + 1) / 2;
-  using P_t = typename std::conditional<PK == PK_F64, double, typename std::conditional<PK == PK_F32, float, float2>::type>::type;
-  const P_t *part = (const P_t *)w.rowpart;
-  double acc = 0.0;
-  fsum2 f;
-  // partials in chunks of 8 per thread, all loads of a chunk issued first;
-  // the direct link's float64 chain runs while the first chunk is in flight
-  for (int s0 = half; s0 <= t; s0 += 16) {
-    P_t v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {  // index clamped into the tile: a valid address even if the load is speculated
-      const int k = min(s0 + 2 * u, t);
-      v[u] = (s0 + 2 * u <= t) ? __ldcg(part + ((base + k) * TILE + jj) * 4 + q) : P_t{};
-    }
-    if (s0 == half && mine && p + 1 < w.N) M = direct_link_fast(w, p);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if constexpr (PK == PK_F32) f.add(v[u]);
-      else if constexpr (PK == PK_FF) f.add2(v[u].x, v[u].y);
-      else acc += v[u];
-    }
-  }
-  fin[jj][q + 4 * half] = PK == PK_F64 ? acc : f.value();
-  __syncthreads();
-  if (mine) {
-    const double *fr = fin[threadIdx.x];
-    double rs = fr[0] + fr[4] + M, r3[3] = {fr[1] + fr[5], fr[2] + fr[6], fr[3] + fr[7]};
-    const double k = w.k;
-    double *fP = F + ((size_t)p * w.P + (w.P - 1)) * 3;
-    bool ok = true;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double rc = fma(M, img<PBC>(w, rp[c] - n1[c]), r3[c]);
-      fP[c] = -k * fma(rs, img<PBC>(w, rp[c] - nb[c]), rc);
-      ok &= isfinite(fP[c]);
-    }
-    if (!ok) atomicOr(w.status, ST_NONFINITE);
-  }
-  if (threadIdx.x == 0) w.rowcnt[t] = 0;  // ready for the next evaluation
-  __syncthreads();
+__device__ __forceinline__ unsigned long long mant64(double m) {  // [1, 2) -> [2^63, 2^64)
+  return ((unsigned long long)__double_as_longlong(m) << 11) | (1ull << 63);
 }
 
-// Bead 1 of the 32 particles of column tile s: blocks (s..NT-1, s) in order.
-template <int PK, bool PBC>
-__device__ void finalize_cols(const Workspace &w, int s, const double *__restrict__ pos, double *__restrict__ F,
-                              double (*fin)[9]) {
-  const int q = threadIdx.x & 3, ii = (threadIdx.x >> 2) & 31, half = threadIdx.x >> 7;
-  const int p = s * TILE + threadIdx.x;
-  const bool mine = threadIdx.x < TILE && p < w.N;
-  double M = 0.0, r1[3] = {0, 0, 0}, pP[3] = {0, 0, 0}, nb[3] = {0, 0, 0};
-  if (mine) {
-    const double *r = w.R1 + 4 * (size_t)p, *nb1 = pos + ((size_t)p * w.P + 1) * 3;  // bead 2 (1-based)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) { r1[c] = r[c]; nb[c] = nb1[c]; }
-    if (p >= 1) {
-      const double *n = w.RP + 4 * (size_t)(p - 1);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) pP[c] = n[c];
-    }
-  }
-  using P_t = typename std::conditional<PK == PK_F64, double, typename std::conditional<PK == PK_F32, float, float2>::type>::type;
-  const P_t *part = (const P_t *)w.colpart;
-  double acc = 0.0;
-  fsum2 f;
-  for (int t0 = s + half; t0 < w.NT; t0 += 16) {
-    P_t v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int t = min(t0 + 2 * u, w.NT - 1);  // clamped into the tile: a valid address even if speculated
-      v[u] = (t0 + 2 * u < w.NT) ? __ldcg(part + (((size_t)t * (t + 1) / 2 + s) * TILE + ii) * 4 + q) : P_t{};
-    }
-    if (t0 == s + half && mine && p >= 1) M = direct_link_fast(w, p - 1);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if constexpr (PK == PK_F32) f.add(v[u]);
-      else if constexpr (PK == PK_FF) f.add2(v[u].x, v[u].y);
-      else acc += v[u];
-    }
-  }
-  fin[ii][q + 4 * half] = PK == PK_F64 ? acc : f.value();
-  __syncthreads();
-  if (mine) {
-    const double *fc = fin[threadIdx.x];
-    double cs = fc[0] + fc[4] + M, c3[3] = {fc[1] + fc[5], fc[2] + fc[6], fc[3] + fc[7]};
-    const double k = w.k;
-    double *f1 = F + (size_t)p * w.P * 3;
-    bool ok = true;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double cc = fma(M, img<PBC>(w, r1[c] - pP[c]), c3[c]);
-      f1[c] = -k * fma(cs, img<PBC>(w, r1[c] - nb[c]), cc);
-      ok &= isfinite(f1[c]);
-    }
-    if (!ok) atomicOr(w.status, ST_NONFINITE);
-  }
-  if (threadIdx.x == 0) w.colcnt[s] = 0;
-  __syncthreads();
+// |x| as a mantissa in [2^62, 2^63) (value M 2^(e - 62)) times the term t:
+// the high product, its exponent e, its sign; a zero has the exponent NO_TERM
+constexpr int NO_TERM = -(1 << 30);
+__device__ __forceinline__ unsigned long long diff_term(unsigned long long t, double x, int &e, int &sgn, int &bad) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int hi = (int)(b >> 32), ex = (hi >> 20) & 0x7ff;
+  sgn = hi >> 31;
+  e = ex ? ex - 1023 : NO_TERM;
+  bad |= ex == 0x7ff;
+  return __umul64hi(t, ((b << 10) & 0x3FFFFFFFFFFFFFFFull) | (1ull << 62));
 }
 
-// One 32 x 32 block of the lower triangle (all 256 threads of the CTA).
-// MIXED keeps the block partials in float32 (each is a float32 sum already).
-template <bool MIXED, bool PBC>
-__device__ __forceinline__ void prob_block(const Workspace &w, int blk, const double *__restrict__ pos,
-                                           double *__restrict__ F,
-                                           typename std::conditional<MIXED, float, double>::type (*red)[32][4],
-                                           double (*fin)[9], int *last) {
-  using P_t = typename std::conditional<MIXED, float, double>::type;
-  {
-    int t, s;
-    block_coords_f(blk, t, s);
-    const int j = threadIdx.x & 31, i0 = threadIdx.x >> 5;
-    const int b = t * TILE + j;
-    const bool bvalid = b < w.N;
-    xd mub{0.0, XZERO_E};
-    double bx = 0, by = 0, bz = 0;
-    float4 bh = make_float4(0.f, 0.f, 0.f, 0.f), bl = bh;
-    if (bvalid) {
-      mub = mu_of(w, b);
-      if (MIXED) {
-        bh = *(const float4 *)(w.RPs + 8 * (size_t)b);
-        bl = *(const float4 *)(w.RPs + 8 * (size_t)b + 4);
-      } else {
-        bx = w.RP[4 * b]; by = w.RP[4 * b + 1]; bz = w.RP[4 * b + 2];
-      }
-    }
-    const float mubf = (float)mub.m;
-    double rs = 0, rx = 0, ry = 0, rz = 0;  // row partials (thread's 4 entries)
-    float frs = 0, frx = 0, fry = 0, frz = 0;
+// stores into the cluster's first CTA, and the cluster barrier
+__device__ __forceinline__ unsigned first_cta(const void *p) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)));
+  return r;
+}
+__device__ __forceinline__ void cluster_store(const void *p, long long v) {
+  asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(first_cta(p)), "l"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_store(const void *p, int v) {
+  asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(first_cta(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_store(const void *p, float v) { cluster_store(p, __float_as_int(v)); }
+__device__ __forceinline__ void cluster_arrive_release() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait_acquire() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ long long shift_in(long long v, int k) { return v >> min(k, 63); }
+
+// a + b, |b| < 2^62; |a| stays below 2^62
+__device__ __forceinline__ void psum_add(PSum &a, const PSum &b) {
+  const int E = max(a.E, b.E), ka = E - a.E, kb = E - b.E;
+  bool big = false;
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      const int i = i0 + 8 * kk;
-      const int a = s * TILE + i;
-      const size_t gi = (size_t)blk * TILE2 + i * TILE + j;
-      const bool valid = bvalid && a <= b;
-      double cs = 0, cx = 0, cy = 0, cz = 0;
-      float fcs = 0, fcx = 0, fcy = 0, fcz = 0;
-      if (valid) {
-        if (MIXED) {
-          float fx, fy, fz;
-          if (PBC) {  // minimum image from the fixed-point copies (bh holds RP's bits)
-            const uint4 ua = *(const uint4 *)(w.R1s + 8 * (size_t)a);
-            fx = fixdiff(__float_as_uint(bh.x), ua.x, w.Lscale);
-            fy = fixdiff(__float_as_uint(bh.y), ua.y, w.Lscale);
-            fz = fixdiff(__float_as_uint(bh.z), ua.z, w.Lscale);
-          } else {
-            const float4 ah = *(const float4 *)(w.R1s + 8 * (size_t)a);
-            const float4 al4 = *(const float4 *)(w.R1s + 8 * (size_t)a + 4);
-            fx = (bh.x - ah.x) + (bl.x - al4.x);
-            fy = (bh.y - ah.y) + (bl.y - al4.y);
-            fz = (bh.z - ah.z) + (bl.z - al4.z);
-          }
-          const float gmf = ((const float *)w.gm)[gi];
-          const int e = ((const int *)w.ale)[a] + mub.e + w.ge[gi];
-          float M = ((const float *)w.alm)[a] * mubf * gmf;
-          M = (e < -150) ? 0.0f : (e > 0 ? M * (float)(1 << min(e, 2)) : M * pow2f_nonpos(e));
-          frs += M; frx += M * fx; fry += M * fy; frz += M * fz;
-          fcs = M; fcx = -M * fx; fcy = -M * fy; fcz = -M * fz;
-        } else {
-          const double dx = img<PBC>(w, bx - w.R1[4 * a]), dy = img<PBC>(w, by - w.R1[4 * a + 1]),
-                       dz = img<PBC>(w, bz - w.R1[4 * a + 2]);
-          const double gmd = ((const double *)w.gm)[gi];
-          // alpha mu g with its exponent applied as an integer-built power of two
-          const double M = (((const double *)w.alm)[a] * mub.m * gmd) * pow2_normal(w.ale[a] + mub.e + w.ge[gi]);
-          rs += M; rx = fma(M, dx, rx); ry = fma(M, dy, ry); rz = fma(M, dz, rz);
-          cs = M; cx = -M * dx; cy = -M * dy; cz = -M * dz;
-        }
-      }
-      // column a: reduce over the 32 lanes (b)
-      if (MIXED) {
+  for (int c = 0; c < 3; ++c) {
+    a.v[c] = shift_in(a.v[c], ka) + shift_in(b.v[c], kb);
+    const int h = (int)(a.v[c] >> 32);
+    big |= (h ^ (h >> 31)) >= (1 << 30);
+  }
+  a.E = E;
+  if (big) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          fcs += __shfl_xor_sync(0xffffffffu, fcs, o);
-          fcx += __shfl_xor_sync(0xffffffffu, fcx, o);
-          fcy += __shfl_xor_sync(0xffffffffu, fcy, o);
-          fcz += __shfl_xor_sync(0xffffffffu, fcz, o);
-        }
-      } else {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          cs += __shfl_xor_sync(0xffffffffu, cs, o);
-          cx += __shfl_xor_sync(0xffffffffu, cx, o);
-          cy += __shfl_xor_sync(0xffffffffu, cy, o);
-          cz += __shfl_xor_sync(0xffffffffu, cz, o);
-        }
-      }
-      if (j == 0) {
-        P_t *cp = (P_t *)w.colpart + ((size_t)blk * TILE + i) * 4;
-        if (MIXED) { cp[0] = fcs; cp[1] = fcx; cp[2] = fcy; cp[3] = fcz; }
-        else { cp[0] = (P_t)cs; cp[1] = (P_t)cx; cp[2] = (P_t)cy; cp[3] = (P_t)cz; }
-      }
-    }
-    if (MIXED) {
-      red[i0][j][0] = frs; red[i0][j][1] = frx; red[i0][j][2] = fry; red[i0][j][3] = frz;
+    for (int c = 0; c < 3; ++c) a.v[c] >>= 1;
+    a.E += 1;
+  }
+}
+
+// Mixed forms: s + c with every rounding error of s in c
+__device__ __forceinline__ void two_sum(float &s, float &c, float x) {
+  const float t = s + x, bp = t - s;
+  c += (s - (t - bp)) + (x - bp);
+  s = t;
+}
+// a mantissa in [1, 2) as float32 high and low parts (23 + 23 fraction bits)
+__device__ __forceinline__ void mant_hl(double m, float &h, float &l) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(m);
+  h = __uint_as_float(0x3F800000u | ((unsigned)(b >> 29) & 0x7FFFFFu));
+  l = (__uint_as_float(0x4B000000u | ((unsigned)(b >> 6) & 0x7FFFFFu)) - 8388608.0f) * 1.4210854715202004e-14f;  // 2^-46
+}
+__device__ __forceinline__ void mant_hl(float m, float &h, float &l) {
+  h = m;
+  l = 0.0f;
+}
+
+constexpr int PROB_THREADS = 256, PROB_WARPS = PROB_THREADS / 32;
+constexpr int PROB_MAX_CL = 8;
+constexpr int PROB_CHUNK = 256;  // most partners staged at a time
+
+// Sums of a warp or a CTA: mixed forms (s, c) per component, FP64 v, E and the
+// non-finite flag.
+template <bool F64>
+struct SumSlot;
+template <>
+struct SumSlot<false> {
+  float s[3][TILE], c[3][TILE];
+};
+template <>
+struct SumSlot<true> {
+  long long v[3][TILE];
+  int E[TILE], bad[TILE];
+};
+// Staged partners.  Mixed forms: the endpoint's high and low parts (or, in a
+// box, its fixed-point words) with the weight's mantissa parts in the fourth
+// places; FP64: coordinates and the weight's 64-bit mantissa.
+template <bool F64>
+struct Partners;
+template <>
+struct Partners<false> {
+  float4 h[PROB_CHUNK], l[PROB_CHUNK];
+  int e[PROB_CHUNK];
+};
+template <>
+struct Partners<true> {
+  double x[PROB_CHUNK], y[PROB_CHUNK], z[PROB_CHUNK];
+  unsigned long long m[PROB_CHUNK];
+  int e[PROB_CHUNK];
+};
+template <bool F64>
+struct ProbSmem {
+  Partners<F64> part;
+  SumSlot<F64> warp[PROB_WARPS];
+  SumSlot<F64> cta[PROB_MAX_CL];  // in the cluster's first CTA
+  double base[3][TILE];
+};
+
+// y_q (row items' partners, column items' own) or mu_q
+__device__ __forceinline__ xd weight_y(const Workspace &w, int q) { return xd{__ldg(w.yfm + q), __ldg(w.yfe + q)}; }
+__device__ __forceinline__ xd weight_mu(const Workspace &w, int q) {
+  return xd{__ldg(w.ybm + (w.N - 1 - q)), __ldg(w.ybe + (w.N - 1 - q))};
+}
+
+template <bool F64, bool PBC>
+__device__ __forceinline__ void stage_partner(const Workspace &w, Partners<F64> &P, int i, int q, bool beadP, xd wt) {
+  const auto ep = pairg::load_end<!F64, PBC>(w, q, beadP);
+  if constexpr (F64) {
+    P.x[i] = ep.x;
+    P.y[i] = ep.y;
+    P.z[i] = ep.z;
+    P.m[i] = mant64(wt.m);
+  } else {
+    float h, l;
+    mant_hl(wt.m, h, l);
+    if constexpr (PBC) {
+      P.h[i] = make_float4(__uint_as_float(ep.u.x), __uint_as_float(ep.u.y), __uint_as_float(ep.u.z), h);
+      P.l[i].w = l;
     } else {
-      red[i0][j][0] = (P_t)rs; red[i0][j][1] = (P_t)rx; red[i0][j][2] = (P_t)ry; red[i0][j][3] = (P_t)rz;
-    }
-    __syncthreads();
-    if (threadIdx.x < 128) {
-      const int jj = threadIdx.x >> 2, q = threadIdx.x & 3;
-      P_t acc = 0;
-#pragma unroll
-      for (int g = 0; g < 8; ++g) acc += red[g][jj][q];
-      ((P_t *)w.rowpart)[((size_t)blk * TILE + jj) * 4 + q] = acc;
-    }
-    // publish this block's partials, then count it in its row and column tile;
-    // the block that completes a tile forms that tile's forces (no waiting)
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      last[0] = atomicAdd(w.rowcnt + t, 1) == t;             // blocks (t, 0..t)
-      last[1] = atomicAdd(w.colcnt + s, 1) == w.NT - 1 - s;  // blocks (s..NT-1, s)
-    }
-    __syncthreads();
-    const bool last_row = last[0], last_col = last[1];
-    if (last_row || last_col) __threadfence();
-    if (last_row) finalize_rows<MIXED ? PK_F32 : PK_F64, PBC>(w, t, pos, F, fin);
-    if (last_col) finalize_cols<MIXED ? PK_F32 : PK_F64, PBC>(w, s, pos, F, fin);
-  }
-}
-
-// Exterior-bead forces of one row tile (bead P) or column tile (bead 1) from
-// complete sums fin[j][0..3] + fin[j][4..7] = (sum Pr, sum Pr (r - r')), used
-// by the recompute pass (the same formulas as the tile finalisers above).
-template <bool PBC>
-__device__ void finish_rows(const Workspace &w, int t, const double *__restrict__ pos, double *__restrict__ F,
-                            double (*fin)[9]) {
-  const int p = t * TILE + threadIdx.x;
-  if (threadIdx.x >= TILE || p >= w.N) return;
-  const double *r = w.RP + 4 * (size_t)p, *nbP = pos + ((size_t)p * w.P + (w.P - 2)) * 3;  // bead P-1
-  const double M = (p + 1 < w.N) ? direct_link_fast(w, p) : 0.0;
-  const double *fr = fin[threadIdx.x];
-  const double rs = fr[0] + fr[4] + M;
-  double *fP = F + ((size_t)p * w.P + (w.P - 1)) * 3;
-  bool ok = true;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const double n1 = (p + 1 < w.N) ? w.R1[4 * (size_t)(p + 1) + c] : 0.0;
-    const double rc = fma(M, img<PBC>(w, r[c] - n1), fr[1 + c] + fr[5 + c]);
-    fP[c] = -w.k * fma(rs, img<PBC>(w, r[c] - nbP[c]), rc);
-    ok &= isfinite(fP[c]);
-  }
-  if (!ok) atomicOr(w.status, ST_NONFINITE);
-}
-template <bool PBC>
-__device__ void finish_cols(const Workspace &w, int s, const double *__restrict__ pos, double *__restrict__ F,
-                            double (*fin)[9]) {
-  const int p = s * TILE + threadIdx.x;
-  if (threadIdx.x >= TILE || p >= w.N) return;
-  const double *r = w.R1 + 4 * (size_t)p, *nb1 = pos + ((size_t)p * w.P + 1) * 3;  // bead 2
-  const double M = (p >= 1) ? direct_link_fast(w, p - 1) : 0.0;
-  const double *fc = fin[threadIdx.x];
-  const double cs = fc[0] + fc[4] + M;
-  double *f1 = F + (size_t)p * w.P * 3;
-  bool ok = true;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const double pP = (p >= 1) ? w.RP[4 * (size_t)(p - 1) + c] : 0.0;
-    const double cc = fma(M, img<PBC>(w, r[c] - pP), fc[1 + c] + fc[5 + c]);
-    f1[c] = -w.k * fma(cs, img<PBC>(w, r[c] - nb1[c]), cc);
-    ok &= isfinite(f1[c]);
-  }
-  if (!ok) atomicOr(w.status, ST_NONFINITE);
-}
-
-// ----------------------------------------------------------- MIXED (config 3)
-// Unevaluated sums h + l of two float32 numbers (|l| <= ulp(h)/2 after
-// renormalisation): about 46 significant bits on the float32 pipe.
-struct ff {
-  float h, l;
-};
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-  const float s = a.h + b.h, bb = s - a.h;
-  const float e = ((a.h - (s - bb)) + (b.h - bb)) + (a.l + b.l);
-  const float h = s + e;
-  return ff{h, e - (h - s)};
-}
-// a * d with a float32 d; a.h * d is exact by FMA (TwoProd)
-__device__ __forceinline__ ff ff_mul(ff a, float d) {
-  const float p = a.h * d;
-  const float e = fmaf(a.h, d, -p) + a.l * d;
-  const float h = p + e;
-  return ff{h, e - (h - p)};
-}
-
-// Pr = alpha mu g of one pair from three extended numbers with double
-// mantissas in [1, 2): the mantissa products on the integer pipe (64-bit
-// truncations, 2^-62 relative), the exponents added as integers; returned as
-// an unevaluated float32 pair (the mantissa cut at 2^-46), 0 below 2^-126.
-__device__ __forceinline__ ff prob_ff(unsigned long long am, int e_am, double gm, int ge) {
-  // am = (alpha mantissa)(mu mantissa) normalised to [2^63, 2^64), value am/2^63 2^e_am
-  const unsigned long long gg = (((unsigned long long)__double_as_longlong(gm) & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 11;
-  unsigned long long pr = __umul64hi(am, gg);  // in [2^62, 2^64)
-  const int sh = (int)(pr >> 63) ^ 1;
-  pr <<= sh;
-  const int E = e_am + ge + 1 - sh;  // Pr = (pr / 2^63) 2^E
-  if (E < -126) return ff{0.0f, 0.0f};
-  const float h = __uint_as_float((unsigned)((E + 127) << 23) | (unsigned)((pr >> 40) & 0x7FFFFFu));
-  const float t = __uint_as_float(0x4B000000u | (unsigned)((pr >> 17) & 0x7FFFFFu)) - 8388608.0f;  // next 23 bits
-  const float sc = (E - 46 >= -126) ? __uint_as_float((unsigned)((E - 46 + 127) << 23)) : 0.0f;
-  return ff{h, t * sc};
-}
-
-// One 32 x 32 block of the lower triangle in the MIXED form (all 256
-// threads).  Thread (i0 = warp, j = lane) forms the pairs (a = 32 s + i0 + 8 k,
-// b = 32 t + j), k = 0..3: Pr and Pr (r_b^P - r_a^1) (float32 bead
-// differences) as float32 pairs into the shared tile V[value][i][j]; then
-// 128 threads sum the 32 rows b over their sources and 128 threads the 32
-// columns a over their rows, in a fixed order, as float32 pairs.
-template <bool PBC>
-__device__ __forceinline__ void prob_block_mixed(const Workspace &w, int blk, const double *__restrict__ pos,
-                                                 double *__restrict__ F, float (*V)[2][TILE][33], double (*fin)[9],
-                                                 int *last) {
-  int t, s;
-  block_coords_f(blk, t, s);
-  const int j = threadIdx.x & 31, i0 = threadIdx.x >> 5;
-  const int b = t * TILE + j;
-  const bool bvalid = b < w.N;
-  unsigned long long mum = 0;
-  int mue = 0;
-  float4 bh = make_float4(0.f, 0.f, 0.f, 0.f), bl = bh;
-  if (bvalid) {
-    const xd mub = mu_of(w, b);
-    mum = (((unsigned long long)__double_as_longlong(mub.m) & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 11;
-    mue = mub.e;
-    bh = *(const float4 *)(w.RPs + 8 * (size_t)b);
-    bl = *(const float4 *)(w.RPs + 8 * (size_t)b + 4);
-  }
-#pragma unroll
-  for (int kk = 0; kk < 4; ++kk) {
-    const int i = i0 + 8 * kk;
-    const int a = s * TILE + i;
-    ff pr{0.0f, 0.0f}, px{0.0f, 0.0f}, py{0.0f, 0.0f}, pz{0.0f, 0.0f};
-    if (bvalid && a <= b) {
-      float fx, fy, fz;
-      if (PBC) {  // minimum image from the fixed-point copies (bh holds RP's bits)
-        const uint4 ua = *(const uint4 *)(w.R1s + 8 * (size_t)a);
-        fx = fixdiff(__float_as_uint(bh.x), ua.x, w.Lscale);
-        fy = fixdiff(__float_as_uint(bh.y), ua.y, w.Lscale);
-        fz = fixdiff(__float_as_uint(bh.z), ua.z, w.Lscale);
-      } else {
-        const float4 ah = *(const float4 *)(w.R1s + 8 * (size_t)a);
-        const float4 al4 = *(const float4 *)(w.R1s + 8 * (size_t)a + 4);
-        fx = (bh.x - ah.x) + (bl.x - al4.x);
-        fy = (bh.y - ah.y) + (bl.y - al4.y);
-        fz = (bh.z - ah.z) + (bl.z - al4.z);
-      }
-      const size_t gi = (size_t)blk * TILE2 + i * TILE + j;
-      const double alm = ((const double *)w.alm)[a];
-      const unsigned long long aa = (((unsigned long long)__double_as_longlong(alm) & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 11;
-      unsigned long long am = __umul64hi(aa, mum);  // in [2^62, 2^64)
-      const int sh = (int)(am >> 63) ^ 1;
-      am <<= sh;
-      pr = prob_ff(am, w.ale[a] + mue + 1 - sh, ((const double *)w.gm)[gi], w.ge[gi]);
-      px = ff_mul(pr, fx);
-      py = ff_mul(pr, fy);
-      pz = ff_mul(pr, fz);
-    }
-    V[0][0][i][j] = pr.h; V[0][1][i][j] = pr.l;
-    V[1][0][i][j] = px.h; V[1][1][i][j] = px.l;
-    V[2][0][i][j] = py.h; V[2][1][i][j] = py.l;
-    V[3][0][i][j] = pz.h; V[3][1][i][j] = pz.l;
-  }
-  __syncthreads();
-  {
-    const int q = (threadIdx.x >> 5) & 3, r = threadIdx.x & 31;
-    ff acc{0.0f, 0.0f};
-    if (threadIdx.x < 128) {  // row r (particle b = 32 t + r): sum over the sources i
-#pragma unroll 8
-      for (int i = 0; i < TILE; ++i) acc = ff_add(acc, ff{V[q][0][i][r], V[q][1][i][r]});
-      ((float2 *)w.rowpart)[((size_t)blk * TILE + r) * 4 + q] = make_float2(acc.h, acc.l);
-    } else {  // column r (particle a = 32 s + r): sum over the rows j; bead-1 sums carry r_a^1 - r_b^P
-#pragma unroll 8
-      for (int jj = 0; jj < TILE; ++jj) acc = ff_add(acc, ff{V[q][0][r][jj], V[q][1][r][jj]});
-      const float sg = q == 0 ? 1.0f : -1.0f;
-      ((float2 *)w.colpart)[((size_t)blk * TILE + r) * 4 + q] = make_float2(sg * acc.h, sg * acc.l);
+      P.h[i] = make_float4(ep.h.x, ep.h.y, ep.h.z, h);
+      P.l[i] = make_float4(ep.l.x, ep.l.y, ep.l.z, l);
     }
   }
-  // publish this block's partials, then count it in its row and column tile;
-  // the block that completes a tile forms that tile's forces (no waiting)
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    last[0] = atomicAdd(w.rowcnt + t, 1) == t;             // blocks (t, 0..t)
-    last[1] = atomicAdd(w.colcnt + s, 1) == w.NT - 1 - s;  // blocks (s..NT-1, s)
-  }
-  __syncthreads();
-  const bool last_row = last[0], last_col = last[1];
-  if (last_row || last_col) __threadfence();
-  if (last_row) finalize_rows<PK_FF, PBC>(w, t, pos, F, fin);
-  if (last_col) finalize_cols<PK_FF, PBC>(w, s, pos, F, fin);
+  P.e[i] = wt.e;
 }
-
-__global__ void __launch_bounds__(256, 4) prob_force_kernel_mixed(Workspace w, const double *__restrict__ pos,
-                                                               double *__restrict__ F) {
-  __shared__ float V[4][2][TILE][33];
-  __shared__ double fin[32][9];
-  __shared__ int last[2];
-  pdl_wait();
-  for (int blk = blockIdx.x; blk < w.NB; blk += gridDim.x) {
-    if (w.pbc) prob_block_mixed<true>(w, blk, pos, F, V, fin, last);
-    else prob_block_mixed<false>(w, blk, pos, F, V, fin, last);
-    __syncthreads();  // V is rewritten by the next block
-  }
-  pdl_trigger();
-}
-
-__global__ void __launch_bounds__(256, 4) prob_force_batched_mixed(const Workspace *__restrict__ ws,
-                                                                const int2 *__restrict__ tab, int ntab,
-                                                                const long long *__restrict__ off,
-                                                                const double *__restrict__ pos,
-                                                                double *__restrict__ F) {
-  __shared__ float V[4][2][TILE][33];
-  __shared__ double fin[32][9];
-  __shared__ int last[2];
-  pdl_wait();
-  for (int k = blockIdx.x; k < ntab; k += gridDim.x) {
-    const int2 e = tab[k];
-    if (ws[e.x].pbc) prob_block_mixed<true>(ws[e.x], e.y, pos + off[e.x], F + off[e.x], V, fin, last);
-    else prob_block_mixed<false>(ws[e.x], e.y, pos + off[e.x], F + off[e.x], V, fin, last);
-    __syncthreads();
-  }
-  pdl_trigger();
-}
-
-// ------------------------------------------------- recompute mode (no table)
-// Probabilities and exterior forces by whole tiles: work item 2k is row tile
-// NT-1-k (all its source tiles), item 2k+1 column tile k (all its row tiles),
-// so that the items come in decreasing size.  A row item forms Pr[b -> a] for
-// its 32 rows b (lanes) and every source a (8 warps, 4 sources each per 32x32
-// block), with g recomputed from the endpoint copies, and accumulates the row
-// sums in registers; the column items do the same for the 32 columns.  Every
-// pair is formed twice (once per item kind) and nothing O(N^2) is stored; the
-// sums are combined across warps in a fixed order (deterministic).
-// Accumulators: float64 (FP64) or compensated float32 pairs (mixed forms).
-template <int MODE>
-struct PAcc {
-  using T = typename std::conditional<MODE == BPIMD_FP64, double, ff>::type;
-  T s, x, y, z;
-  __device__ __forceinline__ void zero() {
-    if constexpr (MODE == BPIMD_FP64) s = x = y = z = 0.0;
-    else s = x = y = z = ff{0.0f, 0.0f};
-  }
-};
-
-// Pr(a, b) for the recompute items: alpha_a, mu_b and g as extended numbers.
-template <int MODE>
-__device__ __forceinline__ typename PAcc<MODE>::T prob_rc(const Workspace &w, int a, xd mu, double gm, int ge) {
-  if constexpr (MODE == BPIMD_FP64) {
-    return (((const double *)w.alm)[a] * mu.m * gm) * pow2_normal(w.ale[a] + mu.e + ge);
-  } else if constexpr (MODE == BPIMD_MIXED) {
-    const unsigned long long aa =
-        (((unsigned long long)__double_as_longlong(((const double *)w.alm)[a]) & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 11;
-    const unsigned long long mm = (((unsigned long long)__double_as_longlong(mu.m) & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 11;
-    unsigned long long am = __umul64hi(aa, mm);
-    const int sh = (int)(am >> 63) ^ 1;
-    am <<= sh;
-    return prob_ff(am, w.ale[a] + mu.e + 1 - sh, gm, ge);
+// partner i's endpoint from shared memory
+template <bool F64, bool PBC>
+__device__ __forceinline__ pairg::EndPt<!F64, PBC> staged_end(const Partners<F64> &P, int i) {
+  pairg::EndPt<!F64, PBC> e;
+  if constexpr (F64) {
+    e.x = P.x[i];
+    e.y = P.y[i];
+    e.z = P.z[i];
+  } else if constexpr (PBC) {
+    const float4 h = P.h[i];
+    e.u = make_uint4(__float_as_uint(h.x), __float_as_uint(h.y), __float_as_uint(h.z), 0u);
   } else {
-    const int e = w.ale[a] + mu.e + ge;
-    float M = ((const float *)w.alm)[a] * (float)mu.m * (float)gm;
-    M = (e < -150) ? 0.0f : (e > 0 ? M * (float)(1 << min(e, 2)) : M * pow2f_nonpos(e));
-    return ff{M, 0.0f};
+    e.h = P.h[i];
+    e.l = P.l[i];
   }
+  return e;
 }
 
-template <int MODE, typename D3>
-__device__ __forceinline__ void acc_add(PAcc<MODE> &A, typename PAcc<MODE>::T pr, D3 d, float sign) {
-  if constexpr (MODE == BPIMD_FP64) {
-    A.s += pr;
-    A.x = fma(sign * pr, d.x, A.x);
-    A.y = fma(sign * pr, d.y, A.y);
-    A.z = fma(sign * pr, d.z, A.z);
-  } else {
-    A.s = ff_add(A.s, pr);
-    A.x = ff_add(A.x, ff_mul(pr, sign * d.x));
-    A.y = ff_add(A.y, ff_mul(pr, sign * d.y));
-    A.z = ff_add(A.z, ff_mul(pr, sign * d.z));
-  }
-}
-
-template <int MODE>
-__device__ __forceinline__ double acc_val(typename PAcc<MODE>::T v) {
-  if constexpr (MODE == BPIMD_FP64) return v;
-  else return (double)v.h + (double)v.l;
-}
-
-// One work item of the recompute pass (all 256 threads).  red: [8][32][4]
-// per-warp sums; fin as in the tile finalisers.
-template <int MODE, bool PBC>
-__device__ void prob_item_rc(const Workspace &w, int item, const double *__restrict__ pos, double *__restrict__ F,
-                             const unsigned long long *T63, double (*red)[32][4], double (*fin)[9]) {
-  using EP = pairg::EndPt<MODE != BPIMD_FP64, PBC>;
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+// One item (all threads of the cluster's CTAs; CTA `rank` of CL).
+template <int MODE, bool RC, bool PBC>
+__device__ __forceinline__ void exterior_item(const Workspace &w, int item, int rank, int CL,
+                                              const double *__restrict__ pos, double *__restrict__ F,
+                                              const unsigned long long *T63, ProbSmem<MODE == BPIMD_FP64> &sm) {
+  constexpr bool F64 = MODE == BPIMD_FP64;
+  using EP = pairg::EndPt<!F64, PBC>;
+  using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, N = w.N;
   const bool row_item = !(item & 1);
   const int tile = row_item ? w.NT - 1 - (item >> 1) : (item >> 1);
-  const int me = tile * TILE + lane;  // this lane's particle (row b or column a)
-  PAcc<MODE> A;
-  A.zero();
-  if (me < w.N) {
-    const EP mine = pairg::load_end<MODE != BPIMD_FP64, PBC>(w, me, row_item);  // bead P of b, or bead 1 of a
-    const xd mub = row_item ? mu_of(w, me) : xd{0.0, 0};
-    const int t0 = row_item ? 0 : tile, t1 = row_item ? tile : w.NT - 1;
-    for (int o = t0; o <= t1; ++o) {
+  const int me = tile * TILE + lane;
+  const int mine_q = min(me, N - 1);  // lanes past N repeat the last particle and are not stored
+  const EP mine = pairg::load_end<!F64, PBC>(w, mine_q, row_item);
+  const xd own_w = row_item ? weight_mu(w, mine_q) : weight_y(w, mine_q);
+  const int own_e = own_w.e + w.scal_i[0];  // with the exponent of 1/(N y_N)
+  const int p0 = row_item ? 0 : tile * TILE, p1 = row_item ? min(N, (tile + 1) * TILE) : N;
+  // partners of a chunk: a multiple of 32, so that each warp takes whole groups of four
+  const int ch = min(PROB_CHUNK, ((p1 - p0 + CL - 1) / CL + 31) & ~31), per = ch / PROB_WARPS;
+  // this lane's pair factors: g(partner q) at gi0 + 32 src, src = q in the
+  // forward copy, N-1-q in the backward one (clamped into the stored triangle)
+  const int r = row_item ? tile * TILE + lane : N - 1 - mine_q;
+  const int gi0 = (((r >> 5) * ((r >> 5) + 1) / 2) << 10) + (r & 31);
+  const M_t *gm = (const M_t *)(row_item ? w.gm : w.gbm) + gi0;
+  const int *ge = (row_item ? w.ge : w.gbe) + gi0;
+  PSum A{{0, 0, 0}, NO_TERM};
+  int bad = 0;
+  float fs[3] = {0.f, 0.f, 0.f}, fc[3] = {0.f, 0.f, 0.f};
+  constexpr int G = 4;
+  for (int c0 = p0 + rank * ch; c0 < p1; c0 += CL * ch) {
+    const int q0 = c0 + wp * per, q1 = min(q0 + per, p1);
+    M_t gmv[G];
+    int gev[G];
+    auto load_g = [&](int q) {
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const int other = o * TILE + wp + 8 * kk;  // source a (row item) or row b (column item)
-        const int a = row_item ? other : me, b = row_item ? me : other;
-        if (a <= b && b < w.N) {
-          const EP oth = pairg::load_end<MODE != BPIMD_FP64, PBC>(w, other, !row_item);
-          const EP &eb = row_item ? mine : oth, &ea = row_item ? oth : mine;
-          int ge;
-          const double gm = (double)pairg::g_of<MODE, PBC>(w, eb, ea, w.cx, T63, ge);
-          const auto pr = prob_rc<MODE>(w, a, row_item ? mub : mu_of(w, b), gm, ge);
-          // row b: Pr (r_b^P - r_a^1); column a: Pr (r_a^1 - r_b^P)
-          acc_add<MODE>(A, pr, pairg::diff3(w, eb, ea), row_item ? 1.0f : -1.0f);
+      for (int k = 0; k < G; ++k) {
+        const int qk = min(q + k, p1 - 1), src = row_item ? qk : N - 1 - max(qk, mine_q);
+        gmv[k] = __ldg(gm + 32 * src);
+        gev[k] = __ldg(ge + 32 * src);
+      }
+    };
+    if (!RC && q0 < q1) load_g(q0);
+    if (c0 != p0 + rank * ch) __syncthreads();  // the previous chunk is read
+    for (int i = threadIdx.x; i < ch; i += PROB_THREADS)
+      if (c0 + i < p1)
+        stage_partner<F64, PBC>(w, sm.part, i, c0 + i, !row_item, row_item ? weight_y(w, c0 + i) : weight_mu(w, c0 + i));
+    __syncthreads();
+    for (int q = q0; q < q1; q += G) {
+      M_t m[G];
+      int e[G];
+#pragma unroll
+      for (int k = 0; k < G; ++k) { m[k] = gmv[k]; e[k] = gev[k]; }
+      if (!RC && q + G < q1) load_g(q + G);
+      unsigned long long p[G][3];
+      int pe[G][3], sg[G][3], E = NO_TERM;
+#pragma unroll
+      for (int k = 0; k < G; ++k) {
+        const int i = min(q + k, p1 - 1) - c0;
+        const bool valid = q + k < p1 && (row_item ? q + k <= me : q + k >= me);
+        const EP oth = staged_end<F64, PBC>(sm.part, i);
+        const EP &eb = row_item ? mine : oth, &ea = row_item ? oth : mine;
+        if constexpr (RC) m[k] = pairg::g_of<MODE, PBC>(w, eb, ea, w.cx, T63, e[k]);
+        auto d = pairg::diff3(w, eb, ea);
+        if constexpr (F64) {
+          const unsigned long long t = valid ? __umul64hi(sm.part.m[i], mant64(m[k])) : 0ull;  // value t 2^(et - 63)
+          const int et = valid ? sm.part.e[i] + e[k] + 1 : NO_TERM;
+          int nonfinite = 0;
+          p[k][0] = diff_term(t, d.x, pe[k][0], sg[k][0], nonfinite);
+          p[k][1] = diff_term(t, d.y, pe[k][1], sg[k][1], nonfinite);
+          p[k][2] = diff_term(t, d.z, pe[k][2], sg[k][2], nonfinite);
+          bad |= valid ? nonfinite : 0;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            pe[k][c] = max(pe[k][c] + et, NO_TERM);
+            E = max(E, pe[k][c]);
+          }
+        } else {
+          const float yh = sm.part.h[i].w, yl = sm.part.l[i].w;
+          const int x = sm.part.e[i] + e[k] + own_e;
+          const float sc = valid && x >= -126 ? __int_as_float((min(x, 100) + 127) << 23) : 0.0f;
+          float gh, gl;
+          mant_hl(m[k], gh, gl);
+          const float t = yh * gh, te = fmaf(yl, gh, fmaf(yh, gl, fmaf(yh, gh, -t)));
+          const float th = t * sc, tl = te * sc;
+          const float dc[3] = {valid ? d.x : 0.0f, valid ? d.y : 0.0f, valid ? d.z : 0.0f};
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float x0 = th * dc[c];
+            fc[c] += fmaf(tl, dc[c], fmaf(th, dc[c], -x0));
+            two_sum(fs[c], fc[c], x0);
+          }
         }
+      }
+      if constexpr (F64) {
+        PSum B{{0, 0, 0}, E + 3};
+#pragma unroll
+        for (int k = 0; k < G; ++k)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const long long x = (long long)(p[k][c] >> min(E - pe[k][c] + 3, 63));
+            B.v[c] += (x ^ sg[k][c]) - sg[k][c];
+          }
+        psum_add(A, B);
       }
     }
   }
-  red[wp][lane][0] = acc_val<MODE>(A.s);
-  red[wp][lane][1] = acc_val<MODE>(A.x);
-  red[wp][lane][2] = acc_val<MODE>(A.y);
-  red[wp][lane][3] = acc_val<MODE>(A.z);
-  __syncthreads();
-  if (threadIdx.x < 128) {  // fixed-order sum over the 8 warps, into the finalisers' layout
-    const int jj = threadIdx.x >> 2, q = threadIdx.x & 3;
-    double v = 0.0;
+  SumSlot<F64> &ws = sm.warp[wp];
 #pragma unroll
-    for (int g = 0; g < 8; ++g) v += red[g][jj][q];
-    fin[jj][q] = v;
-    fin[jj][q + 4] = 0.0;
+  for (int c = 0; c < 3; ++c) {
+    if constexpr (F64) ws.v[c][lane] = A.v[c];
+    else { ws.s[c][lane] = fs[c]; ws.c[c][lane] = fc[c]; }
   }
+  if constexpr (F64) { ws.E[lane] = A.E; ws.bad[lane] = bad; }
   __syncthreads();
-  if (row_item) finish_rows<PBC>(w, tile, pos, F, fin);
-  else finish_cols<PBC>(w, tile, pos, F, fin);
-  __syncthreads();
+  // warp c < 3: component c of the lane's sum over `n` slots, in order
+  auto add_slots = [&](const SumSlot<F64> *sl, int n, int c, long long &v, int &E, int &bd, float &s, float &cc) {
+    if constexpr (F64) {
+      v = 0; E = NO_TERM; bd = 0;
+      for (int k = 0; k < n; ++k) { E = max(E, sl[k].E[lane]); bd |= sl[k].bad[lane]; }
+      for (int k = 0; k < n; ++k) v += shift_in(sl[k].v[c][lane], E - sl[k].E[lane] + 3);
+      E += 3;
+    } else {
+      s = 0.0f; cc = 0.0f;
+      for (int k = 0; k < n; ++k) { two_sum(s, cc, sl[k].s[c][lane]); cc += sl[k].c[c][lane]; }
+    }
+  };
+  long long v = 0;
+  int E = 0, bd = 0;
+  float s = 0.0f, cc = 0.0f;
+  if (wp < 3) {
+    add_slots(sm.warp, PROB_WARPS, wp, v, E, bd, s, cc);
+  } else if (rank == 0 && wp < 6 && me < N) {
+    // meanwhile warps 3..5 of the first CTA: what does not need the sums
+    const int c = wp - 3;
+    const double own = (row_item ? w.RP : w.R1)[4 * (size_t)me + c];
+    const double nb = pos[((size_t)me * w.P + (row_item ? w.P - 2 : 1)) * 3 + c];  // bead P-1, or bead 2
+    double b = img<PBC>(w, own - nb);
+    if (row_item ? me + 1 < N : me >= 1) {  // the direct link me -> me+1, or me-1 -> me
+      const double oth = row_item ? w.R1[4 * (size_t)(me + 1) + c] : w.RP[4 * (size_t)(me - 1) + c];
+      b = fma(direct_link_fast(w, row_item ? me : me - 1), img<PBC>(w, own - oth), b);
+    }
+    sm.base[c][lane] = b;
+  }
+  if (CL > 1) {
+    cluster_wait_acquire();  // every CTA of the cluster has started (it arrived at its start)
+    if (wp < 3) {
+      SumSlot<F64> &cs = sm.cta[rank];
+      if constexpr (F64) {
+        cluster_store(&cs.v[wp][lane], v);
+        if (wp == 0) { cluster_store(&cs.E[lane], E); cluster_store(&cs.bad[lane], bd); }
+      } else {
+        cluster_store(&cs.s[wp][lane], s);
+        cluster_store(&cs.c[wp][lane], cc);
+      }
+    }
+    cluster_arrive_release();
+    cluster_wait_acquire();
+    if (rank == 0 && wp < 3) add_slots(sm.cta, CL, wp, v, E, bd, s, cc);
+  } else {
+    __syncthreads();
+  }
+  if (rank == 0 && wp < 3 && me < N) {
+    const double mz = own_w.m * w.scal[1];
+    double W;
+    if constexpr (F64) {
+      W = ((double)v * mz) * pow2_normal(E - 61 + own_e);
+      if (bd) W = __longlong_as_double(0x7ff8000000000000LL);
+    } else {
+      W = ((double)s + (double)cc) * mz;
+    }
+    const double f = -w.k * (sm.base[wp][lane] + (row_item ? W : -W));
+    F[((size_t)me * w.P + (row_item ? w.P - 1 : 0)) * 3 + wp] = f;
+    if (!isfinite(f)) atomicOr(w.status, ST_NONFINITE);
+  }
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(256) prob_rc_kernel(Workspace w, const double *__restrict__ pos,
-                                                      double *__restrict__ F) {
-  __shared__ double red[8][32][4];
-  __shared__ double fin[32][9];
-  __shared__ unsigned long long T63[256];
-  if (MODE != BPIMD_MIXED32) pairg::table_init(T63);
-  __syncthreads();
-  pdl_wait();
-  for (int item = blockIdx.x; item < 2 * w.NT; item += gridDim.x) {
-    if (w.pbc) prob_item_rc<MODE, true>(w, item, pos, F, T63, red, fin);
-    else prob_item_rc<MODE, false>(w, item, pos, F, T63, red, fin);
+// CL CTAs (one cluster) per item
+template <int MODE, bool RC>
+__global__ void __launch_bounds__(PROB_THREADS) exterior_kernel(Workspace w, const double *__restrict__ pos,
+                                                                double *__restrict__ F, int CL) {
+  __shared__ ProbSmem<MODE == BPIMD_FP64> sm;
+  __shared__ unsigned long long T63[RC ? 256 : 1];
+  if (CL > 1) cluster_arrive_release();
+  if (RC && MODE != BPIMD_MIXED32) {
+    pairg::table_init(T63);
+    __syncthreads();
   }
+  pdl_wait();
+  const int item = blockIdx.x / CL, rank = blockIdx.x % CL;
+  if (w.pbc) exterior_item<MODE, RC, true>(w, item, rank, CL, pos, F, T63, sm);
+  else exterior_item<MODE, RC, false>(w, item, rank, CL, pos, F, T63, sm);
   pdl_trigger();
 }
 
-template <bool MIXED>
-__global__ void __launch_bounds__(256, 4) prob_force_kernel(Workspace w, const double *__restrict__ pos,
-                                                         double *__restrict__ F) {
-  using P_t = typename std::conditional<MIXED, float, double>::type;
-  __shared__ P_t red[8][32][4];
-  __shared__ double fin[32][9];
-  __shared__ int last[2];
-  pdl_wait();
-  for (int blk = blockIdx.x; blk < w.NB; blk += gridDim.x) {
-    if (w.pbc) prob_block<MIXED, true>(w, blk, pos, F, red, fin, last);
-    else prob_block<MIXED, false>(w, blk, pos, F, red, fin, last);
-  }
-  pdl_trigger();
-}
-
-// Replica batch: entry k of tab is (replica, block); positions and forces of
+// Replica batch: entry k of tab is (replica, item); positions and forces of
 // replica r start at element off[r] of the packed arrays.
-template <bool MIXED>
-__global__ void __launch_bounds__(256, 4) prob_force_batched(const Workspace *__restrict__ ws,
-                                                          const int2 *__restrict__ tab, int ntab,
-                                                          const long long *__restrict__ off,
-                                                          const double *__restrict__ pos, double *__restrict__ F) {
-  using P_t = typename std::conditional<MIXED, float, double>::type;
-  __shared__ P_t red[8][32][4];
-  __shared__ double fin[32][9];
-  __shared__ int last[2];
-  pdl_wait();  // launched as a programmatic dependent of the recursions: their epilogue must be complete
+template <int MODE>
+__global__ void __launch_bounds__(PROB_THREADS) exterior_batched(const Workspace *__restrict__ ws,
+                                                                 const int2 *__restrict__ tab, int ntab,
+                                                                 const long long *__restrict__ off,
+                                                                 const double *__restrict__ pos,
+                                                                 double *__restrict__ F) {
+  __shared__ ProbSmem<MODE == BPIMD_FP64> sm;
+  pdl_wait();
   for (int k = blockIdx.x; k < ntab; k += gridDim.x) {
     const int2 e = tab[k];
-    if (ws[e.x].pbc) prob_block<MIXED, true>(ws[e.x], e.y, pos + off[e.x], F + off[e.x], red, fin, last);
-    else prob_block<MIXED, false>(ws[e.x], e.y, pos + off[e.x], F + off[e.x], red, fin, last);
+    exterior_item<MODE, false, false>(ws[e.x], e.y, 0, 1, pos + off[e.x], F + off[e.x], nullptr, sm);
+    __syncthreads();  // the slots are read
   }
   pdl_trigger();
 }
@@ -771,27 +529,43 @@ __global__ void dense_prob_kernel(Workspace w, double *M) {
 
 }  // namespace
 
+namespace {
+template <int MODE, bool RC>
+cudaError_t launch_exterior(const Workspace &w, const double *pos, double *F, cudaStream_t s) {
+  // CTAs per item: enough that a warp has a few groups of four partners (the
+  // longest list is N), few enough that the cluster barrier and the staging do
+  // not outweigh them.  Whole evaluation, mixed, with 1 / 2 / 4 / 8 CTAs: N = 64
+  // 23.0 / 22.7 / 22.4 / 22.4 us, N = 256 34.0 / 32.2 / 31.2 / 31.0, N = 1024
+  // 84.8 / 75.1 / 71.9 / 72.8, N = 1601 138 / 126 / 123 / 120, N = 4096
+  // 502 / 477 / 470 / 478 (past ~64 tiles four fill the GPU).
+  const int CL = w.NT <= 1 ? 1 : w.NT <= 2 ? 2 : w.NT <= 32 ? 4 : w.NT <= 64 ? 8 : 4;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * w.NT * CL);
+  cfg.blockDim = dim3(PROB_THREADS);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = CL;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, exterior_kernel<MODE, RC>, w, pos, F, CL);
+}
+}  // namespace
+
 cudaError_t launch_prob_forces(const Workspace &w, const double *pos, double *F, cudaStream_t s) {
-  const int sms = sm_count();
-  cudaError_t e;
-  if (w.recomp) {
-    const int items = 2 * w.NT, grid_rc = items < sms * 4 ? items : sms * 4;
-    switch (w.mode) {
-      case BPIMD_FP64: e = launch_pdl(prob_rc_kernel<BPIMD_FP64>, grid_rc, 256, 0, s, w, pos, F); break;
-      case BPIMD_MIXED: e = launch_pdl(prob_rc_kernel<BPIMD_MIXED>, grid_rc, 256, 0, s, w, pos, F); break;
-      default: e = launch_pdl(prob_rc_kernel<BPIMD_MIXED32>, grid_rc, 256, 0, s, w, pos, F); break;
-    }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
-  }
-  const int grid = w.NB < sms * 8 ? w.NB : sms * 8;
   switch (w.mode) {
-    case BPIMD_FP64: e = launch_pdl(prob_force_kernel<false>, grid, 256, 0, s, w, pos, F); break;
-    case BPIMD_MIXED: e = launch_pdl(prob_force_kernel_mixed, grid, 256, 0, s, w, pos, F); break;
-    default: e = launch_pdl(prob_force_kernel<true>, grid, 256, 0, s, w, pos, F); break;
+    case BPIMD_FP64:
+      return w.recomp ? launch_exterior<BPIMD_FP64, true>(w, pos, F, s) : launch_exterior<BPIMD_FP64, false>(w, pos, F, s);
+    case BPIMD_MIXED:
+      return w.recomp ? launch_exterior<BPIMD_MIXED, true>(w, pos, F, s) : launch_exterior<BPIMD_MIXED, false>(w, pos, F, s);
+    default:
+      return w.recomp ? launch_exterior<BPIMD_MIXED32, true>(w, pos, F, s)
+                      : launch_exterior<BPIMD_MIXED32, false>(w, pos, F, s);
   }
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
 }
 
 cudaError_t launch_spring_expectation(const Workspace &w, double *part, cudaStream_t s) {
@@ -823,9 +597,9 @@ cudaError_t launch_prob_forces_batched(const Workspace *ws, const int2 *tab, int
   const int grid = ntab < cap ? ntab : cap;
   cudaError_t e;
   switch (mode) {
-    case BPIMD_FP64: e = launch_pdl(prob_force_batched<false>, grid, 256, 0, s, ws, tab, ntab, off, pos, F); break;
-    case BPIMD_MIXED: e = launch_pdl(prob_force_batched_mixed, grid, 256, 0, s, ws, tab, ntab, off, pos, F); break;
-    default: e = launch_pdl(prob_force_batched<true>, grid, 256, 0, s, ws, tab, ntab, off, pos, F); break;
+    case BPIMD_FP64: e = launch_pdl(exterior_batched<BPIMD_FP64>, grid, 256, 0, s, ws, tab, ntab, off, pos, F); break;
+    case BPIMD_MIXED: e = launch_pdl(exterior_batched<BPIMD_MIXED>, grid, 256, 0, s, ws, tab, ntab, off, pos, F); break;
+    default: e = launch_pdl(exterior_batched<BPIMD_MIXED32>, grid, 256, 0, s, ws, tab, ntab, off, pos, F); break;
   }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

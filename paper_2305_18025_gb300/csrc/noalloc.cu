@@ -6,16 +6,15 @@
 // calls can synchronise the whole device and stall other streams, or an
 // embedding with a fixed memory budget set up front.  For them this entry point
 // runs the same kernels as bpimd_exchange_energy_forces, but its scratch memory
-// (pair factors, recursion state, force partial sums) lives in one file-scope
+// (pair factors, recursion state) lives in one file-scope
 // __device__ array of fixed size, so no call allocates anything.
 //
 // Set-up: the first call on a device, with that device current, looks up the
 // array's device address with cudaGetSymbolAddress and caches it for that
 // device.  That first call should therefore come before any stream capture.
 // Shared state: every call on a device uses the same array, which keeps the
-// previous call's contents; each call clears the parts that must start at zero
-// (the device status word and the tile counters) and rewrites the padding of
-// the pair factors, which depends on N.  Two calls whose work overlaps on the GPU (for
+// previous call's contents; each call clears the device status word and
+// rewrites the padding of the pair factors, which depends on N.  Two calls whose work overlaps on the GPU (for
 // example on two different streams) race on the array and give wrong results.
 #include <mutex>
 
@@ -103,10 +102,6 @@ extern "C" int bpimd_exchange_energy_forces_noalloc(const bpimd_config *cfg, con
   layout_workspace(w, (char *)base);
 
   if (cudaMemsetAsync(w.status, 0, sizeof(int), s) != cudaSuccess) return BPIMD_ERR_CUDA;
-  // the tile counters of the probability pass start at zero (a previous call
-  // with another N leaves its counters at zero, but at other offsets)
-  if (cudaMemsetAsync(w.rowcnt, 0, sizeof(int) * w.NT, s) != cudaSuccess) return BPIMD_ERR_CUDA;
-  if (cudaMemsetAsync(w.colcnt, 0, sizeof(int) * w.NT, s) != cudaSuccess) return BPIMD_ERR_CUDA;
   if (launch_gmat_padding(w, s) != cudaSuccess) return BPIMD_ERR_CUDA;
   if (launch_prep(w, positions, forces, s) != cudaSuccess) return BPIMD_ERR_CUDA;
   if (launch_chains(w, V_B, s) != cudaSuccess) return BPIMD_ERR_CUDA;

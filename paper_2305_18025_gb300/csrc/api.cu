@@ -95,13 +95,15 @@ size_t layout_workspace(Workspace &w, char *base) {
   w.yfe = (int *)take(sizeof(int) * (N + 1));
   w.ybm = (double *)take(sizeof(double) * (N + 1));
   w.ybe = (int *)take(sizeof(int) * (N + 1));
-  w.alm = (void *)take(sizeof(double) * N);
-  w.ale = (int *)take(sizeof(int) * N);
   w.scal = (double *)take(sizeof(double) * 4);
   w.scal_i = (int *)take(sizeof(int) * 4);
   w.status = (int *)take(sizeof(int) * 4);
-  w.bk = w.blocks ? (unsigned long long *)take(sizeof(unsigned long long) * 4 * NT * TILE2) : nullptr;
-  w.be = w.blocks ? (int *)take(sizeof(int) * 4 * NT * TILE2) : nullptr;
+  w.nsum = (long long *)take(sizeof(long long));
+  const size_t panels = (N + CHAIN_PANEL - 1) / CHAIN_PANEL, pel = 2 * panels * CHAIN_PANEL * CHAIN_PANEL;
+  w.bk = w.blocks ? (unsigned long long *)take(sizeof(unsigned long long) * pel) : nullptr;
+  w.be = w.blocks ? (int *)take(sizeof(int) * pel) : nullptr;
+  w.Asm = w.blocks ? (unsigned long long *)take(sizeof(unsigned long long) * 2 * CHAIN_SLICES * N) : nullptr;
+  w.Ase = w.blocks ? (int *)take(sizeof(int) * 2 * CHAIN_SLICES * N) : nullptr;
   return off;
 }
 

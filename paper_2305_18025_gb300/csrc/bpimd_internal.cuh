@@ -37,8 +37,9 @@ namespace bpimd {
 constexpr int TILE = 32;              // row / source tile of the recursions and of g
 constexpr int TILE2 = TILE * TILE;
 constexpr int XZERO_E = -(1 << 29);   // exponent carried by an extended zero
-constexpr int CHAIN_THREADS = 640;     // 20 warps: up to 96 registers per thread
-constexpr int CHAIN_CLUSTER = 8;      // CTAs per recursion (small N): one lead + seven bulk CTAs
+constexpr int CHAIN_PANEL = 64;       // rows solved at a time by a recursion cluster
+constexpr int CHAIN_SLICES = 4;       // partial sums a row carries between superblocks
+constexpr int CHAIN_CLUSTER = 8;      // CTAs per recursion (small N)
 constexpr int CHAIN_MAX_N = BPIMD_MAX_N;  // largest N the library accepts
 constexpr int BATCH_MAX_N = 4096;     // largest replica of a batch (one CTA per recursion)
 constexpr int BEAD_BLOCK_PARTICLES = 8;  // particles per block of the bead pass
@@ -165,16 +166,16 @@ struct Workspace {
   // (Yb[w] = mu_{N-1-w} 0-based; the backward row sums are B_{a+1} = Yb[N-a] / c_{a}, 1-based c)
   double *yfm; int *yfe;
   double *ybm; int *ybe;
-  // alpha_a = y_a / (N y_N), a = 0..N-1, extended (float mantissa for MIXED),
-  // written by the forward recursion once y_N is known
-  void *alm; int *ale;
   // scalars: [0] V_B, [1] invZ mantissa, [2] reserved ; int [0] invZ exponent
   double *scal; int *scal_i;
   int *status;          // device status word
-  // blocked recursions (cluster kernel): per recursion and row tile, the
-  // c-scaled coupling block Dc to the previous tile's unknowns and the tile
+  // blocked recursions (cluster kernel): per recursion and panel of 64 rows the
   // inverse M = (I - L)^{-1}, as 64-bit integer mantissas in [2^63, 2^64) and
-  // exponents, [recursion][tile][Dc, M][row][source]
+  // exponents, [recursion][panel][row][column]; the rows' sums over finished
+  // superblocks, [recursion][slice][N]; the exponent parts n summed so far
+  unsigned long long *Asm;
+  int *Ase;
+  long long *nsum;
   int blocks;           // 1: bk/be present (single systems; batch replicas above BATCH_MAX_N)
   unsigned long long *bk;
   int *be;

@@ -150,28 +150,20 @@ __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *
   }
   pdl_trigger();  // the probability pass may launch during the epilogue
   if (!BWD) {
-    // V^{[1,N]} = C'[N] - (ln(y_N) - n ln 2)/beta, normaliser 1/(N y_N), alpha_a = y_a/(N y_N)
+    // V^{[1,N]} = C'[N] - (ln(y_N) - n ln 2)/beta, normaliser 1/(N y_N)
     if (q == 6 && lane == 0) { sm.misc[0] = carry; sm.nsum = ncarry; }
     __syncthreads();
     const xd yN{Ym[N], Ye[N]};
-    if (tid == 0) {  // the normaliser first: the alpha values wait for it
+    if (tid == 0) {
       const xd inv = xnorm(1.0 / (yN.m * (double)N), -yN.e);
       w.scal[1] = inv.m;
       w.scal_i[0] = inv.e;
-      sm.misc[1] = inv.m;
-      sm.misci[0] = inv.e;
     }
-    __syncthreads();
-    if (wid == 0) {  // V_B (a float64 log) on warp 0, alongside the alpha values
-      if (lane == 0) {
-        const double VB = reduced_potential(sm.misc[0], yN, sm.nsum, w.beta);
-        w.scal[0] = VB;
-        if (V_B) *V_B = VB;
-        if (!isfinite(VB)) atomicOr(w.status, ST_NONFINITE);
-      }
-    } else {
-      const xd inv{sm.misc[1], sm.misci[0]};
-      for (int a = tid - 32; a < N; a += blockDim.x - 32) store_alpha<MIXED>(w, a, xd{Ym[a], Ye[a]}, inv);
+    if (tid == 32) {
+      const double VB = reduced_potential(sm.misc[0], yN, sm.nsum, w.beta);
+      w.scal[0] = VB;
+      if (V_B) *V_B = VB;
+      if (!isfinite(VB)) atomicOr(w.status, ST_NONFINITE);
     }
   }
 }

@@ -207,20 +207,6 @@ __device__ __forceinline__ xs xs_fma(xs acc, unsigned long long kk, int ke, xs y
   return xs_norm((acc.m >> min(E - acc.e, 31)) + (p >> min(E - pe, 31)), E);
 }
 
-// alpha = y * inv for extended numbers with double mantissas in [1,2), with
-// integer operations; the mantissa is written as float (MIXED) or double.
-template <bool MIXED>
-__device__ __forceinline__ void store_alpha(const Workspace &w, int a, xd y, xd inv) {
-  const unsigned long long hi = __umul64hi(mant53(y.m) << 11, mant53(inv.m) << 11);  // in [2^62, 2^64)
-  const int sh = (int)(hi >> 63);
-  if (MIXED)
-    ((float *)w.alm)[a] = __int_as_float((int)((hi >> (39 + sh)) & 0x7FFFFFu) | 0x3F800000);
-  else
-    ((double *)w.alm)[a] =
-        __longlong_as_double((long long)(((hi >> (10 + sh)) & 0xFFFFFFFFFFFFFull) | 0x3FF0000000000000ull));
-  w.ale[a] = y.e + inv.e + sh;
-}
-
 // A positive normal float (or 0) as a double, with integer operations.
 __device__ __forceinline__ double f2d_int(float f) {
   const unsigned b = (unsigned)__float_as_int(f);
@@ -335,46 +321,6 @@ struct RowEnds {
   }
 };
 
-// stage_offdiag / stage_diag with H recomputed (same layouts and zeros).
-template <int MODE, bool BWD, bool PBC, int NR>
-__device__ __forceinline__ void stage_offdiag_rc(const Workspace &w, int tt, int i0, void *dmv, int *de,
-                                                 const unsigned long long *T63) {
-  using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
-  const int lane = threadIdx.x & 31;
-  const int srcbase = tt * TILE, row = tt * TILE + TILE + lane;
-  M_t *dm = (M_t *)dmv;
-  RowEnds<MODE, BWD, PBC> re;
-  if (row < w.N) re.load(w, row);
-#pragma unroll 2
-  for (int i = i0; i < i0 + NR; ++i) {
-    M_t m = (M_t)1.0;
-    int e = XZERO_E;
-    if (row < w.N) m = re.h(w, srcbase + i, T63, e);
-    dm[i * 33 + lane] = m;
-    de[i * 33 + lane] = e;
-  }
-}
-template <int MODE, bool BWD, bool PBC, int NR>
-__device__ __forceinline__ void stage_diag_rc(const Workspace &w, int tt, int i0, unsigned long long *dm, int *de,
-                                              const unsigned long long *T63) {
-  using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
-  const int lane = threadIdx.x & 31;
-  const int r0 = tt * TILE, row = r0 + lane;
-  const xd c = (row < w.N) ? xnorm_int(chain_coef<BWD>(w, row)) : xd{1.0, 0};
-  RowEnds<MODE, BWD, PBC> re;
-  if (row < w.N) re.load(w, row);
-#pragma unroll 2
-  for (int i = i0; i < i0 + NR; ++i) {
-    const int src = r0 + i;
-    M_t m = (M_t)1.0;
-    int e = XZERO_E;
-    if (row < w.N && src <= row) m = re.h(w, src, T63, e);
-    const xk k = mul_mant<M_t>(c, m, e);
-    dm[i * 33 + lane] = k.m;
-    de[i * 33 + lane] = k.e;
-  }
-}
-
 // The 32 dependent steps of row tile t, run by one warp.  A is this lane's
 // row sum over sources < 32t except tile t-1 (which is in nxt), crow the row's
 // coefficient.  K (diagonal, c-scaled, integer mantissas) and H (to tile t+1)
@@ -455,49 +401,22 @@ __device__ __forceinline__ void chain_tile(int N, int t, xd A, xd crow, xd &nxt,
   nxt = xnorm_int(nxt);
 }
 
-// ------------------------------------------------ asynchronous copies
-// Bulk copies (TMA) into this CTA's shared memory signal an mbarrier with
-// their byte count; per-thread cp.async copies complete by commit groups.
-// Neither is waited for by the CTA or cluster barriers in between, so a copy
-// issued in one period of a recursion lands during the next.
+// ------------------------------------------------ mbarriers
 __device__ __forceinline__ void mbar_init(unsigned addr, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(addr), "r"(count) : "memory");
 }
 __device__ __forceinline__ void mbar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
+__device__ __forceinline__ void mbar_arrive(unsigned addr) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(addr) : "memory");
+}
 __device__ __forceinline__ void mbar_expect_tx(unsigned addr, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(addr), "r"(bytes) : "memory");
 }
-// generic-proxy accesses of a buffer before the bulk copy that overwrites it
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// bytes (a multiple of 16) from global src to shared dst (both 16-byte aligned)
-__device__ __forceinline__ void bulk_g2s(unsigned dst, const void *src, unsigned bytes, unsigned mbar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(mbar)
-               : "memory");
-}
-// Wait for the mbarrier phase of the given parity, bounded (about a second):
-// on expiry the status word records ST_TIMEOUT and the caller goes on (the
-// evaluation's results are then invalid; the host reports BPIMD_ERR_TIMEOUT).
-__device__ __forceinline__ bool mbar_wait(unsigned addr, unsigned parity, int *status) {
-  for (unsigned i = 0; i < (1u << 25); ++i) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (i >= 64) __nanosleep(32);
-  }
-  atomicOr(status, ST_TIMEOUT);
-  return false;
-}
 // ------------------------------------------ hand-offs between CTAs of a cluster
 // A producer stores into another CTA's shared memory with st.async, each store
-// completing its byte count on an mbarrier of the receiving CTA; one producer
-// thread adds the single expected arrival with the total byte count.  The
-// consumer waits for the phase (its transaction count covers the stores).  No cluster barrier
-// is involved, so producer and consumer run decoupled.
+// completing its byte count on an mbarrier of the receiving CTA, which expects
+// the bytes of the whole hand-off.  No cluster barrier is involved, so
+// producer and consumer run decoupled.
 constexpr unsigned long long WAIT_LIMIT_NS = 1000000000ull;  // bound of every hand-off wait (1 s)
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -510,21 +429,6 @@ __device__ __forceinline__ unsigned cluster_addr(unsigned local, unsigned rank) 
   unsigned r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
   return r;
-}
-__device__ __forceinline__ void st_async_u64(unsigned raddr, unsigned long long v, unsigned rbar) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(raddr), "l"(v),
-               "r"(rbar)
-               : "memory");
-}
-__device__ __forceinline__ void st_async_u32(unsigned raddr, unsigned v, unsigned rbar) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(raddr), "r"(v),
-               "r"(rbar)
-               : "memory");
-}
-// the one expected arrival of a hand-off, with its byte count, on a remote mbarrier
-__device__ __forceinline__ void mbar_arrive_expect_remote(unsigned rbar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(rbar), "r"(bytes)
-               : "memory");
 }
 __device__ __forceinline__ bool mbar_test_cluster(unsigned addr, unsigned parity) {
   unsigned done;
@@ -540,7 +444,6 @@ __device__ __forceinline__ bool mbar_test_cluster(unsigned addr, unsigned parity
 // the caller stops handing off: the status word records ST_TIMEOUT and the
 // evaluation's results are invalid, but every thread still reaches the end.
 __device__ __forceinline__ bool handoff_wait(unsigned addr, unsigned parity, int *status, volatile int *aborted) {
-  if (*aborted) return false;
   if (mbar_test_cluster(addr, parity)) return true;
   const unsigned long long t0 = global_ns();
   while (!mbar_test_cluster(addr, parity)) {
@@ -555,28 +458,6 @@ __device__ __forceinline__ bool handoff_wait(unsigned addr, unsigned parity, int
 // split cluster barrier: arrive (release) once this thread's part is done, wait later
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cp_async16(unsigned dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-// one arrival on a CTA-local mbarrier once this thread's cp.async copies so far
-// have landed (the barrier counts one arrival per copying thread)
-__device__ __forceinline__ void cp_async_arrive(unsigned mbar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(mbar) : "memory");
-}
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-__device__ __forceinline__ void cp_async8(unsigned dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(unsigned dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
 // ------------------------------------------------ the blocked recursion
 // Sums of products in the chain's integer format.  A term K y (K = kk
 // 2^(ke - 63) with kk in [2^63, 2^64), y an xi) is the high product
@@ -621,17 +502,6 @@ __device__ __forceinline__ xi xsum_fin(xsum a) {
   if (e < XZERO_E) return xi{1ull << 62, XZERO_E};
   return xi{a.s << (lz - 1), e};
 }
-// A float partial sum x 2^E (x >= 0) as an xi.
-__device__ __forceinline__ xi xi_from_float(float x, int E) {
-  const unsigned b = (unsigned)__float_as_int(x);
-  if (b < 0x00800000u) return xi{1ull << 62, XZERO_E};
-  return xi{(unsigned long long)((b & 0x7FFFFFu) | 0x800000u) << 39, E + (int)(b >> 23) - 127};
-}
-// The top 24 bits of an xi mantissa as a float in [1, 2) (exponent y.e).
-__device__ __forceinline__ float xi_mant_float(xi y) {
-  return __int_as_float((int)((unsigned)(y.m >> 39) & 0x7FFFFFu) | 0x3F800000);
-}
-
 // Reduced prefix sums C'[i+1] = sum_{q<=i} Ap[q] of tile t (one warp), and the
 // running total of the integer exponent parts n_q that the recursion carries
 // in its exponents (ncarry, exact in 64 bits).

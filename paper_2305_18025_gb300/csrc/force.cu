@@ -29,9 +29,8 @@ __device__ __forceinline__ void block_coords_f(int blk, int &t, int &s) {
   s = blk - tt * (tt + 1) / 2;
 }
 
-__device__ __forceinline__ xd alpha_of(const Workspace &w, int a) {
-  // y_a / (N y_N), stored by the forward recursion
-  return xd{w.mixed ? (double)((const float *)w.alm)[a] : ((const double *)w.alm)[a], w.ale[a]};
+__device__ __forceinline__ xd alpha_of(const Workspace &w, int a) {  // y_a / (N y_N)
+  return xmul(xd{w.yfm[a], w.yfe[a]}, xd{w.scal[1], w.scal_i[0]});
 }
 __device__ __forceinline__ xd mu_of(const Workspace &w, int b) {
   const int r = w.N - 1 - b;  // backward row index of mu_b (0-based mu~_b = Yb[N-1-b])

@@ -108,7 +108,7 @@ size_t layout_workspace(Workspace &w, char *base) {
 }
 
 // one evaluation of V_B and forces on ctx->stream
-int evaluate(bpimd_ctx *ctx, const double *pos, double *V_B, double *F) {
+int evaluate(bpimd_ctx *ctx, const double *pos, double *V_B, double *F, const Beside &beside) {
   const Workspace &w = ctx->w;
   cudaStream_t s = ctx->stream;
   cudaEvent_t *ev = nullptr;
@@ -120,6 +120,7 @@ int evaluate(bpimd_ctx *ctx, const double *pos, double *V_B, double *F) {
   mark(1);
   if (launch_chains(w, V_B, s) != cudaSuccess) return BPIMD_ERR_CUDA;
   mark(2);
+  if (beside && beside() != cudaSuccess) return BPIMD_ERR_CUDA;
   if (launch_prob_forces(w, pos, F, s) != cudaSuccess) return BPIMD_ERR_CUDA;
   mark(3);
   ctx->evaluated = true;

@@ -23,7 +23,7 @@ bool finite_positive(double x) { return std::isfinite(x) && x > 0.0; }
 
 namespace bpimd {
 
-int evaluate_batched(bpimd_ctx *ctx, const double *pos, double *V_B, double *F) {
+int evaluate_batched(bpimd_ctx *ctx, const double *pos, double *V_B, double *F, const Beside &beside) {
   cudaStream_t s = ctx->stream;
   const int mode = ctx->cfg.precision;
   cudaEvent_t *ev = nullptr;
@@ -45,6 +45,7 @@ int evaluate_batched(bpimd_ctx *ctx, const double *pos, double *V_B, double *F) 
                             mode == BPIMD_MIXED32, V_B, s) != cudaSuccess)
     return BPIMD_ERR_CUDA;
   mark(2);
+  if (beside && beside() != cudaSuccess) return BPIMD_ERR_CUDA;
   if (launch_prob_forces_batched(ctx->d_ws, ctx->d_item_tab, ctx->n_item_tab, ctx->d_off, mode, pos, F,
                                  ctx->tune_prob_bpsm, s) != cudaSuccess)
     return BPIMD_ERR_CUDA;

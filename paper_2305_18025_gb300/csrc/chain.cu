@@ -347,6 +347,7 @@ __device__ void run_chain(const Workspace &w, int t0, int np, ChainSmem &sm, dou
   __syncthreads();
   cluster_arrive();
   pdl_wait();
+  pdl_trigger();  // what runs beside the recursions may start; what needs them waits for this grid
   if (t0 == 0 && rank == 0 && tid == 0) {
     gYm[0] = 1.0;
     gYe[0] = 0;
@@ -536,7 +537,6 @@ __device__ void run_chain(const Workspace &w, int t0, int np, ChainSmem &sm, dou
   }
   __syncwarp();
   cluster_arrive();
-  pdl_trigger();
   if (!BWD && rank == 0 && (t0 + np) * PT >= N) {
     // V^{[1,N]} = C'[N] - (ln(y_N) - n ln 2)/beta and the normaliser 1/(N y_N)
     __syncthreads();

@@ -148,7 +148,6 @@ __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *
     }
     __syncthreads();
   }
-  pdl_trigger();  // the probability pass may launch during the epilogue
   if (!BWD) {
     // V^{[1,N]} = C'[N] - (ln(y_N) - n ln 2)/beta, normaliser 1/(N y_N)
     if (q == 6 && lane == 0) { sm.misc[0] = carry; sm.nsum = ncarry; }
@@ -177,6 +176,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, 2) chain_batched_kernel(const W
                                                                          double *V_B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
+  pdl_trigger();  // what runs beside the recursions may start; what needs them waits for this grid
   const int r = order[blockIdx.x >> 1];
   if (blockIdx.x & 1) run_single<MIXED, true>(ws[r], smem_raw, nullptr);
   else run_single<MIXED, false>(ws[r], smem_raw, V_B ? V_B + r : nullptr);

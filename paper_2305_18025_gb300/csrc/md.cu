@@ -24,9 +24,11 @@
 // words become uniforms u = (x + 1/2) 2^-32 and pairs of uniforms become
 // normals by the Box-Muller transform (float64; MIXED: float32).
 //
-// One step (7 kernel launches) is captured once into a CUDA graph bound to the
-// caller's position and velocity buffers and replayed; the step counter lives
-// in device memory and is advanced by the last kernel of the step.
+// A step's closing B and the next step's B A O A are one kernel.  The physical
+// force and the next step's noise need the positions and the counter only, so
+// they are formed while the recursions run.  One step is captured once into a
+// CUDA graph bound to the caller's position and velocity buffers and replayed;
+// the step counter lives in device memory and is advanced by the closing B.
 #include <cmath>
 #include <vector>
 #include <type_traits>
@@ -84,41 +86,56 @@ __device__ __forceinline__ void box_muller(const uint32_t x[4], double z[4]) {
   }
 }
 
-// B A O A of one step (four velocity components per thread: one Philox block).
+// Thermostat kicks c2 z of elements 4g .. 4g+3 (one Philox block) of step s.
+// They depend on the counter only, so the pair-force kernel's spare blocks
+// form them while the recursions run (a float64 Box-Muller is ~15 us of
+// latency on the step's path otherwise).
 template <bool MIXED>
-__global__ void __launch_bounds__(MD_THREADS) md_baoa_kernel(double *__restrict__ x, double *__restrict__ v,
-                                                             const double *__restrict__ F, long long n,
-                                                             double half_dt_over_m, double half_dt, double c1,
-                                                             double c2, uint32_t k0, uint32_t k1,
-                                                             const unsigned long long *__restrict__ step) {
-  const unsigned long long s = *step;
-  for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; 4 * g < n;
-       g += (long long)gridDim.x * blockDim.x) {
-    uint32_t c[4] = {(uint32_t)g, (uint32_t)s, (uint32_t)(s >> 32), 0u};
-    philox4x32_10(c, k0, k1);
-    double z[4];
-    box_muller<MIXED>(c, z);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long long e = 4 * g + i;
-      if (e < n) {
-        double vi = v[e] + half_dt_over_m * F[e];  // B
-        double xi = x[e] + half_dt * vi;           // A
-        vi = c1 * vi + c2 * z[i];                  // O
-        x[e] = xi + half_dt * vi;                  // A
-        v[e] = vi;
-      }
-    }
-  }
+__device__ __forceinline__ void thermostat_kicks(long long g, unsigned long long s, uint32_t k0, uint32_t k1,
+                                                 double (&z)[4]) {
+  uint32_t c[4] = {(uint32_t)g, (uint32_t)s, (uint32_t)(s >> 32), 0u};
+  philox4x32_10(c, k0, k1);
+  box_muller<MIXED>(c, z);
 }
 
-// Closing B of a step; advances the step counter.
-__global__ void __launch_bounds__(MD_THREADS) md_kick_kernel(double *__restrict__ v, const double *__restrict__ F,
-                                                             long long n, double half_dt_over_m,
-                                                             unsigned long long *step) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-    v[e] += half_dt_over_m * F[e];
-  if (blockIdx.x == 0 && threadIdx.x == 0) *step += 1ull;
+// K: closing B of a step (and its counter); A: B A O of the next, with the
+// full force F + Fx (exchange, physical) and the thermostat kicks zc (null:
+// none).  Two elements a thread, 16-byte accesses.
+template <bool K, bool A>
+__global__ void __launch_bounds__(MD_THREADS) md_update_kernel(double *__restrict__ x, double *__restrict__ v,
+                                                               const double *__restrict__ F,
+                                                               const double *__restrict__ Fx,
+                                                               const double *__restrict__ zc, long long n, double h,
+                                                               double half_dt, double c1, unsigned long long *step) {
+  pdl_wait();
+  auto one = [&](double &xe, double &ve, double Fe, double ze) {
+    if (K) ve = fma(h, Fe, ve);  // B
+    if (A) {
+      ve = fma(h, Fe, ve);        // B
+      xe = fma(half_dt, ve, xe);  // A
+      ve = fma(c1, ve, ze);       // O
+      xe = fma(half_dt, ve, xe);  // A
+    }
+  };
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; 2 * g < n; g += stride) {
+    if (2 * g + 1 < n) {
+      const double2 f = ((const double2 *)F)[g], fx = ((const double2 *)Fx)[g];
+      const double2 z = A && zc ? ((const double2 *)zc)[g] : make_double2(0.0, 0.0);
+      double2 ve = ((double2 *)v)[g], xe = A ? ((double2 *)x)[g] : make_double2(0.0, 0.0);
+      one(xe.x, ve.x, f.x + fx.x, z.x);
+      one(xe.y, ve.y, f.y + fx.y, z.y);
+      if (A) ((double2 *)x)[g] = xe;
+      ((double2 *)v)[g] = ve;
+    } else {
+      const long long e = 2 * g;
+      double xe = A ? x[e] : 0.0, ve = v[e];
+      one(xe, ve, F[e] + Fx[e], A && zc ? zc[e] : 0.0);
+      if (A) x[e] = xe;
+      v[e] = ve;
+    }
+  }
+  if (K && blockIdx.x == 0 && threadIdx.x == 0) *step += 1ull;
 }
 
 // Deterministic block sum (fixed shuffle tree, then warps in order); thread 0 gets it.
@@ -181,7 +198,7 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
   return s;
 }
 
-// -grad U-bar added to F, per bead index j = blockIdx.y and particle
+// -grad U-bar into Fx, per bead index j = blockIdx.y and particle
 // l = blockIdx.x * (256 / SPLIT) + thread / SPLIT (all pairs).  The SPLIT
 // lanes of one particle take the partners q = sub, sub + SPLIT, ...
 // of each staged chunk and combine their sums by a fixed shuffle butterfly;
@@ -191,7 +208,7 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
 // periodic box (PBC) pair distances by minimum image.  MIXED: pair terms in
 // float32, accumulated per lane in float32 and added to the float64 force.
 template <bool MIXED, bool PBC, int SPLIT>
-__device__ __forceinline__ double ext_force_body(const double *__restrict__ pos, double *__restrict__ F, int N,
+__device__ __forceinline__ double ext_force_body(const double *__restrict__ pos, double *__restrict__ Fx, int N,
                                                  int P, const PairParams &pp, int lb, int j,
                                                  typename std::conditional<MIXED, float4, Dbl4>::type *sr,
                                                  double *red, unsigned long long *T63s) {
@@ -278,10 +295,10 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
     float ulf = 0.0f;
     if (valid && sub == 0) {
       if (pp.pair == BPIMD_PAIR_GAUSSIAN) u -= 1.0f;  // the self term (d = 0, e = 1) carries no force
-      double *f = F + ((size_t)l * P + j) * 3;
-      f[0] += f64_of_f32(pp.finv_P * (pp.ffs * fx - pp.fkt * px));
-      f[1] += f64_of_f32(pp.finv_P * (pp.ffs * fy - pp.fkt * py));
-      f[2] += f64_of_f32(pp.finv_P * (pp.ffs * fz - pp.fkt * pz));
+      double *f = Fx + ((size_t)l * P + j) * 3;
+      f[0] = f64_of_f32(pp.finv_P * (pp.ffs * fx - pp.fkt * px));
+      f[1] = f64_of_f32(pp.finv_P * (pp.ffs * fy - pp.fkt * py));
+      f[2] = f64_of_f32(pp.finv_P * (pp.ffs * fz - pp.fkt * pz));
       const float up = pp.pair == BPIMD_PAIR_GAUSSIAN ? pp.fup * u : pp.fup * u - pp.fush * (float)nin;
       ulf = pp.finv_P * (up + 0.5f * pp.fkt * (px * px + py * py + pz * pz));
     }
@@ -290,11 +307,11 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
   double ul = 0.0;
   if (valid && sub == 0) {
     if (pp.pair == BPIMD_PAIR_GAUSSIAN) u -= (R)1;  // the self term (d = 0, e = 1) carries no force
-    double *f = F + ((size_t)l * P + j) * 3;
+    double *f = Fx + ((size_t)l * P + j) * 3;
     const double fs = pp.pair == BPIMD_PAIR_GAUSSIAN ? pp.ga * pp.inv_s2 : 24.0 * pp.eps;
-    f[0] += pp.inv_P * (fs * (double)fx - pp.kt * rx);
-    f[1] += pp.inv_P * (fs * (double)fy - pp.kt * ry);
-    f[2] += pp.inv_P * (fs * (double)fz - pp.kt * rz);
+    f[0] = pp.inv_P * (fs * (double)fx - pp.kt * rx);
+    f[1] = pp.inv_P * (fs * (double)fy - pp.kt * ry);
+    f[2] = pp.inv_P * (fs * (double)fz - pp.kt * rz);
     const double up = pp.pair == BPIMD_PAIR_GAUSSIAN ? 0.5 * pp.ga * (double)u
                                                     : 0.5 * (4.0 * pp.eps * (double)u - pp.ushift * nin);
     ul = pp.inv_P * (up + 0.5 * pp.kt * (rx * rx + ry * ry + rz * rz));
@@ -302,15 +319,55 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
   return block_sum(ul, red);
 }
 
+// Thermostat kicks of one step, n elements (see md_run): element's amplitude
+// c2, or per replica c2r with the packed offsets off.
+struct Kicks {
+  double *zc;  // null: none wanted
+  long long n;
+  double c2;
+  const double *c2r;
+  const long long *off;
+  int R;
+  uint32_t k0, k1;
+  const unsigned long long *step;
+  int ahead;   // steps from the counter to the one wanted
+};
+
+// The physical force is launched between the recursions and the exterior
+// forces and needs only the positions, which were final before the recursions
+// could start: it does not wait for them, but runs beside them on the SMs they
+// leave free.  Its first block waits for them before it ends, so that the next
+// kernel's wait for this one covers both.
+__device__ __forceinline__ void after_recursions(bool first_block) {
+  pdl_trigger();
+  if (first_block) pdl_wait();
+}
+
+template <bool MIXED>
+__device__ void kicks_block(const Kicks &k, long long blk, long long nblk);
+
 template <bool MIXED, bool PBC>
-__global__ void __launch_bounds__(EXT_THREADS) ext_force_kernel(const double *__restrict__ pos, double *__restrict__ F,
-                                                                int N, int P, PairParams pp, double *ubar_part) {
+__global__ void __launch_bounds__(EXT_THREADS) ext_force_kernel(const double *__restrict__ pos,
+                                                                double *__restrict__ Fx, int N, int P, PairParams pp,
+                                                                double *ubar_part, Kicks kicks) {
   using R4 = typename std::conditional<MIXED, float4, Dbl4>::type;
   __shared__ R4 sr[EXT_CHUNK];
   __shared__ double red[EXT_THREADS / 32];
   __shared__ unsigned long long T63s[256];  // float64: the table of the integer-pipe power of two
-  const double s = ext_force_body<MIXED, PBC, EXT_SPLIT>(pos, F, N, P, pp, blockIdx.x, blockIdx.y, sr, red, T63s);
-  if (threadIdx.x == 0) ubar_part[blockIdx.y * gridDim.x + blockIdx.x] = s;
+  if ((int)blockIdx.y < P) {
+    const double s = ext_force_body<MIXED, PBC, EXT_SPLIT>(pos, Fx, N, P, pp, blockIdx.x, blockIdx.y, sr, red, T63s);
+    if (threadIdx.x == 0) ubar_part[blockIdx.y * gridDim.x + blockIdx.x] = s;
+  } else {
+    kicks_block<MIXED>(kicks, (blockIdx.y - P) * (long long)gridDim.x + blockIdx.x,
+                       (long long)(gridDim.y - P) * gridDim.x);
+  }
+  after_recursions(blockIdx.x == 0 && blockIdx.y == 0);
+}
+
+// thermostat kicks alone (the cell-list path)
+template <bool MIXED>
+__global__ void __launch_bounds__(EXT_THREADS) md_kicks_kernel(Kicks kicks) {
+  kicks_block<MIXED>(kicks, blockIdx.x, gridDim.x);
 }
 
 // ----------------------------------------------------------- replica batches
@@ -326,33 +383,31 @@ __device__ __forceinline__ int replica_of(const long long *__restrict__ off, int
   return lo;
 }
 
-// B A O A over every replica of a batch: as md_baoa_kernel, with the
-// thermostat amplitude c2 of each element's replica (its own temperature).
+// Blocks blk of nblk of the kicks: four elements a thread.
 template <bool MIXED>
-__global__ void __launch_bounds__(MD_THREADS) md_baoa_batched(double *__restrict__ x, double *__restrict__ v,
-                                                              const double *__restrict__ F, long long n,
-                                                              double half_dt_over_m, double half_dt, double c1,
-                                                              const double *__restrict__ c2r,
-                                                              const long long *__restrict__ off, int R, uint32_t k0,
-                                                              uint32_t k1, const unsigned long long *__restrict__ step) {
-  const unsigned long long s = *step;
-  for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; 4 * g < n;
-       g += (long long)gridDim.x * blockDim.x) {
-    uint32_t c[4] = {(uint32_t)g, (uint32_t)s, (uint32_t)(s >> 32), 0u};
-    philox4x32_10(c, k0, k1);
+__device__ void kicks_block(const Kicks &k, long long blk, long long nblk) {
+  if (!k.zc) return;
+  const unsigned long long s = *k.step + (unsigned long long)k.ahead;
+  for (long long g = blk * (long long)blockDim.x + threadIdx.x; 4 * g < k.n; g += nblk * blockDim.x) {
     double z[4];
-    box_muller<MIXED>(c, z);
+    thermostat_kicks<MIXED>(g, s, k.k0, k.k1, z);
+    int r = 0;
+    long long next = k.n;
+    double c2 = k.c2;
+    if (k.off) {  // one search a block of four; a replica may end inside it
+      r = replica_of(k.off, k.R, 4 * g);
+      next = r + 1 < k.R ? __ldg(k.off + r + 1) : k.n;
+      c2 = __ldg(k.c2r + r);
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const long long e = 4 * g + i;
-      if (e < n) {
-        const double c2 = __ldg(c2r + replica_of(off, R, e));
-        double vi = v[e] + half_dt_over_m * F[e];  // B
-        double xi = x[e] + half_dt * vi;           // A
-        vi = c1 * vi + c2 * z[i];                  // O
-        x[e] = xi + half_dt * vi;                  // A
-        v[e] = vi;
+      while (e >= next && r + 1 < k.R) {
+        ++r;
+        next = r + 1 < k.R ? __ldg(k.off + r + 1) : k.n;
+        c2 = __ldg(k.c2r + r);
       }
+      if (e < k.n) k.zc[e] = c2 * z[i];
     }
   }
 }
@@ -363,25 +418,32 @@ __global__ void __launch_bounds__(MD_THREADS) md_baoa_batched(double *__restrict
 // particles per block (the batch's pair tile, bpimd_batch_set_pair_tile).
 template <bool MIXED, int SPLIT>
 __global__ void __launch_bounds__(EXT_THREADS) ext_force_batched(const double *__restrict__ pos,
-                                                                 double *__restrict__ F,
+                                                                 double *__restrict__ Fx,
                                                                  const Workspace *__restrict__ ws,
                                                                  const long long *__restrict__ off,
                                                                  const int4 *__restrict__ tab, int ntab, PairParams pp,
-                                                                 double *ubar_part) {
+                                                                 double *ubar_part, Kicks kicks, int kick_blocks) {
   using R4 = typename std::conditional<MIXED, float4, Dbl4>::type;
   __shared__ R4 sr[EXT_CHUNK];
   __shared__ double red[EXT_THREADS / 32];
   __shared__ unsigned long long T63s[256];
-  for (int k = blockIdx.x; k < ntab; k += gridDim.x) {
+  if ((int)blockIdx.x < kick_blocks) {
+    kicks_block<MIXED>(kicks, blockIdx.x, kick_blocks);
+    after_recursions(blockIdx.x == 0);
+    return;
+  }
+  const int b0 = blockIdx.x - kick_blocks, nb = gridDim.x - kick_blocks;
+  for (int k = b0; k < ntab; k += nb) {
     const int4 e = tab[k];
     const int N = ws[e.x].N, P = ws[e.x].P;
     PairParams q = pp;
     q.inv_P = ws[e.x].inv_P;
     q.finv_P = f32_of_f64(q.inv_P);
-    const double s = ext_force_body<MIXED, false, SPLIT>(pos + off[e.x], F + off[e.x], N, P, q, e.y, e.z, sr, red, T63s);
+    const double s = ext_force_body<MIXED, false, SPLIT>(pos + off[e.x], Fx + off[e.x], N, P, q, e.y, e.z, sr, red, T63s);
     if (threadIdx.x == 0) ubar_part[k] = s;
     __syncthreads();  // sr is reused by the next entry
   }
+  after_recursions(blockIdx.x == 0);
 }
 
 // energies[4 r + 0..3] of replica r (one block each): V_B, U-bar, kinetic,
@@ -534,42 +596,104 @@ int grid_for(long long work, int threads) {
   return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
-// F(pos) = exchange force (Algorithm 1) + physical force, U-bar partials.
-int total_force(bpimd_ctx *ctx, const MDParams &p, const double *pos) {
-  MDState &md = ctx->md;
-  int rc = evaluate(ctx, pos, md.VB, md.F);
-  if (rc != BPIMD_OK) return rc;
-  if (p.cell_nc > 0)
-    return cell_list_forces(pos, md.F, ctx->cfg.N, ctx->cfg.P, p.pp, ctx->w.bead32, md.cells, md.ubar_part,
-                            ctx->stream) == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
-  const dim3 grid((ctx->cfg.N + EXT_PARTICLES - 1) / EXT_PARTICLES, ctx->cfg.P);
-  const int N = ctx->cfg.N, P = ctx->cfg.P;
-  if (ctx->w.bead32) {
-    if (p.pp.pbc) ext_force_kernel<true, true><<<grid, EXT_THREADS, 0, ctx->stream>>>(pos, md.F, N, P, p.pp, md.ubar_part);
-    else ext_force_kernel<true, false><<<grid, EXT_THREADS, 0, ctx->stream>>>(pos, md.F, N, P, p.pp, md.ubar_part);
-  } else {
-    if (p.pp.pbc) ext_force_kernel<false, true><<<grid, EXT_THREADS, 0, ctx->stream>>>(pos, md.F, N, P, p.pp, md.ubar_part);
-    else ext_force_kernel<false, false><<<grid, EXT_THREADS, 0, ctx->stream>>>(pos, md.F, N, P, p.pp, md.ubar_part);
-  }
-  return cudaGetLastError() == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
+// Which thermostat kicks a force pass forms beside it: those of the step the
+// counter shows, of the one after it, or none.
+enum KickStep { KICKS_NOW = 0, KICKS_NEXT = 1, KICKS_NONE = -1 };
+
+Kicks kicks_of(const MDState &md, const MDParams &p, KickStep ks) {
+  Kicks k = {};
+  k.zc = (ks == KICKS_NONE || p.c1 == 1.0) ? nullptr : md.zc;  // no friction: no kicks
+  k.n = p.n;
+  k.c2 = p.c2;
+  k.c2r = md.c2r;
+  k.k0 = p.k0;
+  k.k1 = p.k1;
+  k.step = md.step;
+  k.ahead = ks == KICKS_NEXT ? 1 : 0;
+  return k;
 }
 
-// Enqueue one step (B A O A, force, B) on the context stream.
-int enqueue_step(bpimd_ctx *ctx, const MDParams &p, double *pos, double *vel) {
+// md.F = exchange force (Algorithm 1) and md.Fx = physical force of pos, with
+// the U-bar partials and the thermostat kicks of step `ks`.
+int total_force(bpimd_ctx *ctx, const MDParams &p, const double *pos, KickStep ks) {
   MDState &md = ctx->md;
   cudaStream_t s = ctx->stream;
-  const int g4 = grid_for((p.n + 3) / 4, MD_THREADS), g1 = grid_for(p.n, MD_THREADS);
-  if (ctx->w.bead32)
-    md_baoa_kernel<true><<<g4, MD_THREADS, 0, s>>>(pos, vel, md.F, p.n, p.half_dt_over_m, p.half_dt, p.c1, p.c2,
-                                                   p.k0, p.k1, md.step);
-  else
-    md_baoa_kernel<false><<<g4, MD_THREADS, 0, s>>>(pos, vel, md.F, p.n, p.half_dt_over_m, p.half_dt, p.c1, p.c2,
-                                                    p.k0, p.k1, md.step);
-  if (cudaGetLastError() != cudaSuccess) return BPIMD_ERR_CUDA;
-  int rc = total_force(ctx, p, pos);
-  if (rc != BPIMD_OK) return rc;
-  md_kick_kernel<<<g1, MD_THREADS, 0, s>>>(vel, md.F, p.n, p.half_dt_over_m, md.step);
-  return cudaGetLastError() == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
+  const Kicks kicks = kicks_of(md, p, ks);
+  const int kick_blocks = kicks.zc ? grid_for((p.n + 3) / 4, EXT_THREADS) : 0;
+  if (p.cell_nc > 0) {
+    // the cell-list kernels run beside the whole evaluation, on a stream of their own
+    if (cudaEventRecord(md.fork, s) != cudaSuccess || cudaStreamWaitEvent(md.side, md.fork, 0) != cudaSuccess)
+      return BPIMD_ERR_CUDA;
+    if (kicks.zc) {
+      if (ctx->w.bead32) md_kicks_kernel<true><<<kick_blocks, EXT_THREADS, 0, md.side>>>(kicks);
+      else md_kicks_kernel<false><<<kick_blocks, EXT_THREADS, 0, md.side>>>(kicks);
+    }
+    int rc = cell_list_forces(pos, md.Fx, ctx->cfg.N, ctx->cfg.P, p.pp, ctx->w.bead32, md.cells, md.ubar_part,
+                              md.side) == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
+    if (cudaEventRecord(md.join, md.side) != cudaSuccess) rc = BPIMD_ERR_CUDA;
+    const int re = evaluate(ctx, pos, md.VB, md.F);
+    if (cudaStreamWaitEvent(s, md.join, 0) != cudaSuccess) return BPIMD_ERR_CUDA;
+    return rc != BPIMD_OK ? rc : re;
+  }
+  const int N = ctx->cfg.N, P = ctx->cfg.P, gx = (N + EXT_PARTICLES - 1) / EXT_PARTICLES;
+  const dim3 grid(gx, P + (kick_blocks + gx - 1) / gx);
+  return evaluate(ctx, pos, md.VB, md.F, [&] {
+    auto go = [&](auto kernel) {
+      return launch_pdl(kernel, grid, EXT_THREADS, 0, s, pos, md.Fx, N, P, p.pp, md.ubar_part, kicks);
+    };
+    if (ctx->w.bead32) return p.pp.pbc ? go(ext_force_kernel<true, true>) : go(ext_force_kernel<true, false>);
+    return p.pp.pbc ? go(ext_force_kernel<false, true>) : go(ext_force_kernel<false, false>);
+  });
+}
+
+// Closing B of a step (K) and B A O A of the next (A), in one pass over the
+// arrays where both are due.
+template <bool K, bool A>
+int launch_update(bpimd_ctx *ctx, const MDParams &p, double *pos, double *vel) {
+  MDState &md = ctx->md;
+  return launch_pdl(md_update_kernel<K, A>, grid_for((p.n + 1) / 2, MD_THREADS), MD_THREADS, 0, ctx->stream, pos, vel,
+                    md.F, md.Fx, p.c1 == 1.0 ? nullptr : md.zc, p.n, p.half_dt_over_m, p.half_dt, p.c1, md.step) ==
+                 cudaSuccess
+             ? BPIMD_OK
+             : BPIMD_ERR_CUDA;
+}
+
+// Steps of one call: `force(ks)` enqueues a force pass.  The first B A O A, then
+// nsteps - 1 times a force pass with the closing B and the next step's B A O A
+// (captured once into a graph bound to the buffers, not on the legacy default
+// stream), then the last force pass and closing B.
+template <typename Force>
+int run_steps(bpimd_ctx *ctx, const MDParams &p, double *pos, double *vel, int32_t nsteps, Force force) {
+  MDState &md = ctx->md;
+  int rc = force(nsteps > 0 ? KICKS_NOW : KICKS_NONE);  // the caller may have moved the positions since the last call
+  if (rc != BPIMD_OK || nsteps == 0) return rc;
+  if ((rc = launch_update<false, true>(ctx, p, pos, vel)) != BPIMD_OK) return rc;
+  auto step = [&] {
+    const int r = force(KICKS_NEXT);
+    return r != BPIMD_OK ? r : launch_update<true, true>(ctx, p, pos, vel);
+  };
+  const bool use_graph = ctx->stream != nullptr && nsteps > 1;
+  if (use_graph && (!md.exec || md.g_pos != pos || md.g_vel != vel)) {
+    if (md.exec) { cudaGraphExecDestroy(md.exec); md.exec = nullptr; }
+    if (md.graph) { cudaGraphDestroy(md.graph); md.graph = nullptr; }
+    if (cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return BPIMD_ERR_CUDA;
+    const int rc_step = step();
+    const cudaError_t e = cudaStreamEndCapture(ctx->stream, &md.graph);
+    if (rc_step != BPIMD_OK || e != cudaSuccess || cudaGraphInstantiate(&md.exec, md.graph, 0) != cudaSuccess) {
+      cudaGetLastError();
+      return BPIMD_ERR_CUDA;
+    }
+    md.g_pos = pos;
+    md.g_vel = vel;
+  }
+  for (int32_t k = 1; k < nsteps && rc == BPIMD_OK; ++k) {
+    if (use_graph) rc = cudaGraphLaunch(md.exec, ctx->stream) == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
+    else rc = step();
+  }
+  if (rc == BPIMD_OK) rc = force(KICKS_NONE);
+  if (rc == BPIMD_OK) rc = launch_update<true, false>(ctx, p, pos, vel);
+  if (rc == BPIMD_OK) md.steps_taken += (uint64_t)nsteps;
+  return rc;
 }
 
 int md_alloc(bpimd_ctx *ctx, const MDParams &p) {
@@ -581,14 +705,21 @@ int md_alloc(bpimd_ctx *ctx, const MDParams &p) {
       return BPIMD_ERR_NOMEM;
     }
     cell_list_layout(md.cells, (char *)md.cell_block, ctx->cfg.N, ctx->cfg.P, p.cell_nc, ctx->w.bead32);
+    if (cudaStreamCreateWithFlags(&md.side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&md.fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&md.join, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      md_free(&md);
+      return BPIMD_ERR_NOMEM;
+    }
   }
   const size_t n = (size_t)ctx->cfg.N * ctx->cfg.P * 3;
   md.ext_blocks = p.cell_nc > 0 ? cell_list_partials(ctx->cfg.N, ctx->cfg.P)
                                  : ((ctx->cfg.N + EXT_PARTICLES - 1) / EXT_PARTICLES) * ctx->cfg.P;
   md.ke_blocks = grid_for((long long)n, MD_THREADS);
   md.spring_blocks = ctx->w.NB;
-  if (cudaMalloc(&md.F, sizeof(double) * n) != cudaSuccess ||
-      cudaMalloc(&md.VB, sizeof(double)) != cudaSuccess ||
+  if (cudaMalloc(&md.F, sizeof(double) * n) != cudaSuccess || cudaMalloc(&md.Fx, sizeof(double) * n) != cudaSuccess ||
+      cudaMalloc(&md.zc, sizeof(double) * n) != cudaSuccess || cudaMalloc(&md.VB, sizeof(double)) != cudaSuccess ||
       cudaMalloc(&md.ubar_part, sizeof(double) * md.ext_blocks) != cudaSuccess ||
       cudaMalloc(&md.ke_part, sizeof(double) * md.ke_blocks) != cudaSuccess ||
       cudaMalloc(&md.spring_part, sizeof(double) * md.spring_blocks) != cudaSuccess ||
@@ -615,6 +746,11 @@ void md_free(MDState *md) {
   if (md->exec) cudaGraphExecDestroy(md->exec);
   if (md->graph) cudaGraphDestroy(md->graph);
   cudaFree(md->F);
+  cudaFree(md->Fx);
+  cudaFree(md->zc);
+  if (md->side) cudaStreamDestroy(md->side);
+  if (md->fork) cudaEventDestroy(md->fork);
+  if (md->join) cudaEventDestroy(md->join);
   cudaFree(md->VB);
   cudaFree(md->ubar_part);
   cudaFree(md->ke_part);
@@ -633,33 +769,7 @@ int md_run(bpimd_ctx *ctx, double *pos, double *vel, int32_t nsteps, double *ene
   // stage profiling is not recorded inside MD steps
   const bool prof = ctx->prof_on;
   ctx->prof_on = false;
-  // the caller may have moved the positions since the last call
-  rc = total_force(ctx, p, pos);
-  // capture one step into a graph (not possible on the legacy default stream)
-  const bool use_graph = ctx->stream != nullptr && nsteps > 1;
-  if (rc == BPIMD_OK && use_graph && (!md.exec || md.g_pos != pos || md.g_vel != vel)) {
-    if (md.exec) { cudaGraphExecDestroy(md.exec); md.exec = nullptr; }
-    if (md.graph) { cudaGraphDestroy(md.graph); md.graph = nullptr; }
-    if (cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-      rc = BPIMD_ERR_CUDA;
-    } else {
-      const int rc_step = enqueue_step(ctx, p, pos, vel);
-      const cudaError_t e = cudaStreamEndCapture(ctx->stream, &md.graph);
-      if (rc_step != BPIMD_OK || e != cudaSuccess ||
-          cudaGraphInstantiate(&md.exec, md.graph, 0) != cudaSuccess) {
-        cudaGetLastError();
-        rc = BPIMD_ERR_CUDA;
-      } else {
-        md.g_pos = pos;
-        md.g_vel = vel;
-      }
-    }
-  }
-  for (int32_t s = 0; s < nsteps && rc == BPIMD_OK; ++s) {
-    if (use_graph) rc = cudaGraphLaunch(md.exec, ctx->stream) == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
-    else rc = enqueue_step(ctx, p, pos, vel);
-  }
-  if (rc == BPIMD_OK) md.steps_taken += (uint64_t)nsteps;
+  rc = run_steps(ctx, p, pos, vel, nsteps, [&](KickStep ks) { return total_force(ctx, p, pos, ks); });
   if (rc == BPIMD_OK && energies) {
     cudaStream_t s = ctx->stream;
     const int g1 = md.ke_blocks;
@@ -680,10 +790,8 @@ int md_run(bpimd_ctx *ctx, double *pos, double *vel, int32_t nsteps, double *ene
 // bpimd_step on a batch context: every replica advances by the same BAOAB
 // steps (shared dt, gamma, trap, Gaussian pair potential and seed; each
 // replica thermostatted at its own kT = 1/beta_r unless cfg.kT_bead > 0).
-// One step is: the batched B A O A kernel, the three evaluation launches of
-// the batch (plus one per replica above 4096 particles), the batched trap and
-// pair forces, and the closing B -- captured once into a CUDA graph bound to
-// the caller's buffers and replayed.  Thermostat noise: Philox4x32-10 with the
+// The steps run as a single system's (run_steps), with the batch evaluation and
+// the batched trap and pair forces.  Thermostat noise: Philox4x32-10 with the
 // element index of the packed arrays as the counter.
 namespace {
 
@@ -726,7 +834,8 @@ int md_alloc_batched(bpimd_ctx *ctx, const MDParams &p) {
     const double kT = ctx->cfg.kT_bead > 0.0 ? ctx->cfg.kT_bead : 1.0 / ctx->h_ws[r].beta;
     c2[r] = std::sqrt((1.0 - p.c1 * p.c1) * kT / ctx->cfg.m);
   }
-  if (cudaMalloc(&md.F, sizeof(double) * n) != cudaSuccess || cudaMalloc(&md.VBr, sizeof(double) * R) != cudaSuccess ||
+  if (cudaMalloc(&md.F, sizeof(double) * n) != cudaSuccess || cudaMalloc(&md.Fx, sizeof(double) * n) != cudaSuccess ||
+      cudaMalloc(&md.zc, sizeof(double) * n) != cudaSuccess || cudaMalloc(&md.VBr, sizeof(double) * R) != cudaSuccess ||
       cudaMalloc(&md.c2r, sizeof(double) * R) != cudaSuccess ||
       cudaMalloc(&md.ext_tab, sizeof(int4) * md.ext_cap) != cudaSuccess ||
       cudaMalloc(&md.ext_first, sizeof(int) * (R + 1)) != cudaSuccess ||
@@ -752,40 +861,25 @@ int md_alloc_batched(bpimd_ctx *ctx, const MDParams &p) {
   return BPIMD_OK;
 }
 
-int total_force_batched(bpimd_ctx *ctx, const MDParams &p, const double *pos) {
+int total_force_batched(bpimd_ctx *ctx, const MDParams &p, const double *pos, KickStep ks) {
   MDState &md = ctx->md;
-  int rc = evaluate_batched(ctx, pos, md.VBr, md.F);
-  if (rc != BPIMD_OK) return rc;
-  const int grid = md.n_ext < sm_count() * 8 ? md.n_ext : sm_count() * 8;
-  auto go = [&](auto kernel) {
-    kernel<<<grid, EXT_THREADS, 0, ctx->stream>>>(pos, md.F, ctx->d_ws, ctx->d_off, md.ext_tab, md.n_ext, p.pp,
-                                                  md.ubar_part);
-  };
-  const bool m = ctx->w.bead32;
-  switch (ctx->pair_lanes) {
-    case 2: m ? go(ext_force_batched<true, 2>) : go(ext_force_batched<false, 2>); break;
-    case 8: m ? go(ext_force_batched<true, 8>) : go(ext_force_batched<false, 8>); break;
-    default: m ? go(ext_force_batched<true, 4>) : go(ext_force_batched<false, 4>); break;
-  }
-  return cudaGetLastError() == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
-}
-
-int enqueue_step_batched(bpimd_ctx *ctx, const MDParams &p, double *pos, double *vel) {
-  MDState &md = ctx->md;
-  cudaStream_t s = ctx->stream;
-  const long long n = ctx->total_elems;
-  const int g4 = grid_for((n + 3) / 4, MD_THREADS), g1 = grid_for(n, MD_THREADS);
-  if (ctx->w.bead32)
-    md_baoa_batched<true><<<g4, MD_THREADS, 0, s>>>(pos, vel, md.F, n, p.half_dt_over_m, p.half_dt, p.c1, md.c2r,
-                                                    ctx->d_off, ctx->R, p.k0, p.k1, md.step);
-  else
-    md_baoa_batched<false><<<g4, MD_THREADS, 0, s>>>(pos, vel, md.F, n, p.half_dt_over_m, p.half_dt, p.c1, md.c2r,
-                                                     ctx->d_off, ctx->R, p.k0, p.k1, md.step);
-  if (cudaGetLastError() != cudaSuccess) return BPIMD_ERR_CUDA;
-  int rc = total_force_batched(ctx, p, pos);
-  if (rc != BPIMD_OK) return rc;
-  md_kick_kernel<<<g1, MD_THREADS, 0, s>>>(vel, md.F, n, p.half_dt_over_m, md.step);
-  return cudaGetLastError() == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
+  Kicks kicks = kicks_of(md, p, ks);
+  kicks.off = ctx->d_off;
+  kicks.R = ctx->R;
+  const int kick_blocks = kicks.zc ? grid_for((p.n + 3) / 4, EXT_THREADS) : 0;
+  const int grid = kick_blocks + (md.n_ext < sm_count() * 8 ? md.n_ext : sm_count() * 8);
+  return evaluate_batched(ctx, pos, md.VBr, md.F, [&] {
+    auto go = [&](auto kernel) {
+      return launch_pdl(kernel, grid, EXT_THREADS, 0, ctx->stream, pos, md.Fx, ctx->d_ws, ctx->d_off, md.ext_tab,
+                        md.n_ext, p.pp, md.ubar_part, kicks, kick_blocks);
+    };
+    const bool m = ctx->w.bead32;
+    switch (ctx->pair_lanes) {
+      case 2: return m ? go(ext_force_batched<true, 2>) : go(ext_force_batched<false, 2>);
+      case 8: return m ? go(ext_force_batched<true, 8>) : go(ext_force_batched<false, 8>);
+      default: return m ? go(ext_force_batched<true, 4>) : go(ext_force_batched<false, 4>);
+    }
+  });
 }
 
 }  // namespace
@@ -832,30 +926,7 @@ int md_run_batched(bpimd_ctx *ctx, double *pos, double *vel, int32_t nsteps, dou
   if (!md.ready && (rc = md_alloc_batched(ctx, p)) != BPIMD_OK) return rc;
   const bool prof = ctx->prof_on;
   ctx->prof_on = false;
-  rc = total_force_batched(ctx, p, pos);
-  const bool use_graph = ctx->stream != nullptr && nsteps > 1;
-  if (rc == BPIMD_OK && use_graph && (!md.exec || md.g_pos != pos || md.g_vel != vel)) {
-    if (md.exec) { cudaGraphExecDestroy(md.exec); md.exec = nullptr; }
-    if (md.graph) { cudaGraphDestroy(md.graph); md.graph = nullptr; }
-    if (cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-      rc = BPIMD_ERR_CUDA;
-    } else {
-      const int rc_step = enqueue_step_batched(ctx, p, pos, vel);
-      const cudaError_t e = cudaStreamEndCapture(ctx->stream, &md.graph);
-      if (rc_step != BPIMD_OK || e != cudaSuccess || cudaGraphInstantiate(&md.exec, md.graph, 0) != cudaSuccess) {
-        cudaGetLastError();
-        rc = BPIMD_ERR_CUDA;
-      } else {
-        md.g_pos = pos;
-        md.g_vel = vel;
-      }
-    }
-  }
-  for (int32_t k = 0; k < nsteps && rc == BPIMD_OK; ++k) {
-    if (use_graph) rc = cudaGraphLaunch(md.exec, ctx->stream) == cudaSuccess ? BPIMD_OK : BPIMD_ERR_CUDA;
-    else rc = enqueue_step_batched(ctx, p, pos, vel);
-  }
-  if (rc == BPIMD_OK) md.steps_taken += (uint64_t)nsteps;
+  rc = run_steps(ctx, p, pos, vel, nsteps, [&](KickStep ks) { return total_force_batched(ctx, p, pos, ks); });
   if (rc == BPIMD_OK && energies) {
     cudaStream_t s = ctx->stream;
     if (launch_spring_expectation_batched(ctx->d_ws, ctx->d_blk_tab, ctx->n_blk_tab, md.spring_part, s) !=

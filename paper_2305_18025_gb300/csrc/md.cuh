@@ -2,6 +2,7 @@
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <functional>
 
 #include "pairs.cuh"
 
@@ -9,7 +10,9 @@ struct bpimd_ctx;
 
 namespace bpimd {
 struct MDState {
-  double *F;                 // [N][P][3] total force of the current positions
+  double *F;                 // [N][P][3] exchange force of the current positions
+  double *Fx;                // [N][P][3] physical force
+  double *zc;                // [N][P][3] thermostat kicks c2 z of the coming step
   double *VB;                // device scalar: V^{[1,N]} of the last evaluation
   double *ubar_part;         // per-block U-bar partial sums of the last force pass
   double *ke_part;           // per-block kinetic-energy partial sums
@@ -22,6 +25,8 @@ struct MDState {
   uint64_t steps_taken;
   void *cell_block;          // cell-list buffers (Lennard-Jones in a box)
   CellList cells;
+  cudaStream_t side;         // the cell-list kernels' stream, forked from and joined to the context's
+  cudaEvent_t fork, join;
   bool ready;
   // replica batches
   double *VBr;               // [R] V_B of every replica
@@ -35,8 +40,13 @@ struct MDState {
 void md_init(MDState *md);
 void md_free(MDState *md);
 int md_run(bpimd_ctx *ctx, double *pos, double *vel, int32_t nsteps, double *energies);
-int evaluate(bpimd_ctx *ctx, const double *pos, double *V_B, double *F);
-int evaluate_batched(bpimd_ctx *ctx, const double *pos, double *V_B, double *F);
+// One evaluation.  `beside`, if given, launches one kernel that needs nothing
+// of the recursions, to run beside them: it is enqueued right after them with
+// the programmatic launch attribute, and must itself end with a wait for them
+// (griddepcontrol.wait in at least one block).
+using Beside = std::function<cudaError_t()>;
+int evaluate(bpimd_ctx *ctx, const double *pos, double *V_B, double *F, const Beside &beside = {});
+int evaluate_batched(bpimd_ctx *ctx, const double *pos, double *V_B, double *F, const Beside &beside = {});
 int md_run_batched(bpimd_ctx *ctx, double *pos, double *vel, int32_t nsteps, double *energies);
 int md_set_pair_tile(bpimd_ctx *ctx, int lanes);
 }  // namespace bpimd

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(CL_THREADS) cl_force(long long nb, int P, Pair
                                                        const int *__restrict__ cellof, const void *__restrict__ sorted,
                                                        const int *__restrict__ start, const int *__restrict__ count,
                                                        const int *__restrict__ list, const double *__restrict__ pos,
-                                                       double *__restrict__ F, double *ubar_part) {
+                                                       double *__restrict__ Fx, double *ubar_part) {
   // one thread per slot of the cell-ordered bead list: neighbouring threads
   // work on the same or adjacent cells, whose coordinates they share in cache
   using R = typename std::conditional<MIXED, float, double>::type;
@@ -199,11 +199,11 @@ __global__ void __launch_bounds__(CL_THREADS) cl_force(long long nb, int P, Pair
   }
   double ul = 0.0;
   if (valid) {
-    double *f = F + 3 * (long long)b;
+    double *f = Fx + 3 * (long long)b;
     const double fs = 24.0 * pp.eps;
-    f[0] += pp.inv_P * (fs * (double)fx - pp.kt * rx);
-    f[1] += pp.inv_P * (fs * (double)fy - pp.kt * ry);
-    f[2] += pp.inv_P * (fs * (double)fz - pp.kt * rz);
+    f[0] = pp.inv_P * (fs * (double)fx - pp.kt * rx);
+    f[1] = pp.inv_P * (fs * (double)fy - pp.kt * ry);
+    f[2] = pp.inv_P * (fs * (double)fz - pp.kt * rz);
     ul = pp.inv_P * (0.5 * (4.0 * pp.eps * (double)u - pp.ushift * nin) + 0.5 * pp.kt * (rx * rx + ry * ry + rz * rz));
   }
 #pragma unroll
@@ -241,7 +241,7 @@ void cell_list_layout(CellList &cl, char *base, int N, int P, int nc, bool mixed
   cl.list = (int *)(base + off);
 }
 
-cudaError_t cell_list_forces(const double *pos, double *F, int N, int P, const PairParams &pp, bool mixed,
+cudaError_t cell_list_forces(const double *pos, double *Fx, int N, int P, const PairParams &pp, bool mixed,
                              const CellList &cl, double *ubar_part, cudaStream_t s) {
   const long long nb = (long long)N * P;
   const long long want = (nb + 255) / 256, cap = (long long)sm_count() * 16;
@@ -259,10 +259,10 @@ cudaError_t cell_list_forces(const double *pos, double *F, int N, int P, const P
   const int blocks = cell_list_partials(N, P);  // one U-bar partial per block
   if (mixed)
     cl_force<true><<<blocks, CL_THREADS, 0, s>>>(nb, P, pp, cl.nc, cl.cellof, cl.sorted, cl.start, cl.count, cl.list,
-                                                 pos, F, ubar_part);
+                                                 pos, Fx, ubar_part);
   else
     cl_force<false><<<blocks, CL_THREADS, 0, s>>>(nb, P, pp, cl.nc, cl.cellof, cl.sorted, cl.start, cl.count, cl.list,
-                                                  pos, F, ubar_part);
+                                                  pos, Fx, ubar_part);
   return cudaGetLastError();
 }
 

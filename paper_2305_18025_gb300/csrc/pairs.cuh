@@ -40,9 +40,9 @@ size_t cell_list_bytes(int N, int P, int nc, bool mixed);
 int cell_list_partials(int N, int P);
 // Lay the buffers out from base (cudaMalloc'd, 256-byte aligned).
 void cell_list_layout(CellList &cl, char *base, int N, int P, int nc, bool mixed);
-// Bin, sort and evaluate Lennard-Jones (+ trap) forces added to F; U-bar
+// Bin, sort and evaluate Lennard-Jones (+ trap) forces into Fx; U-bar
 // partial sums per (particle block of 128, bead index), as the all-pairs kernel.
-cudaError_t cell_list_forces(const double *pos, double *F, int N, int P, const PairParams &pp, bool mixed,
+cudaError_t cell_list_forces(const double *pos, double *Fx, int N, int P, const PairParams &pp, bool mixed,
                              const CellList &cl, double *ubar_part, cudaStream_t s);
 
 }  // namespace bpimd

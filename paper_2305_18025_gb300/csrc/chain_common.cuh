@@ -156,7 +156,7 @@ __device__ __forceinline__ xi xi_fma(xi acc, unsigned long long kk, int ke, xi y
     const unsigned k1 = (unsigned)(kk >> 32);
     p = (unsigned long long)k1 * (unsigned)(y.m >> 32) + (((unsigned long long)k1 * (unsigned)y.m) >> 32);
   } else {
-    p = __umul64hi(kk, y.m);
+    p = pow2fx::mulhi(kk, y.m);
   }
   const int pe = ke + y.e + 1;
   const int E = max(acc.e, pe);
@@ -483,7 +483,7 @@ __device__ __forceinline__ xsum xsum_dot(const unsigned long long *kk, const int
   int E = pe0;
 #pragma unroll
   for (int i = 0; i < K; ++i) {
-    p[i] = __umul64hi(kk[i], y[i].m);
+    p[i] = pow2fx::mulhi(kk[i], y[i].m);
     pe[i] = ke[i] + y[i].e + 1;
     E = max(E, pe[i]);
   }

@@ -97,7 +97,7 @@ __device__ __forceinline__ unsigned long long diff_term(unsigned long long t, do
   sgn = hi >> 31;
   e = ex ? ex - 1023 : NO_TERM;
   bad |= ex == 0x7ff;
-  return __umul64hi(t, ((b << 10) & 0x3FFFFFFFFFFFFFFFull) | (1ull << 62));
+  return pow2fx::mulhi(t, ((b << 10) & 0x3FFFFFFFFFFFFFFFull) | (1ull << 62));
 }
 
 // stores into the cluster's first CTA, and the cluster barrier
@@ -307,7 +307,7 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
         if constexpr (RC) m[k] = pairg::g_of<MODE, PBC>(w, eb, ea, w.cx, T63, e[k]);
         auto d = pairg::diff3(w, eb, ea);
         if constexpr (F64) {
-          const unsigned long long t = valid ? __umul64hi(sm.part.m[i], mant64(m[k])) : 0ull;  // value t 2^(et - 63)
+          const unsigned long long t = valid ? pow2fx::mulhi(sm.part.m[i], mant64(m[k])) : 0ull;  // value t 2^(et - 63)
           const int et = valid ? sm.part.e[i] + e[k] + 1 : NO_TERM;
           int nonfinite = 0;
           p[k][0] = diff_term(t, d.x, pe[k][0], sg[k][0], nonfinite);

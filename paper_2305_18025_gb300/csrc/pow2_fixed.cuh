@@ -31,18 +31,22 @@ namespace pow2fx {
 
 #ifdef __CUDA_ARCH__
 __device__ const unsigned long long T63[256] = {BPIMD_POW2_T63_INIT};
-BPIMD_HD unsigned long long mulhi(unsigned long long a, unsigned long long b) { return __umul64hi(a, b); }
+BPIMD_HD unsigned mulhi32(unsigned a, unsigned b) { return __umulhi(a, b); }
 #else
 static const unsigned long long T63[256] = {BPIMD_POW2_T63_INIT};
-BPIMD_HD unsigned long long mulhi(unsigned long long a, unsigned long long b) {
-  return (unsigned long long)(((unsigned __int128)a * b) >> 64);
-}
+BPIMD_HD unsigned mulhi32(unsigned a, unsigned b) { return (unsigned)(((unsigned long long)a * b) >> 32); }
 #endif
+// High 64 bits of a 64 x 64-bit product without the low words' product: at
+// most 3 units of 2^-64 too small, three multiplications for four.
+BPIMD_HD unsigned long long mulhi(unsigned long long a, unsigned long long b) {
+  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a, bh = (unsigned)(b >> 32), bl = (unsigned)b;
+  return (unsigned long long)ah * bh + mulhi32(ah, bl) + mulhi32(al, bh);
+}
 
 constexpr unsigned long long Q64_HALF = 0x8000000000000000ull;
 constexpr unsigned long long Q64_SIXTH = 0xFFFFFFFFFFFFFFFFull / 6;
-constexpr unsigned long long Q64_24TH = 0xFFFFFFFFFFFFFFFFull / 24;
-constexpr unsigned long long Q64_120TH = 0xFFFFFFFFFFFFFFFFull / 120;
+constexpr unsigned Q32_24TH = 0xFFFFFFFFu / 24;
+constexpr unsigned Q32_120TH = 0xFFFFFFFFu / 120;
 constexpr int ZERO_EXP = -(1 << 28);  // 2^(-2^28): an extended zero for the recursions
 
 struct mexp {
@@ -69,52 +73,83 @@ BPIMD_HD unsigned long long double_to_bits(double d) {
 #endif
 }
 
+// (hi:lo) >> k, low word, k in [0, 31]
+BPIMD_HD unsigned funnel(unsigned lo, unsigned hi, int k) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_r(lo, hi, k);
+#else
+  return (unsigned)((((unsigned long long)hi << 32) | lo) >> k);
+#endif
+}
+
+// 2^(-f) 2^63 of the fraction f = (Fh:Fl) 2^-64.
+BPIMD_HD unsigned long long pow2neg_frac(unsigned Fh, unsigned Fl, const unsigned long long *table) {
+  const unsigned j = Fh >> 24;
+  const unsigned long long r = ((unsigned long long)(Fh & 0x00FFFFFFu) << 32) | Fl;  // f - j/256, times 2^64
+  const unsigned long long u = mulhi(r, BPIMD_LN2_Q64);                              // u 2^64, u = r ln 2
+  // the terms in u^5 and u^4 on 32 bits (u 2^40 < 2^32): they stand below 2^-38
+  const unsigned uh = (unsigned)(u >> 24);
+  const unsigned t4 = Q32_24TH - (mulhi32(uh, Q32_120TH) >> 8);                     // 1/24 - u/120
+  unsigned long long t = Q64_SIXTH - (((unsigned long long)uh * t4) >> 8);          // 1/6 - u t
+  t = Q64_HALF - mulhi(u, t);                                                       // 1/2 - u t
+  const unsigned long long q = u - mulhi(u, mulhi(u, t));                           // u (1 - u t) = 1 - e^(-u)
+  const unsigned long long T = table[j];
+  return T - mulhi(T, q);
+}
+
 // 2^(-x) for x = (H 2^64 + L) 2^S, H in [2^63, 2^64) (a normalised 128-bit
 // mantissa: exact products of two float64 or float32 mantissas fit in it).
 // table: T63 or a shared-memory copy of it.
 BPIMD_HD mexp pow2neg_q(unsigned long long H, unsigned long long L, int S, const unsigned long long *table) {
   if (S >= -99) return mexp{1.0, ZERO_EXP};  // x >= 2^28
-  const int k = -S - 64;                      // x = (H:L) >> (k + 64); k >= 36
-  const unsigned long long n = k < 64 ? (H >> k) : 0ull;
-  unsigned long long F;                       // the 64 fraction bits below the binary point
-  if (k < 64) F = (L >> k) | (H << (64 - k));
-  else F = k < 128 ? (H >> (k - 64)) : 0ull;
-  const unsigned j = (unsigned)(F >> 56);
-  const unsigned long long r = F & 0x00FFFFFFFFFFFFFFull;  // f - j/256, times 2^64
-  const unsigned long long u = mulhi(r, BPIMD_LN2_Q64);      // u 2^64, u = r ln 2
-  unsigned long long t = Q64_24TH - mulhi(u, Q64_120TH);     // 1/24 - u/120
-  t = Q64_SIXTH - mulhi(u, t);                               // 1/6 - u t
-  t = Q64_HALF - mulhi(u, t);                                // 1/2 - u t
-  t = 0ull - mulhi(u, t);                                    // 1 - u t, mod 2^64
-  const unsigned long long q = mulhi(u, t);                  // 1 - e^(-u)
-  const unsigned long long T = table[j];
-  unsigned long long res = T - mulhi(T, q);  // 2^(-f) 2^63, in (2^62, 2^63]
-  if (res >> 63) return mexp{1.0, -(int)n};
-  if (res < (1ull << 62)) res = 1ull << 62;  // truncation cannot take it lower than 2^-1
-  // leading bit at 62: mantissa (res << 1) / 2^63 in (1, 2), exponent -n - 1,
-  // rounded to 53 bits (to nearest, ties up)
-  const unsigned long long v = res << 1;
-  unsigned long long m53 = (v >> 11) + ((v >> 10) & 1ull);
-  int e = -(int)n - 1;
-  if (m53 >> 53) {  // rounded up to the next power of two
-    m53 >>= 1;
-    e += 1;
+  // x = (H:L) >> (k + 64), k >= 36: the integer part n above, the 64 fraction
+  // bits F below that point, by words
+  const int k = -S - 64;
+  const unsigned h1 = (unsigned)(H >> 32), h0 = (unsigned)H, l1 = (unsigned)(L >> 32);
+  unsigned n, Fh, Fl;
+  if (k < 64) {
+    n = h1 >> (k - 32);
+    Fh = funnel(h0, h1, k - 32);
+    Fl = funnel(l1, h0, k - 32);
+  } else {
+    n = 0;
+    Fh = k < 96 ? h1 >> (k - 64) : 0u;
+    Fl = k < 96 ? funnel(h0, h1, k - 64) : (k < 128 ? h1 >> (k - 96) : 0u);
   }
-  return mexp{bits_to_double((m53 & 0x000FFFFFFFFFFFFFull) | 0x3FF0000000000000ull), e};
+  const unsigned long long res = pow2neg_frac(Fh, Fl, table);  // 2^(-f) 2^63, in (2^62 - 8, 2^63]
+  // rounded to 53 bits (to nearest, ties up): in [2^52, 2^53], 2^53 being the
+  // next power of two (which the rounding also reaches from 2^62 - 8 below)
+  const unsigned long long m53 = (res + 512) >> 10;
+  return mexp{bits_to_double((m53 & 0x000FFFFFFFFFFFFFull) | 0x3FF0000000000000ull), (int)(m53 >> 53) - 1 - (int)n};
 }
 
-// Full 128-bit product of two 64-bit mantissas, normalised so that the top
-// bit of the high word is set (both inputs have their top bit set).
-BPIMD_HD void mul128_norm(unsigned long long a, unsigned long long b, unsigned long long &H,
-                          unsigned long long &L, int &shift) {
-  H = mulhi(a, b);
-  L = a * b;
+// (H:L) with its top bit set, shifted left by at most one
+BPIMD_HD void norm128(unsigned long long &H, unsigned long long &L, int &shift) {
   shift = 0;
   if (!(H >> 63)) {
     H = (H << 1) | (L >> 63);
     L <<= 1;
     shift = 1;
   }
+}
+// Full 128-bit product of two 64-bit mantissas, normalised (both inputs have
+// their top bit set).
+BPIMD_HD void mul128_norm(unsigned long long a, unsigned long long b, unsigned long long &H,
+                          unsigned long long &L, int &shift) {
+  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a, bh = (unsigned)(b >> 32), bl = (unsigned)b;
+  const unsigned long long ll = (unsigned long long)al * bl, x = (unsigned long long)ah * bl + (ll >> 32);
+  const unsigned long long y = (unsigned long long)al * bh + (unsigned)x;
+  H = (unsigned long long)ah * bh + (x >> 32) + (y >> 32);
+  L = (y << 32) | (unsigned)ll;
+  norm128(H, L, shift);
+}
+// The same with a = m 2^32, m a 32-bit mantissa with its top bit set.
+BPIMD_HD void mul128_norm(unsigned m, unsigned long long b, unsigned long long &H, unsigned long long &L, int &shift) {
+  const unsigned long long lo = (unsigned long long)m * (unsigned)b, hi = (unsigned long long)m * (unsigned)(b >> 32);
+  const unsigned long long mid = hi + (lo >> 32);  // (m b) >> 32
+  H = mid;
+  L = lo << 32;
+  norm128(H, L, shift);
 }
 
 // 2^(-x) for a double x >= 0 (its bits read by integer instructions).
@@ -140,7 +175,7 @@ BPIMD_HD mexp pow2neg_fd(float a, double c, const unsigned long long *table) {
   if (Ea == 0) return mexp{1.0, 0};
   const unsigned long long cb = double_to_bits(c);
   const int Ec = (int)((cb >> 52) & 0x7FF);
-  const unsigned long long ma = (unsigned long long)((ab & 0x7FFFFFu) | 0x800000u) << 40;  // top bit set
+  const unsigned ma = (ab << 8) | 0x80000000u;  // 24-bit significand, top bit set
   const unsigned long long mc = ((cb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 11;
   unsigned long long H, L;
   int sh;

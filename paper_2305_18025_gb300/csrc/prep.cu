@@ -262,59 +262,58 @@ __device__ __forceinline__ void stage_endpoints(const Workspace &w, const double
   __syncthreads();
 }
 
-// g for one pair from the staged bead-P position of b (slot j of side 0) and
-// bead-1 position of a (slot i of side 1): returns the mantissa (float for
-// MIXED32, else double in [1, 2)) and sets the exponent (pairg.cuh; the
-// recompute mode forms the same bits from the bead pass's copies).
+// A staged endpoint (slot i of side s): the form the pair factor takes.
 template <int MODE, bool PBC>
-__device__ __forceinline__ double pair_factor(const Workspace &w, double cx, const EndTiles &E, int i, int j,
-                                              int &e, const unsigned long long *T63) {
-  using EP = pairg::EndPt<MODE != BPIMD_FP64, PBC>;
-  EP rb, ra;
+__device__ __forceinline__ pairg::EndPt<MODE != BPIMD_FP64, PBC> staged_end(const EndTiles &E, int s, int i) {
+  pairg::EndPt<MODE != BPIMD_FP64, PBC> r;
   if constexpr (MODE == BPIMD_FP64) {
-    rb = EP{E.v[0][j][0], E.v[0][j][1], E.v[0][j][2]};
-    ra = EP{E.v[1][i][0], E.v[1][i][1], E.v[1][i][2]};
+    r.x = E.v[s][i][0];
+    r.y = E.v[s][i][1];
+    r.z = E.v[s][i][2];
   } else if constexpr (PBC) {
-    rb.u = *(const uint4 *)E.v[0][j];
-    ra.u = *(const uint4 *)E.v[1][i];
+    r.u = *(const uint4 *)E.v[s][i];
   } else {
-    rb.h = ((const float4 *)E.v[0][j])[0];
-    rb.l = ((const float4 *)E.v[0][j])[1];
-    ra.h = ((const float4 *)E.v[1][i])[0];
-    ra.l = ((const float4 *)E.v[1][i])[1];
+    r.h = ((const float4 *)E.v[s][i])[0];
+    r.l = ((const float4 *)E.v[s][i])[1];
   }
-  return (double)pairg::g_of<MODE, PBC>(w, rb, ra, cx, T63, e);
+  return r;
 }
 
 // One pass over the forward blocks (a = s*32+i, b = t*32+j): each valid pair
-// a <= b < N is evaluated once and stored in both copies -- the forward one
-// directly (coalesced along b), the backward one (row r = N-1-a, source
+// a <= b < N is evaluated once (pairg.cuh; the recompute mode forms the same
+// bits from the bead pass's copies) and stored in both copies -- the forward
+// one directly (coalesced along b), the backward one (row r = N-1-a, source
 // w = N-1-b) after a transpose through shared memory, so that those stores
 // are coalesced along r.  Entries outside a <= b < N are never written here
-// (gmat_padding_kernel fills them once).
+// (gmat_padding_kernel fills them once).  The pass is bound by issue slots (250
+// instructions a pair before its indices and endpoints were taken out of the
+// loops and the power of two trimmed).
 // One block of g (all threads of the CTA; Tm/Te: 32 x 33 shared tiles).
 template <int MODE, bool PBC>
 __device__ __forceinline__ void gmat_block(const Workspace &w, const double *__restrict__ pos, int blk,
                                            typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type *Tm,
                                            int *Te, EndTiles &E, const unsigned long long *T63) {
   using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
-  const double cx = w.cx;
+  using EP = pairg::EndPt<MODE != BPIMD_FP64, PBC>;
   const int N = w.N;
-  M_t *gm = (M_t *)w.gm, *gbm = (M_t *)w.gbm;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int t, s;
   block_coords(blk, t, s);
   stage_endpoints<MODE != BPIMD_FP64>(w, pos, t, s, E);
   {
-    const int b = t * TILE + lane;
-    for (int i = warp; i < TILE; i += 8) {
-      const int a = s * TILE + i;
-      if (b < N && a <= b) {
+    const int b = t * TILE + lane, last = b < N ? min(b - s * TILE, TILE - 1) : -1;  // valid: i <= last
+    const EP rb = staged_end<MODE, PBC>(E, 0, lane);
+    M_t *gm = (M_t *)w.gm + (size_t)blk * TILE2 + lane;
+    int *ge = w.ge + (size_t)blk * TILE2 + lane;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+      const int i = warp + 8 * k;
+      const EP ra = staged_end<MODE, PBC>(E, 1, i);
+      if (i <= last) {
         int e;
-        const M_t m = (M_t)pair_factor<MODE, PBC>(w, cx, E, i, lane, e, T63);
-        const size_t idx = (size_t)blk * TILE2 + i * TILE + lane;
-        gm[idx] = m;
-        w.ge[idx] = e;
+        const M_t m = pairg::g_of<MODE, PBC>(w, rb, ra, w.cx, T63, e);
+        gm[i * TILE] = m;
+        ge[i * TILE] = e;
         Tm[i * 33 + lane] = m;
         Te[i * 33 + lane] = e;
       }
@@ -322,15 +321,17 @@ __device__ __forceinline__ void gmat_block(const Workspace &w, const double *__r
   }
   __syncthreads();
   {
-    const int a = s * TILE + lane, r = N - 1 - a;
-    for (int jj = warp; jj < TILE; jj += 8) {
-      const int b = t * TILE + jj;
-      if (b < N && a <= b) {
-        const int src = N - 1 - b;
-        const int T = r >> 5, S = src >> 5;
-        const size_t idx = ((size_t)(T * (T + 1) / 2 + S) << 10) + ((src & 31) << 5) + (r & 31);
-        gbm[idx] = Tm[lane * 33 + jj];
-        w.gbe[idx] = Te[lane * 33 + jj];
+    const int a = s * TILE + lane, r = N - 1 - a, T = r >> 5, src0 = N - 1 - t * TILE;
+    const int first = a - t * TILE, end = min(TILE, N - t * TILE);  // valid: first <= jj < end
+    const size_t idx = ((size_t)(T * (T + 1) / 2) << 10) + (r & 31);
+    M_t *gbm = (M_t *)w.gbm + idx;
+    int *gbe = w.gbe + idx;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int jj = warp + 8 * k;
+      if (jj >= first && jj < end) {
+        gbm[(src0 - jj) * TILE] = Tm[lane * 33 + jj];
+        gbe[(src0 - jj) * TILE] = Te[lane * 33 + jj];
       }
     }
   }

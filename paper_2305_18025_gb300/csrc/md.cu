@@ -41,9 +41,12 @@ namespace bpimd {
 namespace {
 
 constexpr int MD_THREADS = 256;
-constexpr int EXT_THREADS = 256;
-constexpr int EXT_SPLIT = 4;  // lanes per particle in the all-pairs force
-constexpr int EXT_PARTICLES = EXT_THREADS / EXT_SPLIT;
+constexpr int EXT_THREADS = 128;
+constexpr int EXT_WARPS = EXT_THREADS / 32;
+// lanes per particle in the all-pairs force (two particles a thread): float64
+// pairs take ~15 times as long, and the smaller blocks spread them evenly
+constexpr int ext_split(bool mixed) { return mixed ? 4 : 8; }
+constexpr int ext_particles(bool mixed) { return 2 * EXT_THREADS / ext_split(mixed); }
 constexpr int EXT_CHUNK = 1024;  // positions of one bead index staged per pass
 
 struct alignas(16) Dbl4 {
@@ -173,19 +176,6 @@ __device__ __forceinline__ double f64_of_f32(float x) {
       (long long)(s | ((unsigned long long)(ex - 127 + 1023) << 52) | ((unsigned long long)(b & 0x7fffffu) << 29)));
 }
 
-// block-wide sum of a float32 per thread: float32 warp sums, float64 across warps
-__device__ __forceinline__ double block_sum_f(float v, double *red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = f64_of_f32(v);
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += red[q];
-  __syncthreads();
-  return s;
-}
-
 __device__ __forceinline__ double block_sum(double v, double *red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -198,55 +188,131 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
   return s;
 }
 
-// -grad U-bar into Fx, per bead index j = blockIdx.y and particle
-// l = blockIdx.x * (256 / SPLIT) + thread / SPLIT (all pairs).  The SPLIT
-// lanes of one particle take the partners q = sub, sub + SPLIT, ...
-// of each staged chunk and combine their sums by a fixed shuffle butterfly;
+// ------------------------------------- float64 Gaussian pairs in fixed point
+// GB300's float64 pipe takes ~75 cycles a warp instruction, and a directed pair
+// needs ten of them beside the integer power of two (720 us a pass at N = 1024,
+// P = 32).  With r' = c r, c^2 = log2(e)/(2 s^2), the Gaussian is 2^(-|d'|^2), so
+// on 64-bit fixed-point r' the whole pair runs on the integer pipe: differences
+// are exact, the three squares sum to the exponent itself (2^-56), and e d' is
+// summed in 96 bits (2^-58 a term; float64 sums round at 2^-53 of their size).
+struct Sum96 {
+  unsigned lo, mid, hi;
+};
+__device__ __forceinline__ void add96(Sum96 &a, long long v) {
+  const unsigned vl = (unsigned)v, vh = (unsigned)((unsigned long long)v >> 32), vs = (unsigned)(v >> 63);
+  asm("add.cc.u32 %0, %0, %3;\n addc.cc.u32 %1, %1, %4;\n addc.u32 %2, %2, %5;"
+      : "+r"(a.lo), "+r"(a.mid), "+r"(a.hi)
+      : "r"(vl), "r"(vh), "r"(vs));
+}
+__device__ __forceinline__ double value96(const Sum96 &a) {
+  const long long top = (long long)(((unsigned long long)a.hi << 32) | a.mid);
+  return fma((double)top, 4294967296.0, (double)a.lo);
+}
+
+// x c 2^S rounded to an integer; c = cm 2^(ce - 63), cm in [2^63, 2^64); the
+// result is below 2^62 (fixed_scale).
+__device__ __forceinline__ long long to_fixed_scaled(double x, unsigned long long cm, int ce, int S) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex == 0) return 0;  // zero or subnormal
+  const unsigned long long H = __umul64hi(((b << 11) | (1ull << 63)), cm);  // |x| c = H 2^(ex - 1023 + ce - 62)
+  const int k = 62 - (ex - 1023) - ce - S;                                   // to shift out, >= 1
+  const unsigned long long v = k > 63 ? 0ull : ((H >> (k - 1)) + 1) >> 1;
+  return (long long)b < 0 ? -(long long)v : (long long)v;
+}
+// Fraction bits S <= 60 at which |r'| stays below 2^(62 - S) (so that no
+// difference overflows), for the largest high word of |r|: 60 up to |r'| = 4.
+__device__ __forceinline__ int fixed_scale(int max_hi, int ce) { return min(60, 62 - ((max_hi >> 20) - 1022 + ce + 1)); }
+constexpr int FIXED_MIN_S = 56;  // |r'| < 64; past it (or with a non-finite coordinate) float64 as before
+
+// One directed pair: adds e d' (2^-58) and e (2^-62), e = 2^(-|d'|^2).
+__device__ __forceinline__ void gauss_fixed(long long X, long long Y, long long Z, long long x, long long y, long long z,
+                                            int sh, const unsigned long long *T63, Sum96 (&f)[3], Sum96 &u) {
+  long long D[3] = {X - x, Y - y, Z - z};
+  int out = 0;  // |d'| >= 8 along an axis: e < 2^-64, taken as 0
+  unsigned long long q = 0;
+  long long w = 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int top = (int)(D[c] >> 32);
+    out |= (top >> (31 - sh)) ^ (top >> 31);
+    D[c] = (long long)((unsigned long long)D[c] << sh);  // d' 2^60
+    const int h = (int)(D[c] >> 32), l = (int)((unsigned)D[c] >> 2);
+    q += (unsigned long long)((long long)h * h);  // (h 2^32 + 4 l)^2 = h^2 2^64 + h l 2^35 + ...
+    w += (long long)h * l;
+  }
+  const unsigned long long x2 = q + (unsigned long long)(w >> 29);  // |d'|^2 2^56
+  const unsigned n = (unsigned)(x2 >> 56);
+  const unsigned long long res = pow2fx::pow2neg_frac((unsigned)(x2 >> 24), (unsigned)(x2 << 8), T63);
+  const unsigned long long e = (out != 0 || n > 62) ? 0ull : res >> (n + 1);  // 2^62 at most
+  const int eh = (int)(e >> 32), el = (int)((unsigned)e >> 1);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int h = (int)(D[c] >> 32);
+    add96(f[c], (long long)eh * h + (long long)__umulhi((unsigned)eh, (unsigned)D[c]) + 2ll * __mulhi(el, h));
+  }
+  add96(u, (long long)e);
+}
+
+// -grad U-bar into Fx, per bead index j = blockIdx.y and block of 256 / SPLIT
+// particles (all pairs).  The SPLIT lanes of a thread group take the partners
+// q = sub, sub + SPLIT, ... of each staged chunk for two particles each (half
+// the block apart), so that one load from shared memory serves two pairs (a
+// 16-byte load a pair kept the shared-memory pipe at 79 % of its rate, 23.6
+// instructions a pair), and combine their sums by a fixed shuffle butterfly;
 // U-bar partial sum per block.  The positions of bead j of all particles pass
 // through shared memory in chunks.  Pairs: Gaussian g exp(-r^2/(2 s^2)), or
 // Lennard-Jones 4 eps ((sig/r)^12 - (sig/r)^6) truncated and shifted at rc; in a
 // periodic box (PBC) pair distances by minimum image.  MIXED: pair terms in
-// float32, accumulated per lane in float32 and added to the float64 force.
+// float32, accumulated per lane in float32.
+__device__ __forceinline__ int max_high(const double *r) {
+  return max(__double2hiint(r[0]) & 0x7fffffff, max(__double2hiint(r[1]) & 0x7fffffff, __double2hiint(r[2]) & 0x7fffffff));
+}
+
 template <bool MIXED, bool PBC, int SPLIT>
 __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos, double *__restrict__ Fx, int N,
                                                  int P, const PairParams &pp, int lb, int j,
                                                  typename std::conditional<MIXED, float4, Dbl4>::type *sr,
-                                                 double *red, unsigned long long *T63s) {
+                                                 double *red, unsigned long long *T63s, int *maxhi) {
   using R = typename std::conditional<MIXED, float, double>::type;
   using R4 = typename std::conditional<MIXED, float4, Dbl4>::type;
-  constexpr int PARTICLES = EXT_THREADS / SPLIT;
+  constexpr int HALF = EXT_THREADS / SPLIT;  // particles of a block: 2 HALF
   const int sub = threadIdx.x % SPLIT;
-  const int l = lb * PARTICLES + threadIdx.x / SPLIT;
-  const bool valid = l < N;
-  double rx = 0, ry = 0, rz = 0;
-  if (valid) {
-    const double *r = pos + ((size_t)l * P + j) * 3;
-    rx = r[0]; ry = r[1]; rz = r[2];
+  int l[2];
+  double rd[2][3];
+  R px[2], py[2], pz[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    l[h] = lb * 2 * HALF + h * HALF + threadIdx.x / SPLIT;
+    const double *r = pos + ((size_t)min(l[h], N - 1) * P + j) * 3;
+    rd[h][0] = r[0]; rd[h][1] = r[1]; rd[h][2] = r[2];
+    // mixed: float32 positions and constants from integer-pipe conversions
+    // and host-formed copies (no float64 work)
+    if constexpr (MIXED) { px[h] = f32_of_f64(r[0]); py[h] = f32_of_f64(r[1]); pz[h] = f32_of_f64(r[2]); }
+    else { px[h] = r[0]; py[h] = r[1]; pz[h] = r[2]; }
   }
-  // mixed: float32 positions and constants from integer-pipe conversions
-  // and host-formed copies, so that no per-thread float64 work remains but the
-  // three force accumulations
-  R px, py, pz, a, L, invL, sig2, rc2;
-  if constexpr (MIXED) {
-    px = f32_of_f64(rx); py = f32_of_f64(ry); pz = f32_of_f64(rz);
-    a = pp.fa; L = pp.fL; invL = pp.finvL; sig2 = pp.fsig2; rc2 = pp.frc2;
-  } else {
-    px = rx; py = ry; pz = rz;
-    a = -0.5 * pp.inv_s2; L = pp.L; invL = pp.invL; sig2 = pp.sig2; rc2 = pp.rc2;
-  }
+  R a, L, invL, sig2, rc2;
+  if constexpr (MIXED) { a = pp.fa; L = pp.fL; invL = pp.finvL; sig2 = pp.fsig2; rc2 = pp.frc2; }
+  else { a = -0.5 * pp.inv_s2; L = pp.L; invL = pp.invL; sig2 = pp.sig2; rc2 = pp.rc2; }
   if (!MIXED) pairg::table_init(T63s);  // float64: the integer-pipe power of two (read after the first barrier)
   auto img = [&](R d) -> R {
     if constexpr (PBC) return d - L * (MIXED ? (R)rintf((float)(d * invL)) : (R)rint((double)(d * invL)));
     else return d;
   };
-  R fx = 0, fy = 0, fz = 0, u = 0;
-  int nin = 0;  // Lennard-Jones pairs inside the cutoff (each carries the shift)
+  constexpr bool FIXED = !MIXED && !PBC;  // Gaussian pairs in fixed point
+  Sum96 sf[2][3] = {}, su[2] = {};
+  R fx[2] = {0, 0}, fy[2] = {0, 0}, fz[2] = {0, 0}, u[2] = {0, 0};
+  int nin[2] = {0, 0};  // Lennard-Jones pairs inside the cutoff (each carries the shift)
   if (pp.pair != BPIMD_PAIR_NONE) {
     for (int base = 0; base < N; base += EXT_CHUNK) {
       const int cnt = min(EXT_CHUNK, N - base);
+      const bool fixed = FIXED && pp.pair == BPIMD_PAIR_GAUSSIAN;
+      int top = 0;  // largest high word of |r| of the chunk and of the block's particles
       __syncthreads();
+      if (fixed && threadIdx.x == 0) *maxhi = 0;
       for (int q = threadIdx.x; q < cnt; q += EXT_THREADS) {
         const double *r = pos + ((size_t)(base + q) * P + j) * 3;
+        if (fixed) top = max(top, max_high(r));
         R4 t;
         if constexpr (MIXED) { t.x = f32_of_f64(r[0]); t.y = f32_of_f64(r[1]); t.z = f32_of_f64(r[2]); }
         else { t.x = r[0]; t.y = r[1]; t.z = r[2]; }
@@ -254,69 +320,130 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
         sr[q] = t;
       }
       __syncthreads();
-      if (valid && pp.pair == BPIMD_PAIR_GAUSSIAN) {
-#pragma unroll 4
-        for (int q = sub; q < cnt; q += SPLIT) {
-          const R4 t = sr[q];
-          const R dx = img(px - t.x), dy = img(py - t.y), dz = img(pz - t.z);
-          const R d2 = dx * dx + dy * dy + dz * dz;
-          R e;
-          if constexpr (MIXED) e = __expf(a * d2);
-          else e = pow2_value(pow2fx::pow2neg_dd((double)d2, pp.g2c, T63s));  // exactly 1 at d = 0
-          fx += e * dx; fy += e * dy; fz += e * dz;
-          u += e;
+      if constexpr (FIXED) {
+        if (fixed) {
+          top = __reduce_max_sync(0xffffffffu, max(top, max(max_high(rd[0]), max_high(rd[1]))));
+          if ((threadIdx.x & 31) == 0) atomicMax(maxhi, top);
+          __syncthreads();
+          const int S = fixed_scale(*maxhi, pp.ce);
+          if (S >= FIXED_MIN_S) {
+            for (int q = threadIdx.x; q < cnt; q += EXT_THREADS) {  // each thread its own entries
+              R4 &t = sr[q];
+              t.x = __longlong_as_double(to_fixed_scaled(t.x, pp.cm, pp.ce, S));
+              t.y = __longlong_as_double(to_fixed_scaled(t.y, pp.cm, pp.ce, S));
+              t.z = __longlong_as_double(to_fixed_scaled(t.z, pp.cm, pp.ce, S));
+            }
+            long long X[2][3];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+              for (int c = 0; c < 3; ++c) X[h][c] = to_fixed_scaled(rd[h][c], pp.cm, pp.ce, S);
+            __syncthreads();
+            for (int q = sub; q < cnt; q += SPLIT) {
+              const R4 t = sr[q];
+              const long long x = __double_as_longlong(t.x), y = __double_as_longlong(t.y), z = __double_as_longlong(t.z);
+#pragma unroll
+              for (int h = 0; h < 2; ++h) gauss_fixed(X[h][0], X[h][1], X[h][2], x, y, z, 60 - S, T63s, sf[h], su[h]);
+            }
+            continue;
+          }
         }
-      } else if (valid) {  // Lennard-Jones: force over 24 eps, energy over 4 eps
+      }
+      if (pp.pair == BPIMD_PAIR_GAUSSIAN) {
 #pragma unroll 4
         for (int q = sub; q < cnt; q += SPLIT) {
           const R4 t = sr[q];
-          const R dx = img(px - t.x), dy = img(py - t.y), dz = img(pz - t.z);
-          const R r2 = dx * dx + dy * dy + dz * dz;
-          if (r2 > (R)0 && r2 < rc2) {
-            const R s2 = sig2 / r2, s6 = s2 * s2 * s2;
-            const R c = (2 * s6 * s6 - s6) / r2;
-            fx += c * dx; fy += c * dy; fz += c * dz;
-            u += s6 * s6 - s6;
-            ++nin;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const R dx = img(px[h] - t.x), dy = img(py[h] - t.y), dz = img(pz[h] - t.z);
+            const R d2 = dx * dx + dy * dy + dz * dz;
+            R e;
+            if constexpr (MIXED) e = __expf(a * d2);
+            else e = pow2_value(pow2fx::pow2neg_dd((double)d2, pp.g2c, T63s));  // exactly 1 at d = 0
+            fx[h] += e * dx; fy[h] += e * dy; fz[h] += e * dz;
+            u[h] += e;
+          }
+        }
+      } else {  // Lennard-Jones: force over 24 eps, energy over 4 eps
+#pragma unroll 2
+        for (int q = sub; q < cnt; q += SPLIT) {
+          const R4 t = sr[q];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const R dx = img(px[h] - t.x), dy = img(py[h] - t.y), dz = img(pz[h] - t.z);
+            const R r2 = dx * dx + dy * dy + dz * dz;
+            if (r2 > (R)0 && r2 < rc2) {
+              const R s2 = sig2 / r2, s6 = s2 * s2 * s2;
+              const R c = (2 * s6 * s6 - s6) / r2;
+              fx[h] += c * dx; fy[h] += c * dy; fz[h] += c * dz;
+              u[h] += s6 * s6 - s6;
+              ++nin[h];
+            }
           }
         }
       }
     }
   }
+  double ub[2];
 #pragma unroll
-  for (int o = 1; o < SPLIT; o <<= 1) {
-    fx += __shfl_xor_sync(0xffffffffu, fx, o);
-    fy += __shfl_xor_sync(0xffffffffu, fy, o);
-    fz += __shfl_xor_sync(0xffffffffu, fz, o);
-    u += __shfl_xor_sync(0xffffffffu, u, o);
-    nin += __shfl_xor_sync(0xffffffffu, nin, o);
-  }
-  if constexpr (MIXED) {
-    float ulf = 0.0f;
-    if (valid && sub == 0) {
-      if (pp.pair == BPIMD_PAIR_GAUSSIAN) u -= 1.0f;  // the self term (d = 0, e = 1) carries no force
-      double *f = Fx + ((size_t)l * P + j) * 3;
-      f[0] = f64_of_f32(pp.finv_P * (pp.ffs * fx - pp.fkt * px));
-      f[1] = f64_of_f32(pp.finv_P * (pp.ffs * fy - pp.fkt * py));
-      f[2] = f64_of_f32(pp.finv_P * (pp.ffs * fz - pp.fkt * pz));
-      const float up = pp.pair == BPIMD_PAIR_GAUSSIAN ? pp.fup * u : pp.fup * u - pp.fush * (float)nin;
-      ulf = pp.finv_P * (up + 0.5f * pp.fkt * (px * px + py * py + pz * pz));
+  for (int h = 0; h < 2; ++h) {
+    if constexpr (FIXED) {
+      fx[h] = fma(value96(sf[h][0]), pp.ic, fx[h]);
+      fy[h] = fma(value96(sf[h][1]), pp.ic, fy[h]);
+      fz[h] = fma(value96(sf[h][2]), pp.ic, fz[h]);
+      u[h] = fma(value96(su[h]), 2.168404344971009e-19, u[h]);  // 2^-62
     }
-    return block_sum_f(ulf, red);
+#pragma unroll
+    for (int o = 1; o < SPLIT; o <<= 1) {
+      fx[h] += __shfl_xor_sync(0xffffffffu, fx[h], o);
+      fy[h] += __shfl_xor_sync(0xffffffffu, fy[h], o);
+      fz[h] += __shfl_xor_sync(0xffffffffu, fz[h], o);
+      u[h] += __shfl_xor_sync(0xffffffffu, u[h], o);
+      nin[h] += __shfl_xor_sync(0xffffffffu, nin[h], o);
+    }
+    const bool mine = l[h] < N && sub == 0;
+    double *f = Fx + ((size_t)l[h] * P + j) * 3;
+    if constexpr (MIXED) {
+      float ulf = 0.0f;
+      if (mine) {
+        if (pp.pair == BPIMD_PAIR_GAUSSIAN) u[h] -= 1.0f;  // the self term (d = 0, e = 1) carries no force
+        f[0] = f64_of_f32(pp.finv_P * (pp.ffs * fx[h] - pp.fkt * px[h]));
+        f[1] = f64_of_f32(pp.finv_P * (pp.ffs * fy[h] - pp.fkt * py[h]));
+        f[2] = f64_of_f32(pp.finv_P * (pp.ffs * fz[h] - pp.fkt * pz[h]));
+        const float up = pp.pair == BPIMD_PAIR_GAUSSIAN ? pp.fup * u[h] : pp.fup * u[h] - pp.fush * (float)nin[h];
+        ulf = pp.finv_P * (up + 0.5f * pp.fkt * (px[h] * px[h] + py[h] * py[h] + pz[h] * pz[h]));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) ulf += __shfl_xor_sync(0xffffffffu, ulf, o);
+      ub[h] = f64_of_f32(ulf);
+    } else {
+      double ul = 0.0;
+      if (mine) {
+        if (pp.pair == BPIMD_PAIR_GAUSSIAN) u[h] -= (R)1;  // the self term (d = 0, e = 1) carries no force
+        const double fs = pp.pair == BPIMD_PAIR_GAUSSIAN ? pp.ga * pp.inv_s2 : 24.0 * pp.eps;
+        f[0] = pp.inv_P * (fs * (double)fx[h] - pp.kt * rd[h][0]);
+        f[1] = pp.inv_P * (fs * (double)fy[h] - pp.kt * rd[h][1]);
+        f[2] = pp.inv_P * (fs * (double)fz[h] - pp.kt * rd[h][2]);
+        const double up = pp.pair == BPIMD_PAIR_GAUSSIAN ? 0.5 * pp.ga * (double)u[h]
+                                                        : 0.5 * (4.0 * pp.eps * (double)u[h] - pp.ushift * nin[h]);
+        ul = pp.inv_P * (up + 0.5 * pp.kt * (rd[h][0] * rd[h][0] + rd[h][1] * rd[h][1] + rd[h][2] * rd[h][2]));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) ul += __shfl_xor_sync(0xffffffffu, ul, o);
+      ub[h] = ul;
+    }
   }
-  double ul = 0.0;
-  if (valid && sub == 0) {
-    if (pp.pair == BPIMD_PAIR_GAUSSIAN) u -= (R)1;  // the self term (d = 0, e = 1) carries no force
-    double *f = Fx + ((size_t)l * P + j) * 3;
-    const double fs = pp.pair == BPIMD_PAIR_GAUSSIAN ? pp.ga * pp.inv_s2 : 24.0 * pp.eps;
-    f[0] = pp.inv_P * (fs * (double)fx - pp.kt * rx);
-    f[1] = pp.inv_P * (fs * (double)fy - pp.kt * ry);
-    f[2] = pp.inv_P * (fs * (double)fz - pp.kt * rz);
-    const double up = pp.pair == BPIMD_PAIR_GAUSSIAN ? 0.5 * pp.ga * (double)u
-                                                    : 0.5 * (4.0 * pp.eps * (double)u - pp.ushift * nin);
-    ul = pp.inv_P * (up + 0.5 * pp.kt * (rx * rx + ry * ry + rz * rz));
+  // the warps' sums in a fixed order: first halves, then second halves
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5] = ub[0];
+    red[EXT_WARPS + (threadIdx.x >> 5)] = ub[1];
   }
-  return block_sum(ul, red);
+  __syncthreads();
+  double sum = 0.0;
+  if (threadIdx.x == 0)
+    for (int q = 0; q < 2 * EXT_WARPS; ++q) sum += red[q];
+  __syncthreads();
+  return sum;
 }
 
 // Thermostat kicks of one step, n elements (see md_run): element's amplitude
@@ -352,10 +479,11 @@ __global__ void __launch_bounds__(EXT_THREADS) ext_force_kernel(const double *__
                                                                 double *ubar_part, Kicks kicks) {
   using R4 = typename std::conditional<MIXED, float4, Dbl4>::type;
   __shared__ R4 sr[EXT_CHUNK];
-  __shared__ double red[EXT_THREADS / 32];
+  __shared__ double red[2 * EXT_WARPS];
   __shared__ unsigned long long T63s[256];  // float64: the table of the integer-pipe power of two
+  __shared__ int maxhi;
   if ((int)blockIdx.y < P) {
-    const double s = ext_force_body<MIXED, PBC, EXT_SPLIT>(pos, Fx, N, P, pp, blockIdx.x, blockIdx.y, sr, red, T63s);
+    const double s = ext_force_body<MIXED, PBC, ext_split(MIXED)>(pos, Fx, N, P, pp, blockIdx.x, blockIdx.y, sr, red, T63s, &maxhi);
     if (threadIdx.x == 0) ubar_part[blockIdx.y * gridDim.x + blockIdx.x] = s;
   } else {
     kicks_block<MIXED>(kicks, (blockIdx.y - P) * (long long)gridDim.x + blockIdx.x,
@@ -425,8 +553,9 @@ __global__ void __launch_bounds__(EXT_THREADS) ext_force_batched(const double *_
                                                                  double *ubar_part, Kicks kicks, int kick_blocks) {
   using R4 = typename std::conditional<MIXED, float4, Dbl4>::type;
   __shared__ R4 sr[EXT_CHUNK];
-  __shared__ double red[EXT_THREADS / 32];
+  __shared__ double red[2 * EXT_WARPS];
   __shared__ unsigned long long T63s[256];
+  __shared__ int maxhi;
   if ((int)blockIdx.x < kick_blocks) {
     kicks_block<MIXED>(kicks, blockIdx.x, kick_blocks);
     after_recursions(blockIdx.x == 0);
@@ -439,7 +568,7 @@ __global__ void __launch_bounds__(EXT_THREADS) ext_force_batched(const double *_
     PairParams q = pp;
     q.inv_P = ws[e.x].inv_P;
     q.finv_P = f32_of_f64(q.inv_P);
-    const double s = ext_force_body<MIXED, false, SPLIT>(pos + off[e.x], Fx + off[e.x], N, P, q, e.y, e.z, sr, red, T63s);
+    const double s = ext_force_body<MIXED, false, SPLIT>(pos + off[e.x], Fx + off[e.x], N, P, q, e.y, e.z, sr, red, T63s, &maxhi);
     if (threadIdx.x == 0) ubar_part[k] = s;
     __syncthreads();  // sr is reused by the next entry
   }
@@ -558,6 +687,14 @@ int md_params(const bpimd_config &c, MDParams &p) {
     q.ga = c.pair_a;
     q.inv_s2 = 1.0 / (c.pair_b * c.pair_b);
     q.g2c = 0.5 * q.inv_s2 * 1.4426950408889634;  // log2(e) / (2 s^2)
+    // c = sqrt(g2c) to 64 bits: its float64 root and the residual's correction
+    const double root = std::sqrt(q.g2c), corr = std::fma(-root, root, q.g2c) / (2.0 * root);
+    int ex;
+    const double m = std::frexp(root, &ex);  // root = m 2^ex, m in [0.5, 1)
+    q.ce = ex - 1;
+    q.cm = (uint64_t)std::ldexp(m, 64) + (uint64_t)(int64_t)std::llround(std::ldexp(corr, 64 - ex));
+    if (!(q.cm >> 63)) q.cm = 1ull << 63;  // the correction took it below the power of two
+    q.ic = std::ldexp(1.0 / root, -58);
   }
   if (c.pair_type == BPIMD_PAIR_LJ) {
     q.eps = c.pair_a;
@@ -635,7 +772,7 @@ int total_force(bpimd_ctx *ctx, const MDParams &p, const double *pos, KickStep k
     if (cudaStreamWaitEvent(s, md.join, 0) != cudaSuccess) return BPIMD_ERR_CUDA;
     return rc != BPIMD_OK ? rc : re;
   }
-  const int N = ctx->cfg.N, P = ctx->cfg.P, gx = (N + EXT_PARTICLES - 1) / EXT_PARTICLES;
+  const int N = ctx->cfg.N, P = ctx->cfg.P, pb = ext_particles(ctx->w.bead32), gx = (N + pb - 1) / pb;
   const dim3 grid(gx, P + (kick_blocks + gx - 1) / gx);
   return evaluate(ctx, pos, md.VB, md.F, [&] {
     auto go = [&](auto kernel) {
@@ -715,7 +852,7 @@ int md_alloc(bpimd_ctx *ctx, const MDParams &p) {
   }
   const size_t n = (size_t)ctx->cfg.N * ctx->cfg.P * 3;
   md.ext_blocks = p.cell_nc > 0 ? cell_list_partials(ctx->cfg.N, ctx->cfg.P)
-                                 : ((ctx->cfg.N + EXT_PARTICLES - 1) / EXT_PARTICLES) * ctx->cfg.P;
+                                 : ((ctx->cfg.N + ext_particles(ctx->w.bead32) - 1) / ext_particles(ctx->w.bead32)) * ctx->cfg.P;
   md.ke_blocks = grid_for((long long)n, MD_THREADS);
   md.spring_blocks = ctx->w.NB;
   if (cudaMalloc(&md.F, sizeof(double) * n) != cudaSuccess || cudaMalloc(&md.Fx, sizeof(double) * n) != cudaSuccess ||
@@ -798,7 +935,7 @@ namespace {
 // (replica, particle block, bead index) table of the batched pair forces for
 // `lanes` lanes per particle (256 / lanes particles per block)
 void pair_table(const bpimd_ctx *ctx, int lanes, std::vector<int4> &tab, std::vector<int> &ext_first) {
-  const int R = ctx->R, pb = EXT_THREADS / lanes;
+  const int R = ctx->R, pb = 2 * EXT_THREADS / lanes;
   tab.clear();
   ext_first.assign(R + 1, 0);
   for (int r = 0; r < R; ++r) {
@@ -867,7 +1004,7 @@ int total_force_batched(bpimd_ctx *ctx, const MDParams &p, const double *pos, Ki
   kicks.off = ctx->d_off;
   kicks.R = ctx->R;
   const int kick_blocks = kicks.zc ? grid_for((p.n + 3) / 4, EXT_THREADS) : 0;
-  const int grid = kick_blocks + (md.n_ext < sm_count() * 8 ? md.n_ext : sm_count() * 8);
+  const int grid = kick_blocks + (md.n_ext < sm_count() * 12 ? md.n_ext : sm_count() * 12);
   return evaluate_batched(ctx, pos, md.VBr, md.F, [&] {
     auto go = [&](auto kernel) {
       return launch_pdl(kernel, grid, EXT_THREADS, 0, ctx->stream, pos, md.Fx, ctx->d_ws, ctx->d_off, md.ext_tab,

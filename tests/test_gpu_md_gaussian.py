@@ -1,5 +1,7 @@
 """Gaussian pair forces of the MD step at the edges of their blocks, chunks and
-number formats, against the MD oracle (one noiseless step).
+number formats, against the MD oracle (one noiseless step; from N = 128 its
+long-double build, as for every parity test of that size: with centres over
++-60 the float64 build's shifted log-sum-exp is 1.3e-11 off in a velocity).
 
 Float64 pairs run in 64-bit fixed point while |r| sqrt(log2(e) / (2 s^2)) stays
 below 64, past that (scale 60 below) in float64; with a wider spread the
@@ -27,8 +29,9 @@ def test_one_step_matches_the_oracle(N, scale):
     rng = np.random.default_rng(N)
     pos = rng.uniform(-scale, scale, (N, 1, 3)) + rng.normal(0.0, 0.1, (N, P, 3))
     vel = rng.normal(0.0, 1.0, (N, P, 3))
-    ox, ov, oe = oracle.float64.md_run(pos.copy(), vel.copy(), 1.0, wP, beta, dt, 0.0, 1, omega0=1.0, pair_type=1,
-                                       pair_a=g, pair_b=s)
+    ref = oracle.long_double if N >= 128 else oracle.float64
+    ox, ov, oe = ref.md_run(pos.copy(), vel.copy(), 1.0, wP, beta, dt, 0.0, 1, omega0=1.0, pair_type=1, pair_a=g,
+                            pair_b=s)
     for prec, tol in (("fp64", 1e-12), ("mixed", 1e-5)):
         md = RingPolymerMD(N, P, 1.0, wP, beta, dt=dt, gamma=0.0, omega0=1.0, gaussian=(g, s), precision=prec)
         x, v = torch.from_numpy(pos.copy()).cuda(), torch.from_numpy(vel.copy()).cuda()

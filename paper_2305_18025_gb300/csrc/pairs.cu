@@ -4,9 +4,9 @@
 // Per bead index j the box is cut into nc^3 cells of side L/nc >= rc, so all
 // partners within rc of a bead lie in its own and the 26 neighbouring cells
 // (nc >= 3 keeps those 27 cells distinct).  Per step:
-//   bin     each bead's cell and its wrapped coordinates (MIXED: 32-bit
-//           fixed-point fractions of L, whose wrap-around difference is the
-//           minimum image exactly; float64: coordinates in [0, L));
+//   bin     each bead's cell and its wrapped coordinates (32-bit fixed-point
+//           fractions of L, whose wrap-around difference is the minimum image
+//           exactly; float64 also: coordinates in [0, L));
 //   scan    cell starts (exclusive prefix sum of the counts, one CTA);
 //   scatter bead indices into their cells;
 //   sort    each cell's indices ascending, so that every force is summed in
@@ -30,7 +30,7 @@ size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 template <bool MIXED>
 __global__ void __launch_bounds__(256) cl_bin(const double *__restrict__ pos, int N, int P, int nc, double invL,
-                                              int *__restrict__ cellof, void *__restrict__ crd,
+                                              int *__restrict__ cellof, uint4 *__restrict__ fix, void *__restrict__ crd,
                                               int *__restrict__ count) {
   const long long nb = (long long)N * P;
   for (long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x; b < nb; b += (long long)gridDim.x * blockDim.x) {
@@ -46,14 +46,15 @@ __global__ void __launch_bounds__(256) cl_bin(const double *__restrict__ pos, in
     }
     const int cid = ((j * nc + c[2]) * nc + c[1]) * nc + c[0];
     cellof[b] = cid;
-    if (MIXED) {
+    {
       uint4 u;
       u.x = (unsigned)fmin(f[0] * 4294967296.0, 4294967295.0);
       u.y = (unsigned)fmin(f[1] * 4294967296.0, 4294967295.0);
       u.z = (unsigned)fmin(f[2] * 4294967296.0, 4294967295.0);
       u.w = 0u;
-      ((uint4 *)crd)[b] = u;
-    } else {
+      fix[b] = u;
+    }
+    if (!MIXED) {
       const double L = 1.0 / invL;
       ((double4 *)crd)[b] = make_double4(f[0] * L, f[1] * L, f[2] * L, 0.0);
     }
@@ -130,23 +131,34 @@ __global__ void __launch_bounds__(256) cl_sort(const int *__restrict__ start, co
 // coordinates in cell order: sorted[slot] = crd[list[slot]]
 template <bool MIXED>
 __global__ void __launch_bounds__(256) cl_gather(const int *__restrict__ list, long long nb,
+                                                 const uint4 *__restrict__ fix, uint4 *__restrict__ sfix,
                                                  const void *__restrict__ crd, void *__restrict__ sorted) {
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nb; q += (long long)gridDim.x * blockDim.x) {
-    if (MIXED) ((uint4 *)sorted)[q] = ((const uint4 *)crd)[list[q]];
-    else ((double4 *)sorted)[q] = ((const double4 *)crd)[list[q]];
+    sfix[q] = fix[list[q]];
+    if (!MIXED) ((double4 *)sorted)[q] = ((const double4 *)crd)[list[q]];
   }
 }
 
+// One thread per slot of the cell-ordered bead list: neighbouring threads work
+// on the same or adjacent cells, whose coordinates they share in cache.  Of the
+// ~9 candidates for each partner inside rc, a float32 test of the fixed-point
+// coordinates keeps the near ones in a list of the thread's own (in shared
+// memory, in order), which is worked off when it is full and at the end: with
+// the pair's arithmetic behind a branch in the candidate loop, some lane took it
+// for nearly every candidate (136 us a pass at N = 4000, P = 64 mixed; float64
+// spent ~30 instructions of its ~75-cycle pipe on each candidate).
+constexpr int CL_LIST = 32;  // near candidates held a thread
+
 template <bool MIXED>
 __global__ void __launch_bounds__(CL_THREADS) cl_force(long long nb, int P, PairParams pp, int nc,
-                                                       const int *__restrict__ cellof, const void *__restrict__ sorted,
+                                                       const int *__restrict__ cellof, const uint4 *__restrict__ sfix,
+                                                       const void *__restrict__ sorted,
                                                        const int *__restrict__ start, const int *__restrict__ count,
                                                        const int *__restrict__ list, const double *__restrict__ pos,
                                                        double *__restrict__ Fx, double *ubar_part) {
-  // one thread per slot of the cell-ordered bead list: neighbouring threads
-  // work on the same or adjacent cells, whose coordinates they share in cache
   using R = typename std::conditional<MIXED, float, double>::type;
   __shared__ double red[CL_THREADS / 32];
+  __shared__ int near[CL_LIST][CL_THREADS];
   const long long slot = blockIdx.x * (long long)CL_THREADS + threadIdx.x;
   const bool valid = slot < nb;
   R fx = 0, fy = 0, fz = 0, u = 0;
@@ -161,10 +173,38 @@ __global__ void __launch_bounds__(CL_THREADS) cl_force(long long nb, int P, Pair
     const int cell = cellof[b] - j * nc * nc * nc;
     const int cx = cell % nc, cy = (cell / nc) % nc, cz = cell / (nc * nc);
     const R sig2 = (R)pp.sig2, rc2 = (R)pp.rc2;
-    uint4 ui = make_uint4(0, 0, 0, 0);
+    const float rc2f = (float)pp.rc2, keep2 = MIXED ? rc2f : rc2f * 1.00001f;  // float64: the test's own rounding aside
+    const uint4 ui = sfix[slot];
     double4 di = make_double4(0, 0, 0, 0);
-    if (MIXED) ui = ((const uint4 *)sorted)[slot];
-    else di = ((const double4 *)sorted)[slot];
+    if (!MIXED) di = ((const double4 *)sorted)[slot];
+    int held = 0;
+    auto work_off = [&] {
+      for (int k = 0; k < held; ++k) {
+        const int q = near[k][threadIdx.x];
+        R ex, ey, ez;
+        if (MIXED) {
+          const uint4 uj = sfix[q];
+          ex = (R)fixdiff(ui.x, uj.x, pp.Lscale);
+          ey = (R)fixdiff(ui.y, uj.y, pp.Lscale);
+          ez = (R)fixdiff(ui.z, uj.z, pp.Lscale);
+        } else {
+          const double4 dj = ((const double4 *)sorted)[q];
+          ex = (R)(di.x - dj.x); ey = (R)(di.y - dj.y); ez = (R)(di.z - dj.z);
+          ex -= (R)(pp.L * rint((double)ex * pp.invL));
+          ey -= (R)(pp.L * rint((double)ey * pp.invL));
+          ez -= (R)(pp.L * rint((double)ez * pp.invL));
+        }
+        const R r2 = ex * ex + ey * ey + ez * ez;
+        if (MIXED || (r2 > (R)0 && r2 < rc2)) {
+          const R s2 = sig2 / r2, s6 = s2 * s2 * s2;
+          const R c = (2 * s6 * s6 - s6) / r2;
+          fx += c * ex; fy += c * ey; fz += c * ez;
+          u += s6 * s6 - s6;
+          ++nin;
+        }
+      }
+      held = 0;
+    };
     for (int dz = -1; dz <= 1; ++dz)
       for (int dy = -1; dy <= 1; ++dy)
         for (int dx = -1; dx <= 1; ++dx) {
@@ -172,30 +212,17 @@ __global__ void __launch_bounds__(CL_THREADS) cl_force(long long nb, int P, Pair
           const int nid = ((j * nc + nz) * nc + ny) * nc + nx;
           const int s0 = start[nid], n = count[nid];
           for (int q = s0; q < s0 + n; ++q) {
-            if (q == slot) continue;
-            R ex, ey, ez;
-            if (MIXED) {
-              const uint4 uj = ((const uint4 *)sorted)[q];
-              ex = (R)fixdiff(ui.x, uj.x, pp.Lscale);
-              ey = (R)fixdiff(ui.y, uj.y, pp.Lscale);
-              ez = (R)fixdiff(ui.z, uj.z, pp.Lscale);
-            } else {
-              const double4 dj = ((const double4 *)sorted)[q];
-              ex = (R)(di.x - dj.x); ey = (R)(di.y - dj.y); ez = (R)(di.z - dj.z);
-              ex -= (R)(pp.L * rint((double)ex * pp.invL));
-              ey -= (R)(pp.L * rint((double)ey * pp.invL));
-              ez -= (R)(pp.L * rint((double)ez * pp.invL));
-            }
-            const R r2 = ex * ex + ey * ey + ez * ez;
-            if (r2 > (R)0 && r2 < rc2) {
-              const R s2 = sig2 / r2, s6 = s2 * s2 * s2;
-              const R c = (2 * s6 * s6 - s6) / r2;
-              fx += c * ex; fy += c * ey; fz += c * ez;
-              u += s6 * s6 - s6;
-              ++nin;
+            const uint4 uj = sfix[q];
+            const float ex = fixdiff(ui.x, uj.x, pp.Lscale), ey = fixdiff(ui.y, uj.y, pp.Lscale),
+                        ez = fixdiff(ui.z, uj.z, pp.Lscale);
+            const float r2 = ex * ex + ey * ey + ez * ez;
+            if (q != slot && (MIXED ? r2 > 0.0f && r2 < keep2 : r2 < keep2)) {
+              near[held++][threadIdx.x] = q;
+              if (held == CL_LIST) work_off();
             }
           }
         }
+    work_off();
   }
   double ul = 0.0;
   if (valid) {
@@ -223,7 +250,7 @@ int cell_list_partials(int N, int P) { return ((N + CL_THREADS - 1) / CL_THREADS
 
 size_t cell_list_bytes(int N, int P, int nc, bool mixed) {
   const size_t nb = (size_t)N * P, ncells = (size_t)P * nc * nc * nc;
-  return a256(sizeof(int) * nb) + 2 * a256((mixed ? 16 : 32) * nb) + 3 * a256(sizeof(int) * ncells) +
+  return a256(sizeof(int) * nb) + 2 * a256(16 * nb) + (mixed ? 0 : 2 * a256(32 * nb)) + 3 * a256(sizeof(int) * ncells) +
          a256(sizeof(int) * nb);
 }
 
@@ -233,8 +260,12 @@ void cell_list_layout(CellList &cl, char *base, int N, int P, int nc, bool mixed
   cl.ncells = (int)ncells;
   size_t off = 0;
   cl.cellof = (int *)(base + off); off += a256(sizeof(int) * nb);
-  cl.crd = (void *)(base + off); off += a256((mixed ? 16 : 32) * nb);
-  cl.sorted = (void *)(base + off); off += a256((mixed ? 16 : 32) * nb);
+  cl.fix = (uint4 *)(base + off); off += a256(16 * nb);
+  cl.sfix = (uint4 *)(base + off); off += a256(16 * nb);
+  if (!mixed) {
+    cl.crd = (void *)(base + off); off += a256(32 * nb);
+    cl.sorted = (void *)(base + off); off += a256(32 * nb);
+  }
   cl.count = (int *)(base + off); off += a256(sizeof(int) * ncells);
   cl.fill = (int *)(base + off); off += a256(sizeof(int) * ncells);
   cl.start = (int *)(base + off); off += a256(sizeof(int) * ncells);
@@ -249,19 +280,19 @@ cudaError_t cell_list_forces(const double *pos, double *Fx, int N, int P, const 
   cudaError_t e = cudaMemsetAsync(cl.count, 0, sizeof(int) * cl.ncells, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(cl.fill, 0, sizeof(int) * cl.ncells, s);
   if (e != cudaSuccess) return e;
-  if (mixed) cl_bin<true><<<g, 256, 0, s>>>(pos, N, P, cl.nc, pp.invL, cl.cellof, cl.crd, cl.count);
-  else cl_bin<false><<<g, 256, 0, s>>>(pos, N, P, cl.nc, pp.invL, cl.cellof, cl.crd, cl.count);
+  if (mixed) cl_bin<true><<<g, 256, 0, s>>>(pos, N, P, cl.nc, pp.invL, cl.cellof, cl.fix, cl.crd, cl.count);
+  else cl_bin<false><<<g, 256, 0, s>>>(pos, N, P, cl.nc, pp.invL, cl.cellof, cl.fix, cl.crd, cl.count);
   cl_scan<<<1, SCAN_THREADS, 0, s>>>(cl.count, cl.start, cl.ncells);
   cl_scatter<<<g, 256, 0, s>>>(cl.cellof, N, P, cl.start, cl.fill, cl.list);
   cl_sort<<<(cl.ncells + 255) / 256, 256, 0, s>>>(cl.start, cl.count, cl.ncells, cl.list);
-  if (mixed) cl_gather<true><<<g, 256, 0, s>>>(cl.list, nb, cl.crd, cl.sorted);
-  else cl_gather<false><<<g, 256, 0, s>>>(cl.list, nb, cl.crd, cl.sorted);
+  if (mixed) cl_gather<true><<<g, 256, 0, s>>>(cl.list, nb, cl.fix, cl.sfix, cl.crd, cl.sorted);
+  else cl_gather<false><<<g, 256, 0, s>>>(cl.list, nb, cl.fix, cl.sfix, cl.crd, cl.sorted);
   const int blocks = cell_list_partials(N, P);  // one U-bar partial per block
   if (mixed)
-    cl_force<true><<<blocks, CL_THREADS, 0, s>>>(nb, P, pp, cl.nc, cl.cellof, cl.sorted, cl.start, cl.count, cl.list,
+    cl_force<true><<<blocks, CL_THREADS, 0, s>>>(nb, P, pp, cl.nc, cl.cellof, cl.sfix, cl.sorted, cl.start, cl.count, cl.list,
                                                  pos, Fx, ubar_part);
   else
-    cl_force<false><<<blocks, CL_THREADS, 0, s>>>(nb, P, pp, cl.nc, cl.cellof, cl.sorted, cl.start, cl.count, cl.list,
+    cl_force<false><<<blocks, CL_THREADS, 0, s>>>(nb, P, pp, cl.nc, cl.cellof, cl.sfix, cl.sorted, cl.start, cl.count, cl.list,
                                                   pos, Fx, ubar_part);
   return cudaGetLastError();
 }

@@ -31,8 +31,8 @@ struct CellList {
   int nc;            // cells per side (>= 3)
   int ncells;        // P nc^3
   int *cellof;       // [N*P] cell of bead (l, j), index l*P + j
-  void *crd;         // [N*P] wrapped coordinates: uint4 fixed point (MIXED) or double4 (float64)
-  void *sorted;      // [N*P] the same coordinates in cell order (slot q holds bead list[q])
+  uint4 *fix, *sfix; // [N*P] wrapped coordinates in 32-bit fixed point, and in cell order (slot q: bead list[q])
+  void *crd, *sorted;  // float64: [N*P] the same as double4
   int *count, *fill, *start;  // [ncells]
   int *list;         // [N*P] bead indices l*P + j grouped by cell, ascending within a cell
 };

@@ -108,7 +108,7 @@ int bpimd_create_batched(bpimd_ctx **out, const bpimd_config *cfg, int32_t R, co
     wbytes += align256(layout_workspace(w, nullptr));
     ctx->h_off[r] = off;
     off += 3LL * N[r] * P[r];
-    for (int l0 = 0; l0 < N[r]; l0 += BEAD_BLOCK_PARTICLES) bead_tab.push_back(make_int2(r, l0));
+    for (int l0 = 0; l0 < N[r]; l0 += BATCH_BEAD_PARTICLES) bead_tab.push_back(make_int2(r, l0));
     for (int b = 0; b < w.NB; ++b) blk_tab.push_back(make_int2(r, b));
     if (N[r] <= BATCH_MAX_N) ctx->maxN = std::max(ctx->maxN, N[r]);
     else ctx->n_big++;

@@ -41,8 +41,10 @@ constexpr int CHAIN_PANEL = 64;       // rows solved at a time by a recursion cl
 constexpr int CHAIN_SLICES = 4;       // partial sums a row carries between superblocks
 constexpr int CHAIN_CLUSTER = 8;      // CTAs per recursion (small N)
 constexpr int CHAIN_MAX_N = BPIMD_MAX_N;  // largest N the library accepts
+constexpr int CHAIN_SMALL_N = 128;    // largest single system on one CTA per recursion
 constexpr int BATCH_MAX_N = 4096;     // largest replica of a batch (one CTA per recursion)
 constexpr int BEAD_BLOCK_PARTICLES = 8;  // particles per block of the bead pass
+constexpr int BATCH_BEAD_PARTICLES = 32; // the same in a replica batch
 constexpr double LOG2E = 1.4426950408889634074;
 constexpr double LOG2E_LO = 2.0355273740931033e-17;  // log2(e) - LOG2E (double-double tail)
 constexpr double LN2 = 0.6931471805599453094;
@@ -263,17 +265,21 @@ cudaError_t launch_prep(const Workspace &w, const double *pos, double *F, cudaSt
 cudaError_t launch_gmat_padding(const Workspace &w, cudaStream_t s);
 // both recursions, prefix sums, V_B (device scalar, may be null), normaliser, alpha
 cudaError_t launch_chains(const Workspace &w, double *V_B, cudaStream_t s);
+// single systems of up to CHAIN_SMALL_N particles, one CTA per recursion
+cudaError_t prepare_chains_small();
+cudaError_t launch_chains_small(const Workspace &w, double *V_B, cudaStream_t s);
 // once per process and device, before any stream capture: kernel attributes
 // and the cluster-size choice of the recursions
 cudaError_t prepare_chains();
 // connection probabilities and all exterior-bead forces
 cudaError_t launch_prob_forces(const Workspace &w, const double *pos, double *F, cudaStream_t s);
 cudaError_t launch_dense_probabilities(const Workspace &w, double *M, cudaStream_t s);
-// per block of g: (1/2) m w_P^2 sum Pr[b -> a] |r_b^P - r_a^1|^2 over a <= b (part[NB])
+// parts (part[NB], one per block of g) of the expected spring energy
 cudaError_t launch_spring_expectation(const Workspace &w, double *part, cudaStream_t s);
-// the same per (replica, block) entry of a batch's block table
-cudaError_t launch_spring_expectation_batched(const Workspace *ws, const int2 *tab, int ntab, double *part,
-                                             cudaStream_t s);
+// the same per (replica, block) entry of a batch's block table, and the replicas'
+// sums of v^2 in part[ntab ..]
+cudaError_t launch_spring_expectation_batched(const Workspace *ws, const int2 *tab, int ntab, const long long *off,
+                                             const double *vel, double *part, cudaStream_t s);
 cudaError_t launch_diag_potentials(const Workspace &w, double *Vf, double *Vb, cudaStream_t s);
 
 // Replica batches: ws[r] is replica r's workspace (device array); block tables

@@ -58,12 +58,11 @@ constexpr int SLICES = CHAIN_SLICES;  // partial sums a row carries from superbl
 constexpr int PINV_THREADS = 512;
 
 // Panels of one chain launch.  One launch while its clusters keep up with the
-// sums of later panels; past that, equal superblocks of at most 16 panels with
-// the whole GPU adding each to the later rows.  Evaluations, one launch /
-// superblocks: N = 1601 103.4 / 106.3 us, N = 2048 133.8 / 130.2, N = 4096
-// 381 (32 panels each) / 377.  Where the pair factors are recomputed a sum
-// costs ~6 times as much: 16 panels (N = 8788 2220 / 2100 us, N = 16384
-// 6258 / 5953, 11 or 8 panels 6029 / 6015).
+// sums of later panels; past that, equal superblocks of at most 16 panels, the
+// whole GPU adding each to the later rows.  Evaluations, one launch /
+// superblocks: N = 1601 103.4 / 106.3 us, N = 2048 133.8 / 130.2.  With 16 / 12 /
+// 8 panels a superblock: N = 4096 349 / 364 / 377, recomputed factors N = 8788
+// 1024 / 1042 / 1092, N = 16384 2787 / 2878 / 2989.
 inline int superblock_panels(int panels, bool RC) {
   if (panels <= (RC ? 16 : 28)) return panels;
   const int k = (panels + 15) / 16;
@@ -75,35 +74,35 @@ __device__ __forceinline__ size_t panel_base(const Workspace &w, bool bwd, int t
   return (size_t)((bwd ? (w.N + PT - 1) / PT : 0) + t) * PT * PT;
 }
 
-// Row r's pair factors H(src, r) as stored, or recomputed from the endpoint
-// copies (bit-identical), as c_r H in the K format.
-template <int MODE, bool BWD, bool RC, bool PBC>
-struct RowFactors {
+// acc += sum_i H(src + i STRIDE, row) y_i over eight sources, H recomputed.
+// The exponents come first: where every lane's eight terms lie below 2^-64 of
+// its sum they would be shifted out of it, and the powers of two (the larger
+// part of the work) are left out.  The sum's bits are the same.
+template <int MODE, bool BWD, bool PBC, int STRIDE>
+__device__ __forceinline__ void add_sources_rc(const Workspace &w, const RowFactors<MODE, BWD, true, PBC> &f, bool row_ok,
+                                               int src, int last, const xi (&y)[8], const unsigned long long *T63,
+                                               xi &acc) {
   using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
-  RowEnds<MODE, BWD, PBC> re;
-  int r;
-  __device__ __forceinline__ void load(const Workspace &w, int row) {
-    r = row;
-    if (RC) re.load(w, row);
+  using D_t = typename std::conditional<MODE == BPIMD_FP64, double, float>::type;
+  D_t d2[8];
+  bool need = false;
+  const float cxf = (float)w.cx;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    d2[i] = f.re.dist2(w, min(src + STRIDE * i, last));
+    // pe = e + y.e + 1 with e <= -floor(gap); the eight terms add three bits
+    need |= !(pairg::g_below(d2[i], cxf) > (float)(y[i].e - acc.e + 70));
   }
-  __device__ __forceinline__ void h(const Workspace &w, int src, const unsigned long long *T63, M_t &m,
-                                    int &e) const {
-    if constexpr (RC) {
-      m = re.h(w, src, T63, e);
-    } else {
-      const size_t gi = hidx(src, r);
-      m = __ldg((const M_t *)chain_gm<BWD>(w) + gi);
-      e = __ldg(chain_ge<BWD>(w) + gi);
-    }
+  if (!__any_sync(0xffffffffu, need && row_ok)) return;
+  unsigned long long kk[8];
+  int e[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const M_t m = pairg::g_of_d2<MODE>(d2[i], w.cx, T63, e[i]);
+    kk[i] = mant53(m) << 11;
   }
-  __device__ __forceinline__ xk k(const Workspace &w, xd c, int src, const unsigned long long *T63) const {
-    M_t m;
-    int e;
-    h(w, src, T63, m, e);
-    return mul_mant<M_t>(c, m, e);
-  }
-};
-
+  if (row_ok) acc = xi_add(acc, xsum_fin<3>(xsum_dot<3, 8>(kk, e, y, 0, 2 * XZERO_E)));
+}
 
 // ---------------------------------------------------------- panel inverses
 // A panel and recursion: a cluster of four CTAs.  The CTA pair of diagonal
@@ -496,20 +495,27 @@ __device__ void run_chain(const Workspace &w, int t0, int np, ChainSmem &sm, dou
       if (p >= np) continue;
       handoff_wait(smem_addr(&sm.xbar[t]), 0, w.status, aborted);
       for (; p < np; p += S::BULK) {
-        if (RC) load_factors(t, p);
         xi acc{sm.Am[p][lane], sm.Ae[p][lane]};
 #pragma unroll
         for (int h = 0; h < SRC; h += 8) {
-          unsigned long long kk[8];
-          int e[8];
           xi y[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            kk[i] = mant53(fm[h + i]) << 11;
-            e[i] = fe[h + i];
-            y[i] = wire_get(&sm.X[t][part + PARTS * (h + i)]);
+          for (int i = 0; i < 8; ++i) y[i] = wire_get(&sm.X[t][part + PARTS * (h + i)]);
+          if constexpr (RC) {
+            const int r = row0 + p * PT + (int)rank * R + rr;
+            RowFactors<MODE, BWD, true, PBC> f;
+            f.load(w, min(r, N - 1));
+            add_sources_rc<MODE, BWD, PBC, PARTS>(w, f, r < N, row0 + t * PT + 1 + part + PARTS * h, N - 1, y, sm.T63, acc);
+          } else {
+            unsigned long long kk[8];
+            int e[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              kk[i] = mant53(fm[h + i]) << 11;
+              e[i] = fe[h + i];
+            }
+            acc = xi_add(acc, xsum_fin<3>(xsum_dot<3, 8>(kk, e, y, 0, 2 * XZERO_E)));
           }
-          acc = xi_add(acc, xsum_fin<3>(xsum_dot<3, 8>(kk, e, y, 0, 2 * XZERO_E)));
         }
         if (!RC) {
           npan += S::BULK;
@@ -579,10 +585,14 @@ __global__ void __launch_bounds__(ChainShape<CL>::THREADS, 1) chain_kernel(Works
 }
 
 // ------------------------------------------------------ between superblocks
-// Sources s0 .. s0+ns-1 (finished Y) added to the sums of rows r0 .. N-1 (r0 a
-// multiple of 32): one CTA per (row tile, recursion, slice of the sources),
+// Sources s0 .. s0+ns-1 (finished Y) added to the sums of the rows from r0 (a
+// multiple of 32) on: one CTA per (row tile, recursion, slice of the sources),
 // lane = row, a warp an eighth of the slice; the warps' sums meet in a fixed
-// order.  `first`: the slice's sum starts here.
+// order.  `first`: the slice's sum starts here.  The next superblock's rows
+// come first; the later ones are added while its recursions run (`beside`:
+// launched behind them without waiting for them, as their predecessors' end
+// was theirs to wait for; the first block waits before it ends, so that the
+// next kernel's wait covers both).
 constexpr int UPD_THREADS = 256, UPD_WARPS = UPD_THREADS / 32;
 constexpr int UPD_MAX_SRC = 1024;  // sources of a slice staged at a time
 
@@ -607,20 +617,24 @@ __device__ void source_update(const Workspace &w, int r0, int s0, int ns, bool f
       Y[i].e = y.e;
     }
     __syncthreads();
-    if (r < w.N)
-      for (int i0 = 8 * wid; i0 < n8; i0 += 8 * UPD_WARPS) {
+    for (int i0 = 8 * wid; i0 < n8; i0 += 8 * UPD_WARPS) {
+      xi y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) y[i] = wire_get(&Y[i0 + i]);
+      if constexpr (RC) {
+        add_sources_rc<MODE, BWD, PBC, 1>(w, f, r < w.N, base + i0, base + n - 1, y, T63, acc);
+      } else if (r < w.N) {
         unsigned long long kk[8];
         int e[8];
-        xi y[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           M_t m;
           f.h(w, base + min(i0 + i, n - 1), T63, m, e[i]);
           kk[i] = mant53(m) << 11;
-          y[i] = wire_get(&Y[i0 + i]);
         }
         acc = xi_add(acc, xsum_fin<3>(xsum_dot<3, 8>(kk, e, y, 0, 2 * XZERO_E)));
       }
+    }
   }
   pm[wid][lane] = acc.m;
   pe[wid][lane] = acc.e;
@@ -636,20 +650,27 @@ __device__ void source_update(const Workspace &w, int r0, int s0, int ns, bool f
 }
 
 template <int MODE, bool RC>
-__global__ void __launch_bounds__(UPD_THREADS) source_update_kernel(Workspace w, int r0, int s0, int ns, bool first) {
+__global__ void __launch_bounds__(UPD_THREADS) source_update_kernel(Workspace w, int r0, int s0, int ns, bool first,
+                                                                    bool beside) {
   __shared__ Wire Y[UPD_MAX_SRC];
   __shared__ unsigned long long pm[UPD_WARPS][32];
   __shared__ int pe[UPD_WARPS][32];
   __shared__ unsigned long long T63[RC ? 256 : 1];
   if (RC) pairg::table_init(T63);  // published by the staging's barrier
-  pdl_wait();
-  pdl_trigger();
+  if (!beside) {
+    pdl_wait();
+    pdl_trigger();
+  }
   if (RC && w.pbc) {
     if (blockIdx.y == 0) source_update<MODE, false, RC, RC>(w, r0, s0, ns, first, Y, T63, pm, pe);
     else source_update<MODE, true, RC, RC>(w, r0, s0, ns, first, Y, T63, pm, pe);
   } else {
     if (blockIdx.y == 0) source_update<MODE, false, RC, false>(w, r0, s0, ns, first, Y, T63, pm, pe);
     else source_update<MODE, true, RC, false>(w, r0, s0, ns, first, Y, T63, pm, pe);
+  }
+  if (beside) {
+    pdl_trigger();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) pdl_wait();
   }
 }
 
@@ -673,23 +694,26 @@ cudaError_t launch_chain_cluster(const Workspace &w, double *V_B, cudaStream_t s
   cfg.dynamicSmemBytes = sizeof(PinvSmem);
   cfg.numAttrs = 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, panel_inverse_kernel<MODE, RC>, w);
-  const int sb = superblock_panels(panels, RC);
-  for (int t0 = 0; t0 < panels && e == cudaSuccess; t0 += sb) {
-    const int np = panels - t0 < sb ? panels - t0 : sb;
-    if (t0) {
-      const int s0 = t0 == sb ? 0 : (t0 - sb) * PT + 1, r0 = t0 * PT;
-      cfg.gridDim = dim3((w.N - r0 + TILE - 1) / TILE, 2, SLICES);
-      cfg.blockDim = dim3(UPD_THREADS);
-      cfg.dynamicSmemBytes = 0;
-      cfg.numAttrs = 1;
-      e = cudaLaunchKernelEx(&cfg, source_update_kernel<MODE, RC>, w, r0, s0, r0 + 1 - s0, t0 == sb);
-      if (e != cudaSuccess) return e;
-    }
+  const int sb = superblock_panels(panels, RC), rows = sb * PT;
+  // superblock k's Y into the rows from r0 to r1
+  auto update = [&](int k, int r0, int r1, bool beside) {
+    const int s0 = k == 0 ? 0 : k * rows + 1, ns = (k + 1) * rows + 1 - s0;
+    cfg.gridDim = dim3((r1 - r0 + TILE - 1) / TILE, 2, SLICES);
+    cfg.blockDim = dim3(UPD_THREADS);
+    cfg.dynamicSmemBytes = 0;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, source_update_kernel<MODE, RC>, w, r0, s0, ns, k == 0, beside);
+  };
+  for (int t0 = 0, k = 0; t0 < panels && e == cudaSuccess; t0 += sb, ++k) {
+    const int np = panels - t0 < sb ? panels - t0 : sb, r0 = k * rows, r1 = r0 + rows;  // this superblock's rows
+    if (k > 0) e = update(k - 1, r0, r1 < w.N ? r1 : w.N, false);
+    if (e != cudaSuccess) return e;
     cfg.gridDim = dim3(2 * CL);
     cfg.blockDim = dim3(ChainShape<CL>::THREADS);
     cfg.dynamicSmemBytes = sizeof(ChainSmem);
     cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, chain_kernel<MODE, CL, RC>, w, t0, np, V_B);
+    if (e == cudaSuccess && k > 0 && r1 < w.N) e = update(k - 1, r1, w.N, true);
   }
   return e;
 }
@@ -770,7 +794,8 @@ cudaError_t prepare_chains() {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_chain_mutex);
   if (g_chain_ready[dev]) return cudaSuccess;
-  e = prepare_chain_variants<CHAIN_CLUSTER>();
+  e = prepare_chains_small();
+  if (e == cudaSuccess) e = prepare_chain_variants<CHAIN_CLUSTER>();
   if (e != cudaSuccess) return e;
   bool large = prepare_chain_variants<CHAIN_CLUSTER_LARGE>() == cudaSuccess;
   cudaGetLastError();
@@ -784,6 +809,10 @@ cudaError_t launch_chains(const Workspace &w, double *V_B, cudaStream_t s) {
   if (!w.blocks) return cudaErrorInvalidValue;  // no panel-inverse storage in this workspace
   cudaError_t e = prepare_chains();
   if (e != cudaSuccess) return e;
+  // One CTA per recursion with 32-row tiles and no panel inverses, against the
+  // panels on clusters: N = 16 16.7 / 20.8 us, N = 64 20.5 / 25.5, N = 128
+  // 25.5 / 26.6, N = 192 31.7 / 28.3.
+  if (!w.mixed && !w.test_timeout && w.N <= CHAIN_SMALL_N) return launch_chains_small(w, V_B, s);
   int dev = 0;
   cudaGetDevice(&dev);
   bool large_ok;

@@ -26,36 +26,11 @@ __device__ __forceinline__ double scale_nonpos(double x, int k) {
   return (ex + k <= 0) ? 0.0 : __longlong_as_double(b + ((long long)k << 52));
 }
 
-// acc + K * y, branch-free, for the dependency chain.  Operands are extended
-// numbers whose mantissas are normal doubles in [1, 2^60) (an extended zero is
-// carried as mantissa 1 with exponent XZERO_E, i.e. 2^-536870912).  Both
-// operands are scaled by 2^k, k <= 0 clamped at -1000, by adding k to the
-// exponent field of the high word: a clamped operand is below 2^-900 of the
-// other and cannot change the float64 sum.  One float64 FMA, five integer ops.
-__device__ __forceinline__ xd fma_chain(xd acc, double km, int ke, xd y) {
-  const int pe = ke + y.e;
-  const int E = max(acc.e, pe);
-  const int k1 = max(pe - E, -1000), k2 = max(acc.e - E, -1000);
-  const double ks = __hiloint2double(__double2hiint(km) + k1 * (1 << 20), __double2loint(km));
-  const double as = __hiloint2double(__double2hiint(acc.m) + k2 * (1 << 20), __double2loint(acc.m));
-  return xd{fma(ks, y.m, as), E};
-}
-
 // Explicit shared-memory loads (32-bit shared-window addresses).
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ double lds_f64(unsigned a) {
-  double v;
-  asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a));
-  return v;
-}
 __device__ __forceinline__ unsigned long long lds_u64(unsigned a) {
   unsigned long long v;
   asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ float lds_f32(unsigned a) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
   return v;
 }
 __device__ __forceinline__ int lds_s32(unsigned a) {
@@ -174,24 +149,10 @@ struct xs {
   unsigned m;
   int e;
 };
-__device__ __forceinline__ xs xs_from(xd a) {
-  const long long b = __double_as_longlong(a.m);
-  if (b <= 0) return xs{1u << 30, XZERO_E};
-  return xs{(unsigned)((((unsigned long long)b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) >> 22), a.e + (int)(b >> 52) - 1023};
-}
-__device__ __forceinline__ xd xs_to_xd(xs a) {
-  return xd{__longlong_as_double((long long)((((unsigned long long)a.m << 22) & 0xFFFFFFFFFFFFFull) |
-                                             0x3FF0000000000000ull)),
-            a.e};
-}
 // s * 2^(E - 30) with s in [2^29, 2^32), brought back to [2^30, 2^31)
 __device__ __forceinline__ xs xs_norm(unsigned s, int E) {
   const unsigned top = s >> 29;  // 1: [2^29, 2^30), 2-3: in range, 4-7: [2^31, 2^32)
   return xs{top >= 4 ? (s >> 1) : (top >= 2 ? s : (s << 1)), top >= 4 ? E + 1 : (top >= 2 ? E : E - 1)};
-}
-__device__ __forceinline__ xs xs_add(xs a, xs b) {
-  const int E = max(a.e, b.e);
-  return xs_norm((a.m >> min(E - a.e, 31)) + (b.m >> min(E - b.e, 31)), E);
 }
 // a * c (c: positive normal double mantissa, any binary exponent)
 __device__ __forceinline__ xs xs_mul(xs a, xd c) {
@@ -249,60 +210,6 @@ __device__ __forceinline__ const void *chain_gm(const Workspace &w) { return BWD
 template <bool BWD>
 __device__ __forceinline__ const int *chain_ge(const Workspace &w) { return BWD ? w.gbe : w.ge; }
 
-// Staging issues no float64 instruction (the SM's float64 pipe belongs to the
-// dependency chain).  Pairs outside src <= row < N hold the extended zero
-// 1 * 2^XZERO_E; loads are coalesced along rows and issued before use.
-// Off-diagonal block: H(tt*32+i, (tt+1)*32+lane), rows i in [i0, i0+NR), as
-// stored (float for MIXED), into dm/de[i*33 + lane].
-template <bool MIXED, bool BWD, int NR>
-__device__ __forceinline__ void stage_offdiag(const Workspace &w, int tt, int i0, void *dmv, int *de) {
-  using M_t = typename std::conditional<MIXED, float, double>::type;
-  const int lane = threadIdx.x & 31;
-  const int srcbase = tt * TILE, row = tt * TILE + TILE + lane;
-  const M_t *gm = (const M_t *)chain_gm<BWD>(w);
-  const int *ge = chain_ge<BWD>(w);
-  M_t *dm = (M_t *)dmv;
-#pragma unroll
-  for (int i = i0; i < i0 + NR; ++i) {
-    M_t m = (M_t)1.0;
-    int e = XZERO_E;
-    if (row < w.N) {
-      const size_t gi = hidx(srcbase + i, row);
-      m = __ldg(gm + gi);
-      e = __ldg(ge + gi);
-    }
-    dm[i * 33 + lane] = m;
-    de[i * 33 + lane] = e;
-  }
-}
-
-// Diagonal block of tile tt, K = c_row * H as 64-bit integer mantissas (the
-// chain format of xi_fma), rows i in [i0, i0+NR): the mantissa product is
-// formed on the integer pipe (mul_mant).
-template <bool MIXED, bool BWD, int NR>
-__device__ __forceinline__ void stage_diag(const Workspace &w, int tt, int i0, unsigned long long *dm, int *de) {
-  using M_t = typename std::conditional<MIXED, float, double>::type;
-  const int lane = threadIdx.x & 31;
-  const int r0 = tt * TILE, row = r0 + lane;
-  const M_t *gm = (const M_t *)chain_gm<BWD>(w);
-  const int *ge = chain_ge<BWD>(w);
-  const xd c = (row < w.N) ? xnorm_int(chain_coef<BWD>(w, row)) : xd{1.0, 0};
-#pragma unroll
-  for (int i = i0; i < i0 + NR; ++i) {
-    const int src = r0 + i;
-    M_t m = (M_t)1.0;
-    int e = XZERO_E;
-    if (row < w.N && src <= row) {
-      const size_t gi = hidx(src, row);
-      m = __ldg(gm + gi);
-      e = __ldg(ge + gi);
-    }
-    const xk k = mul_mant<M_t>(c, m, e);
-    dm[i * 33 + lane] = k.m;
-    de[i * 33 + lane] = k.e;
-  }
-}
-
 // ------------------------------------------ recompute mode (no stored g)
 // H(src, row) of a recursion from the bead pass's endpoint copies: forward
 // H(w, r) = g(a = w, b = r); backward H(w, r) = g(a = N-1-r, b = N-1-w), b the
@@ -319,86 +226,149 @@ struct RowEnds {
     const auto s = pairg::load_end<MODE != BPIMD_FP64, PBC>(w, BWD ? w.N - 1 - src : src, BWD);
     return BWD ? pairg::g_of<MODE, PBC>(w, s, row, w.cx, T63, e) : pairg::g_of<MODE, PBC>(w, row, s, w.cx, T63, e);
   }
+  // the squared distance h() takes its power of
+  __device__ __forceinline__ typename std::conditional<MODE == BPIMD_FP64, double, float>::type dist2(const Workspace &w,
+                                                                                                  int src) const {
+    const auto s = pairg::load_end<MODE != BPIMD_FP64, PBC>(w, BWD ? w.N - 1 - src : src, BWD);
+    if constexpr (MODE == BPIMD_FP64) return BWD ? pairg::dist2<PBC>(w, s, row) : pairg::dist2<PBC>(w, row, s);
+    else return BWD ? pairg::dist2(w, s, row) : pairg::dist2(w, row, s);
+  }
 };
 
+// Row r's pair factors H(src, r) as stored, or recomputed from the endpoint
+// copies (bit-identical), as c_r H in the K format.
+template <int MODE, bool BWD, bool RC, bool PBC>
+struct RowFactors {
+  using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
+  RowEnds<MODE, BWD, PBC> re;
+  size_t base;  // H(src, row) is at base + 32 src (a tile's blocks lie one after the other)
+  __device__ __forceinline__ void load(const Workspace &w, int row) {
+    if (RC) re.load(w, row);
+    else base = hidx(0, row);
+  }
+  __device__ __forceinline__ void h(const Workspace &w, int src, const unsigned long long *T63, M_t &m,
+                                    int &e) const {
+    if constexpr (RC) {
+      m = re.h(w, src, T63, e);
+    } else {
+      const size_t gi = base + 32 * src;
+      m = __ldg((const M_t *)chain_gm<BWD>(w) + gi);
+      e = __ldg(chain_ge<BWD>(w) + gi);
+    }
+  }
+  __device__ __forceinline__ xk k(const Workspace &w, xd c, int src, const unsigned long long *T63) const {
+    M_t m;
+    int e;
+    h(w, src, T63, m, e);
+    return mul_mant<M_t>(c, m, e);
+  }
+};
+
+
+// Staging issues no float64 instruction.  Pairs outside src <= row < N hold the
+// extended zero 1 * 2^XZERO_E; loads are coalesced along rows and issued
+// before use.
+// Off-diagonal block: H(tt*32+i, (tt+1)*32+lane), rows i in [i0, i0+NR), as
+// stored (float for MIXED32), into dm/de[i*33 + lane].
+template <int MODE, bool BWD, bool RC, bool PBC, int NR>
+__device__ __forceinline__ void stage_offdiag(const Workspace &w, int tt, int i0, void *dmv, int *de,
+                                              const unsigned long long *T63) {
+  using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
+  const int lane = threadIdx.x & 31;
+  const int srcbase = tt * TILE, row = tt * TILE + TILE + lane;
+  M_t *dm = (M_t *)dmv;
+  RowFactors<MODE, BWD, RC, PBC> f;
+  f.load(w, min(row, w.N - 1));
+#pragma unroll
+  for (int i = i0; i < i0 + NR; ++i) {
+    M_t m = (M_t)1.0;
+    int e = XZERO_E;
+    if (row < w.N) f.h(w, srcbase + i, T63, m, e);
+    dm[i * 33 + lane] = m;
+    de[i * 33 + lane] = e;
+  }
+}
+
+// Diagonal block of tile tt, K = c_row * H as 64-bit integer mantissas (the
+// chain format of xi_fma), rows i in [i0, i0+NR): the mantissa product is
+// formed on the integer pipe (mul_mant).
+template <int MODE, bool BWD, bool RC, bool PBC, int NR>
+__device__ __forceinline__ void stage_diag(const Workspace &w, int tt, int i0, unsigned long long *dm, int *de,
+                                           const unsigned long long *T63) {
+  using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
+  const int lane = threadIdx.x & 31;
+  const int r0 = tt * TILE, row = r0 + lane;
+  const xd c = (row < w.N) ? xnorm_int(chain_coef<BWD>(w, row)) : xd{1.0, 0};
+  RowFactors<MODE, BWD, RC, PBC> f;
+  f.load(w, min(row, w.N - 1));
+#pragma unroll
+  for (int i = i0; i < i0 + NR; ++i) {
+    const int src = r0 + i;
+    M_t m = (M_t)1.0;
+    int e = XZERO_E;
+    if (row < w.N && src <= row) f.h(w, src, T63, m, e);
+    const xk k = mul_mant<M_t>(c, m, e);
+    dm[i * 33 + lane] = k.m;
+    de[i * 33 + lane] = k.e;
+  }
+}
+
 // The 32 dependent steps of row tile t, run by one warp.  A is this lane's
-// row sum over sources < 32t except tile t-1 (which is in nxt), crow the row's
-// coefficient.  K (diagonal, c-scaled, integer mantissas) and H (to tile t+1)
-// are the staged blocks.  Y_v lives at Ym/Ye[v & ymask] in shared memory and,
-// unless gYm is null, at gYm/gYe[v] in global memory.  On return nxt holds
-// the partial sums of tile t+1's rows over source tile t.
+// row sum over sources < 32t, crow the row's coefficient; K (diagonal,
+// c-scaled, integer mantissas) is the staged block.  Y_v lives at Ym/Ye[v] in
+// shared memory (with its xi mantissa at Yk[v]) and at gYm/gYe[v] in global memory.
 // 32 steps, no branches and no stores: rows past N and finished rows see
 // extended zeros in the staged blocks, and row j's accumulator is final after
 // step j.  The chain (acc, y) is in an integer format (xs for MIXED, xi for
 // FP64); block entries of step i+1 are loaded (explicit ld.shared) before
-// step i's shuffle.
+// step i's shuffle.  Nothing else sits in the loop: a float64 sum for the next
+// tile's rows beside it made a step 240 cycles instead of ~100.
 template <bool MIXED>
-__device__ __forceinline__ void chain_tile(int N, int t, xd A, xd crow, xd &nxt, const unsigned long long *Kdm,
-                                           const int *Kde, const double *Hom, const int *Hoe, double *Ym, int *Ye,
-                                           int ymask, double *gYm, int *gYe) {
+__device__ __forceinline__ void chain_tile(int N, int t, xi A, xd crow, const unsigned long long *Kdm, const int *Kde,
+                                           double *Ym, int *Ye, unsigned long long *Yk, double *gYm, int *gYe) {
   // the chain format: 32-bit words (MIXED, xs) or 64-bit mantissas (FP64, xi)
   using X = typename std::conditional<MIXED, xs, xi>::type;
   const int lane = threadIdx.x & 31;
   const int r0 = t * TILE, row = r0 + lane;
-  const xd y0{Ym[r0 & ymask], Ye[r0 & ymask]};
   X acc, y;
   if constexpr (MIXED) {
     acc = xs{1u << 30, XZERO_E};
-    if (row < N) acc = xs_mul(xs_add(xs_from(A), xs_from(nxt)), crow);  // c_row * (sum over sources < r0)
-    y = xs_from(y0);
+    if (row < N) acc = xs_mul(xs{(unsigned)(A.m >> 32), A.e}, crow);  // c_row * (sum over sources < r0)
+    y = xs{(unsigned)(Yk[r0] >> 32), Ye[r0]};
   } else {
     acc = xi{1ull << 62, XZERO_E};
-    if (row < N) acc = xi_mul(xi_add(xi_from(A), xi_from(nxt)), crow);
-    y = xi_from(y0);
+    if (row < N) acc = xi_mul(A, crow);
+    y = xi{Yk[r0], Ye[r0]};
   }
-  nxt = xd{1.0, XZERO_E};
-  float nsum = 0.0f;  // MIXED: the next tile's partial sum in float32
-  int nexp = XZERO_E;
-  const unsigned aKm = smem_addr(Kdm + lane), aKe = smem_addr(Kde + lane), aHe = smem_addr(Hoe + lane);
-  const unsigned aHm = MIXED ? smem_addr((const float *)Hom + lane) : smem_addr(Hom + lane);
+  const unsigned aKm = smem_addr(Kdm + lane), aKe = smem_addr(Kde + lane);
   unsigned long long km = lds_u64(aKm);
-  double hm = MIXED ? 0.0 : lds_f64(aHm);
-  float hf = MIXED ? lds_f32(aHm) : 0.0f;
-  int ke = lds_s32(aKe), he = lds_s32(aHe);
+  int ke = lds_s32(aKe);
 #pragma unroll
   for (int i = 0; i < TILE; ++i) {
     unsigned long long km1 = 0;
-    double hm1 = 0.0;
-    float hf1 = 0.0f;
-    int ke1 = 0, he1 = 0;
+    int ke1 = 0;
     if (i + 1 < TILE) {
       km1 = lds_u64(aKm + (i + 1) * 33 * 8);
-      if (MIXED) hf1 = lds_f32(aHm + (i + 1) * 33 * 4);
-      else hm1 = lds_f64(aHm + (i + 1) * 33 * 8);
       ke1 = lds_s32(aKe + (i + 1) * 33 * 4);
-      he1 = lds_s32(aHe + (i + 1) * 33 * 4);
     }
-    if constexpr (MIXED) {
-      acc = xs_fma(acc, km, ke, y);  // the dependency chain
-      // next tile's rows, off the chain: float32 on the top 24 bits of y
-      fmerge(nsum, nexp, __int_as_float((int)((y.m >> 7) & 0x7FFFFFu) | 0x3F800000) * hf, he + y.e);
-    } else {
-      acc = xi_fma<false>(acc, km, ke, y);  // the dependency chain
-      nxt = fma_chain(nxt, hm, he, xi_to_xd(y));
-    }
+    if constexpr (MIXED) acc = xs_fma(acc, km, ke, y);
+    else acc = xi_fma<false>(acc, km, ke, y);
     y.m = __shfl_sync(0xffffffffu, acc.m, i);
     y.e = __shfl_sync(0xffffffffu, acc.e, i);
-    km = km1; hm = hm1; hf = hf1; ke = ke1; he = he1;
+    km = km1;
+    ke = ke1;
   }
-  if (MIXED) nxt = xd{f2d_int(nsum), nexp};
-
   if (row < N) {  // Y_{row+1} = final accumulator of row `row`
-    xd yn;
-    if constexpr (MIXED) yn = xs_to_xd(acc);
-    else yn = xi_to_xd(acc);
-    Ym[(row + 1) & ymask] = yn.m;
-    Ye[(row + 1) & ymask] = yn.e;
-    if (gYm) {
-      gYm[row + 1] = yn.m;
-      gYe[row + 1] = yn.e;
-    }
+    xi yk;
+    if constexpr (MIXED) yk = xi{(unsigned long long)acc.m << 32, acc.e};
+    else yk = acc;
+    const xd yn = xi_to_xd(yk);
+    Yk[row + 1] = yk.m;
+    Ym[row + 1] = yn.m;
+    Ye[row + 1] = yn.e;
+    gYm[row + 1] = yn.m;
+    gYe[row + 1] = yn.e;
   }
-  nxt = xnorm_int(nxt);
 }
 
 // ------------------------------------------------ mbarriers

@@ -304,8 +304,17 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
         const bool valid = q + k < p1 && (row_item ? q + k <= me : q + k >= me);
         const EP oth = staged_end<F64, PBC>(sm.part, i);
         const EP &eb = row_item ? mine : oth, &ea = row_item ? oth : mine;
-        if constexpr (RC) m[k] = pairg::g_of<MODE, PBC>(w, eb, ea, w.cx, T63, e[k]);
         auto d = pairg::diff3(w, eb, ea);
+        if constexpr (RC && !F64) {
+          // below 2^-126 a term is zero: where every lane's is, by a bound on
+          // g's exponent, the power of two is left out with the rest
+          const float d2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
+          const bool zero = !valid || pairg::g_below(d2, (float)w.cx) > (float)(sm.part.e[i] + own_e + 128);
+          if (__all_sync(0xffffffffu, zero)) continue;
+          m[k] = pairg::g_of_d2<MODE>(d2, w.cx, T63, e[k]);
+        } else if constexpr (RC) {
+          m[k] = pairg::g_of<MODE, PBC>(w, eb, ea, w.cx, T63, e[k]);
+        }
         if constexpr (F64) {
           const unsigned long long t = valid ? pow2fx::mulhi(sm.part.m[i], mant64(m[k])) : 0ull;  // value t 2^(et - 63)
           const int et = valid ? sm.part.e[i] + e[k] + 1 : NO_TERM;
@@ -455,37 +464,60 @@ __global__ void __launch_bounds__(PROB_THREADS) exterior_batched(const Workspace
   pdl_trigger();
 }
 
-// Expected exterior-spring energy over representative permutations, per block
-// of the lower triangle: (1/2) m w_P^2 sum_{a<=b in block} Pr[b -> a] |r_b^P - r_a^1|^2
-// (the direct links l -> l+1 are added by the caller).  Float64 throughout;
-// run once per molecular-dynamics call, for the primitive energy estimator.
-// All threads of the block call it; thread 0 gets the sum.
-__device__ double spring_block(const Workspace &w, int blk, double *red) {
-  int t, s;
-  block_coords_f(blk, t, s);
-  double acc = 0.0;
-  for (int e = threadIdx.x; e < TILE2; e += blockDim.x) {
-    const int a = s * TILE + (e >> 5), b = t * TILE + (e & 31);
-    if (b < w.N && a <= b) {
-      const size_t gi = (size_t)blk * TILE2 + e;
-      const xd g = w.recomp ? pairg::g_runtime(w, a, b)
-                            : xd{w.mixed ? (double)((const float *)w.gm)[gi] : ((const double *)w.gm)[gi], w.ge[gi]};
-      const xd al = alpha_of(w, a), mu = mu_of(w, b);
-      const double M = xtod(xd{al.m * mu.m * g.m, al.e + mu.e + g.e});
-      const double dx = mimage(w, w.RP[4 * b] - w.R1[4 * a]), dy = mimage(w, w.RP[4 * b + 1] - w.R1[4 * a + 1]),
-                   dz = mimage(w, w.RP[4 * b + 2] - w.R1[4 * a + 2]);
-      acc += M * (dx * dx + dy * dy + dz * dz);
-    }
-  }
+// Sum over the block's threads (fixed order); thread 0 gets it.
+__device__ double sum_block(double v, double *red) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   double sum = 0.0;
   if (threadIdx.x == 0)
     for (int q = 0; q < (int)(blockDim.x >> 5); ++q) sum += red[q];
   __syncthreads();
-  return w.half_k * sum;
+  return sum;
+}
+
+// Expected spring energy over representative permutations, in parts: block blk
+// of the lower triangle gives (1/2) m w_P^2 sum_{a<=b in block} Pr[b -> a]
+// |r_b^P - r_a^1|^2, and particles 256 blk .. 256 blk + 255 their interior
+// springs and direct links.  Float64 throughout; run once per
+// molecular-dynamics call, for the primitive energy estimator.  The exponents
+// of a probability's factors are added first: below 2^-100 it adds nothing to a
+// sum of order N kT, and its float64 arithmetic (~75 cycles an instruction, ~30
+// of them) and loads are left out -- nearly every pair of a liquid (391 us a
+// call at N = 4000 before).  All threads of the block call it; thread 0 gets the sum.
+__device__ double spring_block(const Workspace &w, int blk, double *red) {
+  int t, s;
+  block_coords_f(blk, t, s);
+  const int inv_e = w.scal_i[0];
+  const double inv_m = w.scal[1];
+  double acc = 0.0;
+  for (int e = threadIdx.x; e < TILE2; e += blockDim.x) {
+    const int a = s * TILE + (e >> 5), b = t * TILE + (e & 31);
+    if (b < w.N && a <= b) {
+      const size_t gi = (size_t)blk * TILE2 + e;
+      const int r = w.N - 1 - b;
+      int ex = w.yfe[a] + w.ybe[r] + inv_e;
+      xd g{0.0, 0};
+      if (w.recomp) g = pairg::g_runtime(w, a, b);
+      else g.e = w.ge[gi];
+      ex += g.e;
+      if (ex >= -100) {
+        if (!w.recomp) g.m = w.mixed ? (double)((const float *)w.gm)[gi] : ((const double *)w.gm)[gi];
+        const double M = (w.yfm[a] * w.ybm[r]) * (g.m * inv_m) * pow2_normal(ex);
+        const double dx = mimage(w, w.RP[4 * b] - w.R1[4 * a]), dy = mimage(w, w.RP[4 * b + 1] - w.R1[4 * a + 1]),
+                     dz = mimage(w, w.RP[4 * b + 2] - w.R1[4 * a + 2]);
+        acc += M * (dx * dx + dy * dy + dz * dz);
+      }
+    }
+  }
+  acc *= w.half_k;
+  const int l = blk * blockDim.x + threadIdx.x;
+  if (l < w.N) {
+    acc += w.Eint[l];
+    if (l + 1 < w.N) acc += direct_link_fast(w, l) * w.link[l];
+  }
+  return sum_block(acc, red);
 }
 
 __global__ void __launch_bounds__(256) spring_expect_kernel(Workspace w, double *part) {
@@ -496,14 +528,26 @@ __global__ void __launch_bounds__(256) spring_expect_kernel(Workspace w, double 
   }
 }
 
-// Replica batch: entry k of tab is (replica, block); part[k] as above.
+// Replica batch: entry k of tab is (replica, block); part[k] as above, and
+// part[ntab + k] the sum of v^2 over the block's share of the replica's
+// velocities (packed, replica r at element off[r]).
 __global__ void __launch_bounds__(256) spring_expect_batched(const Workspace *__restrict__ ws,
-                                                             const int2 *__restrict__ tab, int ntab, double *part) {
+                                                             const int2 *__restrict__ tab, int ntab,
+                                                             const long long *__restrict__ off,
+                                                             const double *__restrict__ vel, double *part) {
   __shared__ double red[8];
   for (int k = blockIdx.x; k < ntab; k += gridDim.x) {
     const int2 e = tab[k];
-    const double v = spring_block(ws[e.x], e.y, red);
-    if (threadIdx.x == 0) part[k] = v;
+    const Workspace &w = ws[e.x];
+    const double v = spring_block(w, e.y, red);
+    const long long n = 3LL * w.N * w.P, lo = n * e.y / w.NB, hi = n * (e.y + 1) / w.NB;
+    double ke = 0.0;
+    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) ke = fma(vel[off[e.x] + i], vel[off[e.x] + i], ke);
+    ke = sum_block(ke, red);
+    if (threadIdx.x == 0) {
+      part[k] = v;
+      part[ntab + k] = ke;
+    }
   }
 }
 
@@ -569,17 +613,17 @@ cudaError_t launch_prob_forces(const Workspace &w, const double *pos, double *F,
 
 cudaError_t launch_spring_expectation(const Workspace &w, double *part, cudaStream_t s) {
   const int sms = sm_count();
-  const int grid = w.NB < sms * 4 ? w.NB : sms * 4;
+  const int grid = w.NB < sms * 8 ? w.NB : sms * 8;
   spring_expect_kernel<<<grid, 256, 0, s>>>(w, part);
   return cudaGetLastError();
 }
 
-cudaError_t launch_spring_expectation_batched(const Workspace *ws, const int2 *tab, int ntab, double *part,
-                                             cudaStream_t s) {
+cudaError_t launch_spring_expectation_batched(const Workspace *ws, const int2 *tab, int ntab, const long long *off,
+                                             const double *vel, double *part, cudaStream_t s) {
   if (ntab <= 0) return cudaSuccess;
   const int sms = sm_count();
-  const int grid = ntab < sms * 4 ? ntab : sms * 4;
-  spring_expect_batched<<<grid, 256, 0, s>>>(ws, tab, ntab, part);
+  const int grid = ntab < sms * 8 ? ntab : sms * 8;
+  spring_expect_batched<<<grid, 256, 0, s>>>(ws, tab, ntab, off, vel, part);
   return cudaGetLastError();
 }
 

@@ -41,6 +41,7 @@ namespace bpimd {
 namespace {
 
 constexpr int MD_THREADS = 256;
+constexpr int ENERGY_THREADS = 1024;  // the one block that adds a call's partial energies
 constexpr int EXT_THREADS = 128;
 constexpr int EXT_WARPS = EXT_THREADS / 32;
 // lanes per particle in the all-pairs force (two particles a thread): float64
@@ -578,26 +579,21 @@ __global__ void __launch_bounds__(EXT_THREADS) ext_force_batched(const double *_
 // energies[4 r + 0..3] of replica r (one block each): V_B, U-bar, kinetic,
 // primitive estimator, from the partial sums of the last force pass.
 __global__ void __launch_bounds__(MD_THREADS) energies_batched(const Workspace *__restrict__ ws,
-                                                               const long long *__restrict__ off,
                                                                const double *__restrict__ VBr,
                                                                const double *__restrict__ ubar_part,
                                                                const int *__restrict__ ext_first,
                                                                const double *__restrict__ spring_part,
-                                                               const int *__restrict__ blk_first,
-                                                               const double *__restrict__ v, double half_m,
-                                                               double *energies) {
+                                                               const int *__restrict__ blk_first, int ntab,
+                                                               double half_m, double *energies) {
   __shared__ double red[MD_THREADS / 32];
   const int r = blockIdx.x;
   const Workspace &w = ws[r];
   double sp = 0.0, ub = 0.0, ke = 0.0;
-  for (int q = blk_first[r] + threadIdx.x; q < blk_first[r + 1]; q += blockDim.x) sp += spring_part[q];
-  for (int l = threadIdx.x; l < w.N; l += blockDim.x) {
-    sp += w.Eint[l];
-    if (l + 1 < w.N) sp += direct_link_prob(w, l) * w.link[l];
+  for (int q = blk_first[r] + threadIdx.x; q < blk_first[r + 1]; q += blockDim.x) {
+    sp += spring_part[q];
+    ke += spring_part[ntab + q];
   }
   for (int q = ext_first[r] + threadIdx.x; q < ext_first[r + 1]; q += blockDim.x) ub += ubar_part[q];
-  const long long n = 3LL * w.N * w.P;
-  for (long long e = threadIdx.x; e < n; e += blockDim.x) ke += v[off[r] + e] * v[off[r] + e];
   sp = block_sum(sp, red);
   ub = block_sum(ub, red);
   ke = block_sum(ke, red);
@@ -624,16 +620,12 @@ __global__ void __launch_bounds__(MD_THREADS) ke_kernel(const double *__restrict
 
 // energies[0..3] = V_B, U-bar, kinetic, primitive estimator 3NP/(2 beta) - <springs> + U-bar,
 // with <springs> = sum_l E_int + sum Pr[l -> u<=l] (1/2)k d^2 + sum Pr[l -> l+1] link_l.
-__global__ void __launch_bounds__(MD_THREADS) energies_kernel(Workspace w, const double *VB, const double *ubar_part,
+__global__ void __launch_bounds__(ENERGY_THREADS) energies_kernel(Workspace w, const double *VB, const double *ubar_part,
                                                               int n_ubar, const double *ke_part, int n_ke,
                                                               const double *spring_part, double *energies) {
-  __shared__ double red[MD_THREADS / 32];
+  __shared__ double red[ENERGY_THREADS / 32];
   double sp = 0.0, ub = 0.0, ke = 0.0;
   for (int q = threadIdx.x; q < w.NB; q += blockDim.x) sp += spring_part[q];
-  for (int l = threadIdx.x; l < w.N; l += blockDim.x) {
-    sp += w.Eint[l];
-    if (l + 1 < w.N) sp += direct_link_prob(w, l) * w.link[l];
-  }
   for (int q = threadIdx.x; q < n_ubar; q += blockDim.x) ub += ubar_part[q];
   for (int q = threadIdx.x; q < n_ke; q += blockDim.x) ke += ke_part[q];
   sp = block_sum(sp, red);
@@ -914,7 +906,7 @@ int md_run(bpimd_ctx *ctx, double *pos, double *vel, int32_t nsteps, double *ene
     if (cudaGetLastError() != cudaSuccess || launch_spring_expectation(ctx->w, md.spring_part, s) != cudaSuccess)
       rc = BPIMD_ERR_CUDA;
     if (rc == BPIMD_OK) {
-      energies_kernel<<<1, MD_THREADS, 0, s>>>(ctx->w, md.VB, md.ubar_part, md.ext_blocks, md.ke_part, g1,
+      energies_kernel<<<1, ENERGY_THREADS, 0, s>>>(ctx->w, md.VB, md.ubar_part, md.ext_blocks, md.ke_part, g1,
                                               md.spring_part, energies);
       if (cudaGetLastError() != cudaSuccess) rc = BPIMD_ERR_CUDA;
     }
@@ -963,7 +955,7 @@ int md_alloc_batched(bpimd_ctx *ctx, const MDParams &p) {
   }
   blk_first[R] = blk;
   md.n_ext = (int)tab.size();
-  md.spring_blocks = ctx->n_blk_tab;
+  md.spring_blocks = 2 * ctx->n_blk_tab;  // spring and kinetic parts
   md.ke_blocks = 0;
   md.ext_blocks = md.n_ext;
   std::vector<double> c2(R);
@@ -1066,12 +1058,12 @@ int md_run_batched(bpimd_ctx *ctx, double *pos, double *vel, int32_t nsteps, dou
   rc = run_steps(ctx, p, pos, vel, nsteps, [&](KickStep ks) { return total_force_batched(ctx, p, pos, ks); });
   if (rc == BPIMD_OK && energies) {
     cudaStream_t s = ctx->stream;
-    if (launch_spring_expectation_batched(ctx->d_ws, ctx->d_blk_tab, ctx->n_blk_tab, md.spring_part, s) !=
-        cudaSuccess)
+    if (launch_spring_expectation_batched(ctx->d_ws, ctx->d_blk_tab, ctx->n_blk_tab, ctx->d_off, vel, md.spring_part,
+                                          s) != cudaSuccess)
       rc = BPIMD_ERR_CUDA;
     if (rc == BPIMD_OK) {
-      energies_batched<<<ctx->R, MD_THREADS, 0, s>>>(ctx->d_ws, ctx->d_off, md.VBr, md.ubar_part, md.ext_first,
-                                                     md.spring_part, md.blk_first, vel, 0.5 * ctx->cfg.m, energies);
+      energies_batched<<<ctx->R, MD_THREADS, 0, s>>>(ctx->d_ws, md.VBr, md.ubar_part, md.ext_first, md.spring_part,
+                                                     md.blk_first, ctx->n_blk_tab, 0.5 * ctx->cfg.m, energies);
       if (cudaGetLastError() != cudaSuccess) rc = BPIMD_ERR_CUDA;
     }
   }

@@ -126,6 +126,25 @@ g_of_d2(typename std::conditional<MODE == BPIMD_FP64, double, float>::type d2, d
   }
 }
 
+// An upper bound of g's exponent from the squared distance, in float32 (cxf =
+// (float)cx; the product's relative error is below 2^-21): what is already
+// negligible by it needs no power of two.  NaN (no bound: compares false) where
+// the distance is not finite or its product overflows.
+template <typename T>
+__device__ __forceinline__ float g_below(T d2, float cxf) {  // -exponent(g) >= floor of this
+  float f;
+  if constexpr (sizeof(T) == 4) {
+    f = d2;
+  } else {  // truncated to float32 by integer instructions; past 2^96 no bound is needed
+    const long long b = __double_as_longlong(d2);
+    const int ex = (int)(b >> 52) - 896;
+    f = ex <= 0 ? 0.0f : (ex > 223 ? (ex >= 1151 ? __int_as_float(0x7fffffff) : 1e28f)
+                                   : __int_as_float((ex << 23) | (int)((b >> 29) & 0x7FFFFF)));
+  }
+  const float x = f * cxf;
+  return x <= 3e38f ? (x > 5e8f ? 5e8f : x) * 0.999999f : __int_as_float(0x7fffffff);
+}
+
 // g(a, b) from the endpoint b (bead P) and a (bead 1).
 template <int MODE, bool PBC>
 __device__ __forceinline__ typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type

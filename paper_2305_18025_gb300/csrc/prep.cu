@@ -33,8 +33,8 @@
 namespace bpimd {
 namespace {
 
-constexpr int BEAD_WARPS = BEAD_BLOCK_PARTICLES;  // particles per block (one warp each)
-static_assert(32 * BEAD_WARPS == 256, "bead-pass and pair-factor blocks share one launch shape");
+constexpr int BEAD_WARPS = 8;
+static_assert(BEAD_BLOCK_PARTICLES == BEAD_WARPS, "single systems: one warp a particle");
 
 // Non-finite test on the exponent bits (integer instructions only).
 __device__ __forceinline__ bool finite_bits(double x) {
@@ -100,19 +100,26 @@ __device__ __forceinline__ void bead_springs(const Workspace &w, const double *_
   }
 }
 
-// Particles l0 .. l0+7 of one system (all threads of the block).  MIXED:
-// the float32 bead pass of both mixed forms.
-template <bool MIXED>
+// Particles l0 .. l0 + 8 PER - 1 of one system (all threads of the block; PER
+// particles a warp).  MIXED: the float32 bead pass of both mixed forms.
+// Phase 2 is a chain of ~120 float64 instructions, each of which keeps a
+// sub-partition's float64 pipe for ~75 cycles whatever the number of lanes: a
+// single system takes eight particles a block (one block an SM, short phase 1),
+// a batch 32, so that the pipe runs full warps, and the blocks' phase 2 warps
+// (`warp2`) lie on all four sub-partitions.
+template <bool MIXED, int PER>
 __device__ __forceinline__ void bead_pass_body(const Workspace &w, const double *__restrict__ pos,
-                                               double *__restrict__ F, int l0) {
-  __shared__ double eint_s[BEAD_WARPS];
-  __shared__ int finite_s[BEAD_WARPS];
+                                               double *__restrict__ F, int l0, int warp2) {
+  constexpr int COUNT = BEAD_WARPS * PER;
+  __shared__ double eint_s[COUNT];
+  __shared__ int finite_s[COUNT];
   __shared__ __align__(16) double stage_s[BEAD_WARPS][STAGE_DOUBLES];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int P = w.P;
   // phase 1: one warp per particle -- interior springs and interior forces
-  {
-    const int l = l0 + wp;
+#pragma unroll 1
+  for (int h = 0; h < PER; ++h) {
+    const int slot = wp * PER + h, l = l0 + slot;
     bool finite = true;
     double s64 = 0.0;
     float s32 = 0.0f;
@@ -131,14 +138,14 @@ __device__ __forceinline__ void bead_pass_body(const Workspace &w, const double 
     }
     finite = __all_sync(0xffffffffu, finite);
     if (lane == 0) {
-      eint_s[wp] = w.half_k * (MIXED ? (double)s32 : s64);
-      finite_s[wp] = finite;
+      eint_s[slot] = w.half_k * (MIXED ? (double)s32 : s64);
+      finite_s[slot] = finite;
     }
   }
   __syncthreads();
   // phase 2: one lane per particle -- links, endpoint copies and the
   // coefficient c (the float64 transcendentals run once per 8 particles)
-  if (wp == 0 && lane < BEAD_WARPS) {
+  if (wp == warp2 && lane < COUNT) {
     const int l = l0 + lane;
     if (l < w.N) {
       if (!finite_s[lane]) atomicOr(w.status, ST_NONFINITE);
@@ -352,7 +359,7 @@ __global__ void __launch_bounds__(256) prep_kernel(Workspace w, const double *__
   if (MODE != BPIMD_MIXED32) pairg::table_init(T63);  // published by gmat_block's first barrier
   pdl_wait();
   if ((int)blockIdx.x < nbead) {
-    bead_pass_body<MODE != BPIMD_FP64>(w, pos, F, blockIdx.x * BEAD_WARPS);
+    bead_pass_body<MODE != BPIMD_FP64, 1>(w, pos, F, blockIdx.x * BEAD_WARPS, 0);
   } else {
     for (int blk = blockIdx.x - nbead; blk < w.NB; blk += gridDim.x - nbead) {
       if (w.pbc) gmat_block<MODE, true>(w, pos, blk, Tm, Te, E, T63);
@@ -380,7 +387,8 @@ __global__ void __launch_bounds__(256) prep_batched(const Workspace *__restrict_
   pdl_wait();
   if ((int)blockIdx.x < nbead) {
     const int2 e = bead_tab[blockIdx.x];
-    bead_pass_body<MODE != BPIMD_FP64>(ws[e.x], pos + off[e.x], F + off[e.x], e.y);
+    bead_pass_body<MODE != BPIMD_FP64, BATCH_BEAD_PARTICLES / BEAD_WARPS>(ws[e.x], pos + off[e.x], F + off[e.x], e.y,
+                                                                          blockIdx.x & 7);
   } else {
     for (int k = blockIdx.x - nbead; k < nblk; k += gridDim.x - nbead) {
       const int2 e = blk_tab[k];

@@ -266,6 +266,31 @@ __device__ __forceinline__ void gauss_fixed(long long X, long long Y, long long 
 // Lennard-Jones 4 eps ((sig/r)^12 - (sig/r)^6) truncated and shifted at rc; in a
 // periodic box (PBC) pair distances by minimum image.  MIXED: pair terms in
 // float32, accumulated per lane in float32.
+// Two float32 numbers in one 64-bit register: one instruction issued for two
+// IEEE operations (rounded as the scalar ones).
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 pack2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(F2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 __device__ __forceinline__ int max_high(const double *r) {
   return max(__double2hiint(r[0]) & 0x7fffffff, max(__double2hiint(r[1]) & 0x7fffffff, __double2hiint(r[2]) & 0x7fffffff));
 }
@@ -348,6 +373,32 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
             }
             continue;
           }
+        }
+      }
+      if constexpr (MIXED && !PBC) {
+        if (pp.pair == BPIMD_PAIR_GAUSSIAN) {
+          // the two particles in the halves of packed float32 instructions
+          const F2 X = pack2(px[0], px[1]), Y = pack2(py[0], py[1]), Z = pack2(pz[0], pz[1]), A = pack2(a, a),
+                   K = pack2(1.44269504f, 1.44269504f);
+          F2 FX = pack2(fx[0], fx[1]), FY = pack2(fy[0], fy[1]), FZ = pack2(fz[0], fz[1]), U = pack2(u[0], u[1]);
+#pragma unroll 4
+          for (int q = sub; q < cnt; q += SPLIT) {
+            const R4 t = sr[q];
+            const F2 dx = add2(X, pack2(-t.x, -t.x)), dy = add2(Y, pack2(-t.y, -t.y)), dz = add2(Z, pack2(-t.z, -t.z));
+            const F2 d2 = fma2(dz, dz, fma2(dx, dx, mul2(dy, dy)));  // the rounding of dx dx + dy dy + dz dz
+            float e0, e1;
+            unpack2(mul2(mul2(A, d2), K), e0, e1);
+            const F2 e = pack2(pairg::ex2_approx(e0), pairg::ex2_approx(e1));  // e^(a d2) = 2^(a d2 log2 e)
+            FX = fma2(e, dx, FX);
+            FY = fma2(e, dy, FY);
+            FZ = fma2(e, dz, FZ);
+            U = add2(U, e);
+          }
+          unpack2(FX, fx[0], fx[1]);
+          unpack2(FY, fy[0], fy[1]);
+          unpack2(FZ, fz[0], fz[1]);
+          unpack2(U, u[0], u[1]);
+          continue;
         }
       }
       if (pp.pair == BPIMD_PAIR_GAUSSIAN) {

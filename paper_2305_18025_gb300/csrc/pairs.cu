@@ -140,13 +140,14 @@ __global__ void __launch_bounds__(256) cl_gather(const int *__restrict__ list, l
 }
 
 // One thread per slot of the cell-ordered bead list: neighbouring threads work
-// on the same or adjacent cells, whose coordinates they share in cache.  Of the
-// ~9 candidates for each partner inside rc, a float32 test of the fixed-point
+// on the same or adjacent cells, whose coordinates they share in cache.  One
+// candidate in nine lies inside rc, and some lane takes the pair's branch for
+// nearly every candidate.  Float64: a float32 test of the fixed-point
 // coordinates keeps the near ones in a list of the thread's own (in shared
-// memory, in order), which is worked off when it is full and at the end: with
-// the pair's arithmetic behind a branch in the candidate loop, some lane took it
-// for nearly every candidate (136 us a pass at N = 4000, P = 64 mixed; float64
-// spent ~30 instructions of its ~75-cycle pipe on each candidate).
+// memory, in order), worked off when it is full and at the end; each candidate
+// cost ~30 instructions of the ~75-cycle float64 pipe before (N = 2048, P = 64:
+// 8449 -> 2281 us for four force passes).  Mixed pairs are cheap enough to stay
+// behind the branch (136 us a pass at N = 4000, P = 64; by lists 170).
 constexpr int CL_LIST = 32;  // near candidates held a thread
 
 template <bool MIXED>
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(CL_THREADS) cl_force(long long nb, int P, Pair
                                                        double *__restrict__ Fx, double *ubar_part) {
   using R = typename std::conditional<MIXED, float, double>::type;
   __shared__ double red[CL_THREADS / 32];
-  __shared__ int near[CL_LIST][CL_THREADS];
+  __shared__ int near[MIXED ? 1 : CL_LIST][CL_THREADS];
   const long long slot = blockIdx.x * (long long)CL_THREADS + threadIdx.x;
   const bool valid = slot < nb;
   R fx = 0, fy = 0, fz = 0, u = 0;
@@ -173,35 +174,27 @@ __global__ void __launch_bounds__(CL_THREADS) cl_force(long long nb, int P, Pair
     const int cell = cellof[b] - j * nc * nc * nc;
     const int cx = cell % nc, cy = (cell / nc) % nc, cz = cell / (nc * nc);
     const R sig2 = (R)pp.sig2, rc2 = (R)pp.rc2;
-    const float rc2f = (float)pp.rc2, keep2 = MIXED ? rc2f : rc2f * 1.00001f;  // float64: the test's own rounding aside
+    const float rc2f = (float)pp.rc2, keep2 = rc2f * 1.00001f;  // the float32 test's own rounding aside
     const uint4 ui = sfix[slot];
     double4 di = make_double4(0, 0, 0, 0);
     if (!MIXED) di = ((const double4 *)sorted)[slot];
+    auto pair = [&](R ex, R ey, R ez, R r2) {
+      const R s2 = sig2 / r2, s6 = s2 * s2 * s2;
+      const R c = (2 * s6 * s6 - s6) / r2;
+      fx += c * ex; fy += c * ey; fz += c * ez;
+      u += s6 * s6 - s6;
+      ++nin;
+    };
     int held = 0;
-    auto work_off = [&] {
+    auto work_off = [&] {  // float64
       for (int k = 0; k < held; ++k) {
-        const int q = near[k][threadIdx.x];
-        R ex, ey, ez;
-        if (MIXED) {
-          const uint4 uj = sfix[q];
-          ex = (R)fixdiff(ui.x, uj.x, pp.Lscale);
-          ey = (R)fixdiff(ui.y, uj.y, pp.Lscale);
-          ez = (R)fixdiff(ui.z, uj.z, pp.Lscale);
-        } else {
-          const double4 dj = ((const double4 *)sorted)[q];
-          ex = (R)(di.x - dj.x); ey = (R)(di.y - dj.y); ez = (R)(di.z - dj.z);
-          ex -= (R)(pp.L * rint((double)ex * pp.invL));
-          ey -= (R)(pp.L * rint((double)ey * pp.invL));
-          ez -= (R)(pp.L * rint((double)ez * pp.invL));
-        }
+        const double4 dj = ((const double4 *)sorted)[near[k][threadIdx.x]];
+        R ex = (R)(di.x - dj.x), ey = (R)(di.y - dj.y), ez = (R)(di.z - dj.z);
+        ex -= (R)(pp.L * rint((double)ex * pp.invL));
+        ey -= (R)(pp.L * rint((double)ey * pp.invL));
+        ez -= (R)(pp.L * rint((double)ez * pp.invL));
         const R r2 = ex * ex + ey * ey + ez * ez;
-        if (MIXED || (r2 > (R)0 && r2 < rc2)) {
-          const R s2 = sig2 / r2, s6 = s2 * s2 * s2;
-          const R c = (2 * s6 * s6 - s6) / r2;
-          fx += c * ex; fy += c * ey; fz += c * ez;
-          u += s6 * s6 - s6;
-          ++nin;
-        }
+        if (r2 > (R)0 && r2 < rc2) pair(ex, ey, ez, r2);
       }
       held = 0;
     };
@@ -216,13 +209,15 @@ __global__ void __launch_bounds__(CL_THREADS) cl_force(long long nb, int P, Pair
             const float ex = fixdiff(ui.x, uj.x, pp.Lscale), ey = fixdiff(ui.y, uj.y, pp.Lscale),
                         ez = fixdiff(ui.z, uj.z, pp.Lscale);
             const float r2 = ex * ex + ey * ey + ez * ez;
-            if (q != slot && (MIXED ? r2 > 0.0f && r2 < keep2 : r2 < keep2)) {
+            if constexpr (MIXED) {
+              if (q != slot && r2 > 0.0f && r2 < rc2f) pair(ex, ey, ez, r2);
+            } else if (q != slot && r2 < keep2) {
               near[held++][threadIdx.x] = q;
               if (held == CL_LIST) work_off();
             }
           }
         }
-    work_off();
+    if (!MIXED) work_off();
   }
   double ul = 0.0;
   if (valid) {

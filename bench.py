@@ -39,8 +39,8 @@ sys.path.insert(0, ROOT)
 
 METRIC = "exchange V_B+force evals/s at N=1024,P=32 (mixed vs FP64 GPU); MD steps/s"
 N_DEF, P_DEF, BETA_DEF, SEED_DEF = 1024, 32, 1.0, 3
-LAUNCHES_PER_EVAL = 4          # bead pass + pair factors, tile inverses, recursions (2 clusters), probabilities + forces
-BATCH_LAUNCHES_PER_EVAL = 3    # replica batch: bead pass + pair factors, recursions, probabilities + forces
+LAUNCHES_PER_EVAL = 4          # bead pass + pair factors, panel inverses, recursions (2 clusters), exterior forces
+BATCH_LAUNCHES_PER_EVAL = 3    # replica batch: bead pass + pair factors, recursions, exterior forces
 BATCH_MD = dict(dt=0.01, gamma=1.0, omega0=1.0, gaussian=(1.0, 0.5), seed=77)  # 256-replica workload
 DFMA_LATENCY_CYCLES = 64       # measured on GB300: dependent float64 FMA latency
 FLUSH_BYTES = 256 << 20        # > 129 MB L2
@@ -207,17 +207,17 @@ def roofline(stage_ms_per_eval, args, sm_mhz, peaks, precision="mixed"):
 
 # Counted per-pair work of the O(N^2) stages (thread-level operations of the
 # kernels as written; the counts are listed with the kernels' rooflines):
-#   probability pass, float64: 13 float64 ops per pair (bead differences,
-#     Pr = alpha mu g, row and column terms) + 20 float64 adds of the column
-#     butterfly (4 sums x 5 levels, every lane) = 33 float64 ops;
-#   probability pass, mixed: 2 64 x 64-bit high products (alpha mu, then g)
-#     = 8 integer 32 x 32 -> 64 multiply-adds per pair;
-#   probability pass, mixed32: float32 only (12 ops per pair + 20 butterfly adds);
+#   exterior forces (every pair formed twice, for its row and its column),
+#     float64: 3 float64 differences each = 6 float64 ops per pair (the
+#     products and sums are on the integer pipe);
+#   mixed forms: float32 pairs -- 9 operations for the differences, 10 for the
+#     weight, 33 for three compensated products and sums, twice = 104 float32
+#     ops per pair, and 2 integer multiply-adds of addresses;
 #   pair factors, float64: 6 float64 ops per pair (difference and square);
-#   pair factors, mixed: the 128-bit product and 6 64-bit high products of
-#     the integer power (pow2_fixed.cuh) = 28 integer multiply-adds.
-PROB_F64_OPS, PROB_MIXED_IMADS, PROB_M32_F32OPS = 33, 8, 32
-G_F64_OPS, G_MIXED_IMADS = 6, 28
+#   pair factors, mixed: the integer power's products (pow2_fixed.cuh)
+#     = 19 integer multiply-adds.
+PROB_F64_OPS, PROB_MIXED_IMADS, PROB_M32_F32OPS = 6, 2, 104
+G_F64_OPS, G_MIXED_IMADS = 6, 19
 
 
 def measure_unit_peaks(dev, stream, iters=2000):
@@ -260,14 +260,15 @@ def roofline_stages(stage_ms_per_eval, args, sm_mhz, peaks, unit_peaks, precisio
     rec["achieved"] = N / t_rec
     rec["frac"] = rec["achieved"] / rec["peak"]
     rec.update(step_latency(t_rec, N, (sm_mhz or peaks.get("sm_max_mhz", 2070.0)) * 1e6))
+    fp32_peak = (sm_mhz or peaks.get("sm_max_mhz", 2070.0)) * 1e6 * 152 * 128
     if precision == "fp64":
         prob = {"bound": "fp64", "unit": "float64 ops/s", "achieved": PROB_F64_OPS * pairs / t_prob,
                 "peak": unit_peaks["fp64_fma_per_s"], "peak_source": "library float64 FMA probe (measured)"}
     elif precision == "mixed":
         prob = {"bound": "int", "unit": "32-bit integer multiply-adds/s", "achieved": PROB_MIXED_IMADS * pairs / t_prob,
                 "peak": unit_peaks["int_mad_per_s"], "peak_source": "library integer multiply-add probe (measured)"}
+        prob["fp32_frac"] = PROB_M32_F32OPS * pairs / t_prob / fp32_peak
     else:
-        fp32_peak = (sm_mhz or peaks.get("sm_max_mhz", 2070.0)) * 1e6 * 152 * 128
         prob = {"bound": "fp32", "unit": "float32 ops/s", "achieved": PROB_M32_F32OPS * pairs / t_prob,
                 "peak": fp32_peak, "peak_source": "nominal 128 float32 lanes per SM x 152 SMs x sampled clock"}
     prob["frac"] = prob["achieved"] / prob["peak"]
@@ -493,7 +494,7 @@ def md_throughput(args, pos_np, wP, dev, max_over_ranks, barrier, world):
         en = md.step(x, v, 1).cpu().tolist()
         md.close()
         out[prec] = {"value": aggregate_rate(world, steps, ms * 1e-3), "unit": "MD steps/s", "steps": steps,
-                     "gpu_launches": (LAUNCHES_PER_EVAL + 3) * steps + LAUNCHES_PER_EVAL + 1,
+                     "gpu_launches": (LAUNCHES_PER_EVAL + 2) * (steps + 1),
                      "ms_per_step": ms / steps, "energies_after": dict(zip(["V_B", "U_bar", "kinetic", "E_prim"], en))}
     out["config"] = {"workload": f"trapped bosons N={args.N} P={args.P} beta={args.beta:g}, harmonic trap w0=1, "
                                  "Gaussian repulsion g=3 s=0.5 between equal-index beads",
@@ -559,7 +560,7 @@ def batched_md_throughput(args, dev, reps, wPs, max_over_ranks, barrier, world):
     """BAOAB molecular dynamics of the whole replica batch: harmonic trap w0 = 1
     and Gaussian repulsion g = 1, s = 0.5 between equal-index beads, each
     replica thermostatted at its own beta; the steps are CUDA-graph replays on
-    a dedicated stream (batch evaluation, pair forces, integrator: 6 launches
+    a dedicated stream (batch evaluation, pair forces, integrator: 5 launches
     per step), with the pair tile (lanes per particle) picked by the
     autotuner on scratch copies first.  Back to back as in a trajectory, so
     the L2 is not flushed."""
@@ -590,7 +591,7 @@ def batched_md_throughput(args, dev, reps, wPs, max_over_ranks, barrier, world):
         eng.close()
         out[prec] = {"value": aggregate_rate(world, steps, ms * 1e-3), "unit": "batch MD steps/s", "steps": steps,
                      "replica_steps_per_s": aggregate_rate(world, steps * len(reps), ms * 1e-3),
-                     "ms_per_step": ms / steps, "gpu_launches": (BATCH_LAUNCHES_PER_EVAL + 3) * steps,
+                     "ms_per_step": ms / steps, "gpu_launches": (BATCH_LAUNCHES_PER_EVAL + 2) * (steps + 1),
                      "finite": bool(np.isfinite(en).all()),
                      "tuning": {"pair_tile_lanes": int(tuned["choice"]), "cached": tuned["cached"],
                                 "timings_ms": tuned["timings_ms"]},

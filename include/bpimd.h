@@ -78,30 +78,29 @@ extern "C" {
  *   distances and forces; pair Boltzmann factors g = 2^(-x) of the exact
  *   float64 product x by a 64-bit fixed-point table method (integer pipe,
  *   2^-60 relative before the final float64 rounding); the blocked recursions
- *   (tile inverses, the lead's tile products and the bulk sums) on 64-bit
- *   integer mantissas with int32 exponents (truncation 2^-61 per operation);
- *   float64 probabilities and force sums.
+ *   (panel inverses, panel products and the sums over earlier sources) on
+ *   64-bit integer mantissas with int32 exponents (truncation 2^-60 per
+ *   operation); exterior forces from float64 differences by 64-bit integer
+ *   products and sums (2^-57 of the largest term of a group of four); float64
+ *   direct links and results.
  * BPIMD_MIXED: float32 bead differences, per-particle spring energies (float32
  *   warp sums) and closing-spring distances; everything after them at float64
  *   accuracy or better: the link coefficients and the prefix sums of spring
  *   energies in float64, g = 2^(-x) of the exact product of the float32
  *   closing-spring term and the float64 constant beta k/2 log2(e) by the same
  *   integer table method, the recursions on 64-bit integer mantissas as in
- *   BPIMD_FP64, probabilities Pr = alpha mu g from 64-bit integer
- *   mantissa products, and the probability and force sums as unevaluated
- *   sums of two float32 numbers (compensated: 2^-46 relative) over float32
- *   bead differences.
- * BPIMD_MIXED32: the fastest form: float32 bead differences and spring
- *   energies, g from the float32 hardware exponential (ex2.approx), the
- *   recursions' bulk sums as float32 products over 8 sources, the tile
- *   inverses and the lead's tile products on 64-bit integer mantissas,
- *   float32 probabilities and block-local force sums (combined across blocks
- *   with float32 TwoSum compensation); float64 prefix sums, link coefficients,
- *   and outputs.
+ *   BPIMD_FP64, and the exterior forces' weights, products with the float32
+ *   bead differences and sums as unevaluated sums of two float32 numbers
+ *   (compensated: 2^-46 relative).
+ * BPIMD_MIXED32: float32 bead differences and spring energies, g from the
+ *   float32 hardware exponential (ex2.approx); everything after it as
+ *   BPIMD_MIXED.
  * Replica batches (bpimd_create_batched) run each recursion of a replica of
  * up to 4096 particles on one CTA as 32 dependent steps per tile, in the same
  * formats, except that BPIMD_MIXED32 multiplies there by the top 32 bits of
- * the 64-bit factor mantissa (truncation 2^-30 per step).
+ * the 64-bit factor mantissa (truncation 2^-30 per step) and takes its sums
+ * over earlier tiles in float32.  Single BPIMD_FP64 and BPIMD_MIXED systems of
+ * up to 128 particles take that one-CTA form too.
  * All three meet the mixed tolerances (1e-6 relative on V_B, 1e-5 RMS on
  * forces); BPIMD_FP64 meets 1e-12 / 1e-10. */
 #define BPIMD_FP64 0
@@ -113,13 +112,10 @@ extern "C" {
 #define BPIMD_MAX_N 16384
 /* Up to this N a context tabulates the pair Boltzmann factors g(u, v) of the
  * closing springs once per evaluation (two coalesced copies, O(N^2) device
- * memory: 12 or 16 bytes per pair and copy, ~0.8 GB at N = 8192) and the
- * probability pass keeps O(N^2 / 32) block partial sums.  Above it -- or at
- * any N when cfg.flags has BPIMD_FLAG_RECOMPUTE -- nothing O(N^2) is stored:
- * the recursions and the probability pass recompute each g where they use it
- * (the same bits), and the probability pass forms every pair twice, once for
- * its row and once for its column, so that each force sum is completed by one
- * CTA.  Device memory is then O(N + N P). */
+ * memory: 12 or 8 bytes per pair and copy, ~0.8 GB at N = 8192).  Above it --
+ * or at any N when cfg.flags has BPIMD_FLAG_RECOMPUTE -- nothing O(N^2) is
+ * stored: the recursions and the exterior forces recompute each g where they
+ * use it (the same bits).  Device memory is then O(N + N P). */
 #define BPIMD_STORE_MAX_N 8192
 #define BPIMD_FLAG_RECOMPUTE 1
 /* Test hook of the error path (bpimd_create only): the forward recursion's
@@ -340,7 +336,7 @@ int bpimd_profile_end(bpimd_ctx *ctx, double *stage_ms, int *n_evals);
  * caller, cuda_stream is a cudaStream_t (NULL = default stream) that must
  * belong to the current device (a stream of another device returns
  * BPIMD_ERR_ARG: the scratch array used is the current device's).  It allocates
- * nothing: its scratch memory is one file-scope __device__ array of 1 MiB per
+ * nothing: its scratch memory is one file-scope __device__ array of 2 MiB per
  * device, which bounds the size to N <= BPIMD_NOALLOC_MAX_N (larger N returns
  * BPIMD_ERR_SIZE before any work is enqueued).
  *   - The first call on a device, with that device current, looks up the

@@ -67,7 +67,7 @@ int read_status(bpimd_ctx *ctx) {
 namespace bpimd {
 
 size_t layout_workspace(Workspace &w, char *base) {
-  const size_t N = w.N, NB = w.NB, NT = w.NT, gelems = NB * TILE2;
+  const size_t N = w.N, NB = w.NB, gelems = NB * TILE2;
   const size_t gm_bytes = (w.mixed ? sizeof(float) : sizeof(double)) * gelems;
   const bool tables = !w.recomp;  // recompute mode: nothing O(N^2)
   size_t off = 0;
@@ -208,6 +208,7 @@ int bpimd_create(bpimd_ctx **out, const bpimd_config *cfg, void *cuda_stream) {
   w.recomp = (cfg->flags & BPIMD_FLAG_RECOMPUTE) || cfg->N > BPIMD_STORE_MAX_N;
   w.test_timeout = (cfg->flags & BPIMD_FLAG_TEST_TIMEOUT) != 0;
   w.blocks = 1;
+  w.gstr = w.N > CHAIN_SMALL_N ? 4 : 32;
   set_box(w, cfg->box_L);
   const size_t N = w.N;
   // one allocation: the workspace, then the diagnostic potentials

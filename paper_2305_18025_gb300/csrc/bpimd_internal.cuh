@@ -136,6 +136,7 @@ struct Workspace {
   double m, omega_P, beta, k, half_k;
   double inv_P;         // 1/P (kernels take it from here: a float64 division costs a GB300 SM ~20 warp-cycles per lane)
   double cx;            // beta (1/2) k log2(e): g = 2^(-cx d^2)
+  int gstr;             // source stride of the pair-factor tables (below)
   int recomp;           // recompute mode: no O(N^2) table; g is formed where it is used
   int test_timeout;     // BPIMD_FLAG_TEST_TIMEOUT: the forward lead waits for a hand-off never made
   // periodic cubic box of side L (0: open boundaries); every spring joins the
@@ -155,12 +156,18 @@ struct Workspace {
   int *nexp;            // [N] n_i = integer part of beta link_i log2(e) (in c_{i+1}'s exponent)
   double *Ap;           // [N] E_int_i + (beta link_i log2(e) - n_i) ln2 / beta
   double *C;            // [N+1] reduced prefix sums C'[v] = sum_{i<v} Ap[i] (0-based i)
-  // g matrix, tile-packed triangle: block (t, s), s <= t, at (t(t+1)/2 + s) * TILE2,
-  // entry [i][j] = g for a = s*TILE + i (bead 1 particle), b = t*TILE + j (bead P particle)
+  // g matrix: row tile t (32 particles b, bead P) of every source a < 32 (t + 1)
+  // (bead 1) at t(t+1)/2 * TILE2, entry (a, b) at gbase(b) + gstr a.  gstr = 32:
+  // a source's 32 rows lie together (a lane a row: replicas, small systems).
+  // gstr = 4: four rows by all sources (the recursion clusters, whose CTAs own
+  // four rows of a panel: eight sources of them are 256 contiguous bytes, where
+  // the other order gives eight pieces of 32: recursions of N = 1024 42.1 ->
+  // 38.8 us, N = 1601 70.6 -> 61.7, N = 4096 200 -> 177, at 0-7 % more in the
+  // preparation and the exterior pass, which go along rows).
   void *gm;             // double (FP64) or float (MIXED) mantissas
   int *ge;              // exponents
   // the same factors in the backward recursion's coordinates (rows r = N-1-a,
-  // sources w = N-1-b), same tile-packed layout, so that both recursions read
+  // sources w = N-1-b), same layout, so that both recursions read
   // their blocks with coalesced loads
   void *gbm;
   int *gbe;
@@ -250,6 +257,21 @@ inline void set_box(Workspace &w, double L) {
   w.invL32 = w.invL * 4294967296.0;
   w.Lscale = (float)(w.L / 4294967296.0);
   w.pbc = L > 0.0 ? 1 : 0;
+}
+
+// Source stride of the pair-factor tables: GS where a kernel knows it (the
+// replica kernels: 32; 256 replicas 466 us, 485 with the stride read from the
+// workspace), 0: the workspace's.
+template <int GS = 0>
+__device__ __forceinline__ int gstride(const Workspace &w) {
+  return GS ? GS : w.gstr;
+}
+// Start of row `row` of a pair-factor table (entry of source a: + gstr a).
+template <int GS = 0>
+__device__ __forceinline__ size_t gbase(const Workspace &w, int row) {
+  const int t = row >> 5;
+  const size_t tile = (size_t)(t * (t + 1) / 2) << 10;
+  return tile + (gstride<GS>(w) == 4 ? (((row >> 2) & 7) * (t + 1) << 7) + (row & 3) : row & 31);
 }
 
 // Lay the workspace out from `base` (nullptr: only measure); returns the bytes

@@ -129,7 +129,7 @@ __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *
         if (T >= NT) break;
         const int r = T * TILE + lane;
         const int ra = r < N ? r : 0;
-        RowFactors<MODE, BWD, RC, PBC> f;  // rows past N: their tile's padding, or particle 0's (sums not kept)
+        RowFactors<MODE, BWD, RC, PBC, 32> f;  // rows past N: their tile's padding, or particle 0's (sums not kept)
         f.load(w, RC ? ra : r);
         auto load = [&](int src, M_t &m, int &e) { f.h(w, min(src, RC && r >= N ? 0 : src), sm.T63, m, e); };
         if constexpr (MIXED) {

@@ -12,12 +12,6 @@ namespace chain_detail {
 
 constexpr int BLK = 32 * 33;  // padded 32 x 32 block in shared memory
 
-// index of H(src, row) in the tile-packed pair-factor layout
-__device__ __forceinline__ size_t hidx(int src, int row) {
-  const int t = row >> 5, s = src >> 5;
-  return ((size_t)(t * (t + 1) / 2 + s) << 10) + ((src & 31) << 5) + (row & 31);
-}
-
 // x * 2^k for k <= 0 by integer arithmetic on the exponent field (x >= 0 normal
 // or zero); 0 when the result would leave the normal range.
 __device__ __forceinline__ double scale_nonpos(double x, int k) {
@@ -237,21 +231,21 @@ struct RowEnds {
 
 // Row r's pair factors H(src, r) as stored, or recomputed from the endpoint
 // copies (bit-identical), as c_r H in the K format.
-template <int MODE, bool BWD, bool RC, bool PBC>
+template <int MODE, bool BWD, bool RC, bool PBC, int GS = 0>
 struct RowFactors {
   using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
   RowEnds<MODE, BWD, PBC> re;
-  size_t base;  // H(src, row) is at base + 32 src (a tile's blocks lie one after the other)
+  size_t base;  // H(src, row) is at base + gstr src
   __device__ __forceinline__ void load(const Workspace &w, int row) {
     if (RC) re.load(w, row);
-    else base = hidx(0, row);
+    else base = gbase<GS>(w, row);
   }
   __device__ __forceinline__ void h(const Workspace &w, int src, const unsigned long long *T63, M_t &m,
                                     int &e) const {
     if constexpr (RC) {
       m = re.h(w, src, T63, e);
     } else {
-      const size_t gi = base + 32 * src;
+      const size_t gi = base + gstride<GS>(w) * src;
       m = __ldg((const M_t *)chain_gm<BWD>(w) + gi);
       e = __ldg(chain_ge<BWD>(w) + gi);
     }
@@ -277,7 +271,7 @@ __device__ __forceinline__ void stage_offdiag(const Workspace &w, int tt, int i0
   const int lane = threadIdx.x & 31;
   const int srcbase = tt * TILE, row = tt * TILE + TILE + lane;
   M_t *dm = (M_t *)dmv;
-  RowFactors<MODE, BWD, RC, PBC> f;
+  RowFactors<MODE, BWD, RC, PBC, 32> f;
   f.load(w, min(row, w.N - 1));
 #pragma unroll
   for (int i = i0; i < i0 + NR; ++i) {
@@ -299,7 +293,7 @@ __device__ __forceinline__ void stage_diag(const Workspace &w, int tt, int i0, u
   const int lane = threadIdx.x & 31;
   const int r0 = tt * TILE, row = r0 + lane;
   const xd c = (row < w.N) ? xnorm_int(chain_coef<BWD>(w, row)) : xd{1.0, 0};
-  RowFactors<MODE, BWD, RC, PBC> f;
+  RowFactors<MODE, BWD, RC, PBC, 32> f;
   f.load(w, min(row, w.N - 1));
 #pragma unroll
   for (int i = i0; i < i0 + NR; ++i) {

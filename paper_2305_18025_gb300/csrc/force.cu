@@ -244,7 +244,7 @@ __device__ __forceinline__ pairg::EndPt<!F64, PBC> staged_end(const Partners<F64
 }
 
 // One item (all threads of the cluster's CTAs; CTA `rank` of CL).
-template <int MODE, bool RC, bool PBC>
+template <int MODE, bool RC, bool PBC, int GS>
 __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int rank, int CL,
                                               const double *__restrict__ pos, double *__restrict__ F,
                                               const unsigned long long *T63, ProbSmem<MODE == BPIMD_FP64> &sm) {
@@ -262,10 +262,10 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
   const int p0 = row_item ? 0 : tile * TILE, p1 = row_item ? min(N, (tile + 1) * TILE) : N;
   // partners of a chunk: a multiple of 32, so that each warp takes whole groups of four
   const int ch = min(PROB_CHUNK, ((p1 - p0 + CL - 1) / CL + 31) & ~31), per = ch / PROB_WARPS;
-  // this lane's pair factors: g(partner q) at gi0 + 32 src, src = q in the
+  // this lane's pair factors: g(partner q) at gi0 + gstr src, src = q in the
   // forward copy, N-1-q in the backward one (clamped into the stored triangle)
   const int r = row_item ? tile * TILE + lane : N - 1 - mine_q;
-  const int gi0 = (((r >> 5) * ((r >> 5) + 1) / 2) << 10) + (r & 31);
+  const int gi0 = (int)gbase<GS>(w, r), gstr = gstride<GS>(w);
   const M_t *gm = (const M_t *)(row_item ? w.gm : w.gbm) + gi0;
   const int *ge = (row_item ? w.ge : w.gbe) + gi0;
   PSum A{{0, 0, 0}, NO_TERM};
@@ -280,8 +280,8 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
 #pragma unroll
       for (int k = 0; k < G; ++k) {
         const int qk = min(q + k, p1 - 1), src = row_item ? qk : N - 1 - max(qk, mine_q);
-        gmv[k] = __ldg(gm + 32 * src);
-        gev[k] = __ldg(ge + 32 * src);
+        gmv[k] = __ldg(gm + gstr * src);
+        gev[k] = __ldg(ge + gstr * src);
       }
     };
     if (!RC && q0 < q1) load_g(q0);
@@ -441,8 +441,8 @@ __global__ void __launch_bounds__(PROB_THREADS) exterior_kernel(Workspace w, con
   }
   pdl_wait();
   const int item = blockIdx.x / CL, rank = blockIdx.x % CL;
-  if (w.pbc) exterior_item<MODE, RC, true>(w, item, rank, CL, pos, F, T63, sm);
-  else exterior_item<MODE, RC, false>(w, item, rank, CL, pos, F, T63, sm);
+  if (w.pbc) exterior_item<MODE, RC, true, 0>(w, item, rank, CL, pos, F, T63, sm);
+  else exterior_item<MODE, RC, false, 0>(w, item, rank, CL, pos, F, T63, sm);
   pdl_trigger();
 }
 
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(PROB_THREADS) exterior_batched(const Workspace
   pdl_wait();
   for (int k = blockIdx.x; k < ntab; k += gridDim.x) {
     const int2 e = tab[k];
-    exterior_item<MODE, false, false>(ws[e.x], e.y, 0, 1, pos + off[e.x], F + off[e.x], nullptr, sm);
+    exterior_item<MODE, false, false, 32>(ws[e.x], e.y, 0, 1, pos + off[e.x], F + off[e.x], nullptr, sm);
     __syncthreads();  // the slots are read
   }
   pdl_trigger();
@@ -495,7 +495,7 @@ __device__ double spring_block(const Workspace &w, int blk, double *red) {
   for (int e = threadIdx.x; e < TILE2; e += blockDim.x) {
     const int a = s * TILE + (e >> 5), b = t * TILE + (e & 31);
     if (b < w.N && a <= b) {
-      const size_t gi = (size_t)blk * TILE2 + e;
+      const size_t gi = gbase(w, b) + w.gstr * a;
       const int r = w.N - 1 - b;
       int ex = w.yfe[a] + w.ybe[r] + inv_e;
       xd g{0.0, 0};
@@ -557,8 +557,7 @@ __global__ void dense_prob_kernel(Workspace w, double *M) {
     const int b = (int)(idx / w.N), a = (int)(idx % w.N);  // row l = b, column l' = a
     double v = 0.0;
     if (a <= b) {
-      const int t = b >> 5, s = a >> 5;
-      const size_t gi = ((size_t)(t * (t + 1) / 2 + s) << 10) + ((a & 31) << 5) + (b & 31);
+      const size_t gi = gbase(w, b) + w.gstr * a;
       const xd g = w.recomp ? pairg::g_runtime(w, a, b)
                             : xd{w.mixed ? (double)((const float *)w.gm)[gi] : ((const double *)w.gm)[gi], w.ge[gi]};
       const xd al = alpha_of(w, a), mu = mu_of(w, b);

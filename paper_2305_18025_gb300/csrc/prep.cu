@@ -288,21 +288,28 @@ __device__ __forceinline__ pairg::EndPt<MODE != BPIMD_FP64, PBC> staged_end(cons
 
 // One pass over the forward blocks (a = s*32+i, b = t*32+j): each valid pair
 // a <= b < N is evaluated once (pairg.cuh; the recompute mode forms the same
-// bits from the bead pass's copies) and stored in both copies -- the forward
-// one directly (coalesced along b), the backward one (row r = N-1-a, source
-// w = N-1-b) after a transpose through shared memory, so that those stores
-// are coalesced along r.  Entries outside a <= b < N are never written here
+// bits from the bead pass's copies) and stored in both copies, by rows b
+// (sources a) for the forward recursion and by rows r = N-1-a (sources N-1-b)
+// for the backward one.  Entries outside a <= b < N are never written here
 // (gmat_padding_kernel fills them once).  The pass is bound by issue slots (250
 // instructions a pair before its indices and endpoints were taken out of the
 // loops and the power of two trimmed).
-// One block of g (all threads of the CTA; Tm/Te: 32 x 33 shared tiles).
-template <int MODE, bool PBC>
+// One block of g (all threads of the CTA; Tm/Te: 32 rows of TPAD in shared
+// memory).  GS = 32: the forward copy is stored directly (coalesced along b),
+// the backward one after a transpose (coalesced along r).  GS = 4: both are
+// written after it, a warp's lanes four rows by eight sources, in pieces of 256
+// and 128 contiguous bytes: mixed N = 1024 59.8 -> 55.8 us an evaluation
+// against lanes along the rows, whose pieces are 32 bytes.  The kernel is held
+// to the registers that keep 6 CTAs an SM (5 in float64): with 8 more, mixed
+// N = 8192 takes 290 us for 283.
+constexpr int TPAD = 37;  // few bank conflicts in any of the patterns
+template <int MODE, bool PBC, int GS>
 __device__ __forceinline__ void gmat_block(const Workspace &w, const double *__restrict__ pos, int blk,
                                            typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type *Tm,
                                            int *Te, EndTiles &E, const unsigned long long *T63) {
   using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
   using EP = pairg::EndPt<MODE != BPIMD_FP64, PBC>;
-  const int N = w.N;
+  const int N = w.N, gstr = GS;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int t, s;
   block_coords(blk, t, s);
@@ -310,8 +317,9 @@ __device__ __forceinline__ void gmat_block(const Workspace &w, const double *__r
   {
     const int b = t * TILE + lane, last = b < N ? min(b - s * TILE, TILE - 1) : -1;  // valid: i <= last
     const EP rb = staged_end<MODE, PBC>(E, 0, lane);
-    M_t *gm = (M_t *)w.gm + (size_t)blk * TILE2 + lane;
-    int *ge = w.ge + (size_t)blk * TILE2 + lane;
+    const size_t idx = (size_t)blk * TILE2 + lane;
+    M_t *gm = (M_t *)w.gm + idx;
+    int *ge = w.ge + idx;
 #pragma unroll 1
     for (int k = 0; k < 4; ++k) {
       const int i = warp + 8 * k;
@@ -319,26 +327,48 @@ __device__ __forceinline__ void gmat_block(const Workspace &w, const double *__r
       if (i <= last) {
         int e;
         const M_t m = pairg::g_of<MODE, PBC>(w, rb, ra, w.cx, T63, e);
-        gm[i * TILE] = m;
-        ge[i * TILE] = e;
-        Tm[i * 33 + lane] = m;
-        Te[i * 33 + lane] = e;
+        if (gstr == TILE) {
+          gm[i * TILE] = m;
+          ge[i * TILE] = e;
+        }
+        Tm[i * TPAD + lane] = m;
+        Te[i * TPAD + lane] = e;
       }
     }
   }
   __syncthreads();
-  {
-    const int a = s * TILE + lane, r = N - 1 - a, T = r >> 5, src0 = N - 1 - t * TILE;
-    const int first = a - t * TILE, end = min(TILE, N - t * TILE);  // valid: first <= jj < end
-    const size_t idx = ((size_t)(T * (T + 1) / 2) << 10) + (r & 31);
+  const int end = min(TILE, N - t * TILE);  // rows of tile t
+  if (gstr == 4) {
+    // forward: rows 4 warp.. of tile t; backward: the particles l of tile s whose
+    // rows N-1-a are one group of four (they wrap round the tile)
+    const int j = 4 * warp + (lane & 3), b = t * TILE + j;
+    const int l = (4 * warp + ((N - 1) & 3) - (lane & 3)) & (TILE - 1), a = s * TILE + l;
+    const size_t fi = gbase<GS>(w, b) + 4 * s * TILE, bi = gbase<GS>(w, max(N - 1 - a, 0));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = 8 * k + (lane >> 2);  // source in tile s; partner in tile t
+      if (j < end && s * TILE + i <= b) {
+        ((M_t *)w.gm)[fi + 4 * i] = Tm[i * TPAD + j];
+        w.ge[fi + 4 * i] = Te[i * TPAD + j];
+      }
+      const int q = t * TILE + i;
+      if (i < end && a <= q) {
+        ((M_t *)w.gbm)[bi + 4 * (N - 1 - q)] = Tm[l * TPAD + i];
+        w.gbe[bi + 4 * (N - 1 - q)] = Te[l * TPAD + i];
+      }
+    }
+  } else {
+    const int a = s * TILE + lane, r = N - 1 - a, src0 = N - 1 - t * TILE;
+    const int first = a - t * TILE;  // valid: first <= jj < end
+    const size_t idx = gbase<32>(w, max(r, 0));
     M_t *gbm = (M_t *)w.gbm + idx;
     int *gbe = w.gbe + idx;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int jj = warp + 8 * k;
       if (jj >= first && jj < end) {
-        gbm[(src0 - jj) * TILE] = Tm[lane * 33 + jj];
-        gbe[(src0 - jj) * TILE] = Te[lane * 33 + jj];
+        gbm[(src0 - jj) * TILE] = Tm[lane * TPAD + jj];
+        gbe[(src0 - jj) * TILE] = Te[lane * TPAD + jj];
       }
     }
   }
@@ -348,12 +378,12 @@ __device__ __forceinline__ void gmat_block(const Workspace &w, const double *__r
 // One evaluation's preparation: blocks 0..nbead-1 run the bead pass (8
 // particles each), the others stride over the blocks of g.  MODE is the
 // precision form (BPIMD_FP64, BPIMD_MIXED, BPIMD_MIXED32).
-template <int MODE>
-__global__ void __launch_bounds__(256) prep_kernel(Workspace w, const double *__restrict__ pos,
+template <int MODE, int GS>
+__global__ void __launch_bounds__(256, MODE == BPIMD_FP64 || (MODE == BPIMD_MIXED32 && GS == 32) ? 5 : 6) prep_kernel(Workspace w, const double *__restrict__ pos,
                                                    double *__restrict__ F, int nbead) {
   using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
-  __shared__ M_t Tm[TILE * 33];
-  __shared__ int Te[TILE * 33];
+  __shared__ M_t Tm[TILE * TPAD];
+  __shared__ int Te[TILE * TPAD];
   __shared__ EndTiles E;
   __shared__ unsigned long long T63[256];
   if (MODE != BPIMD_MIXED32) pairg::table_init(T63);  // published by gmat_block's first barrier
@@ -362,8 +392,8 @@ __global__ void __launch_bounds__(256) prep_kernel(Workspace w, const double *__
     bead_pass_body<MODE != BPIMD_FP64, 1>(w, pos, F, blockIdx.x * BEAD_WARPS, 0);
   } else {
     for (int blk = blockIdx.x - nbead; blk < w.NB; blk += gridDim.x - nbead) {
-      if (w.pbc) gmat_block<MODE, true>(w, pos, blk, Tm, Te, E, T63);
-      else gmat_block<MODE, false>(w, pos, blk, Tm, Te, E, T63);
+      if (w.pbc) gmat_block<MODE, true, GS>(w, pos, blk, Tm, Te, E, T63);
+      else gmat_block<MODE, false, GS>(w, pos, blk, Tm, Te, E, T63);
     }
   }
   pdl_trigger();
@@ -379,8 +409,8 @@ __global__ void __launch_bounds__(256) prep_batched(const Workspace *__restrict_
                                                     const long long *__restrict__ off,
                                                     const double *__restrict__ pos, double *__restrict__ F) {
   using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
-  __shared__ M_t Tm[TILE * 33];
-  __shared__ int Te[TILE * 33];
+  __shared__ M_t Tm[TILE * TPAD];
+  __shared__ int Te[TILE * TPAD];
   __shared__ EndTiles E;
   __shared__ unsigned long long T63[256];
   if (MODE != BPIMD_MIXED32) pairg::table_init(T63);  // published by gmat_block's first barrier
@@ -392,8 +422,8 @@ __global__ void __launch_bounds__(256) prep_batched(const Workspace *__restrict_
   } else {
     for (int k = blockIdx.x - nbead; k < nblk; k += gridDim.x - nbead) {
       const int2 e = blk_tab[k];
-      if (ws[e.x].pbc) gmat_block<MODE, true>(ws[e.x], pos + off[e.x], e.y, Tm, Te, E, T63);
-      else gmat_block<MODE, false>(ws[e.x], pos + off[e.x], e.y, Tm, Te, E, T63);
+      if (ws[e.x].pbc) gmat_block<MODE, true, 32>(ws[e.x], pos + off[e.x], e.y, Tm, Te, E, T63);
+      else gmat_block<MODE, false, 32>(ws[e.x], pos + off[e.x], e.y, Tm, Te, E, T63);
     }
   }
   pdl_trigger();
@@ -411,7 +441,7 @@ __device__ __forceinline__ void gmat_padding_block(const Workspace &w, int blk) 
   for (int i = threadIdx.x >> 5; i < TILE; i += 8) {
     const int lo = s * TILE + i;
     if (col >= w.N || lo > col) {
-      const size_t idx = (size_t)blk * TILE2 + i * TILE + j;
+      const size_t idx = gbase(w, col) + w.gstr * lo;
       ((M_t *)w.gm)[idx] = (M_t)1.0;
       w.ge[idx] = XZERO_E;
       ((M_t *)w.gbm)[idx] = (M_t)1.0;
@@ -515,14 +545,20 @@ cudaError_t launch_diag_potentials(const Workspace &w, double *Vf, double *Vb, c
   return cudaGetLastError();
 }
 
+template <int MODE>
+cudaError_t prep_go(const Workspace &w, int grid, const double *pos, double *F, int nbead, cudaStream_t s) {
+  return w.gstr == 4 ? launch_pdl(prep_kernel<MODE, 4>, grid, 256, 0, s, w, pos, F, nbead)
+                     : launch_pdl(prep_kernel<MODE, 32>, grid, 256, 0, s, w, pos, F, nbead);
+}
+
 cudaError_t launch_prep(const Workspace &w, const double *pos, double *F, cudaStream_t s) {
   const int nbead = (w.N + BEAD_WARPS - 1) / BEAD_WARPS;
   const int cap = sm_count() * 8;
   const int grid = nbead + (w.recomp ? 0 : (w.NB < cap ? w.NB : cap));  // recompute mode: bead pass only
   switch (w.mode) {
-    case BPIMD_FP64: return launch_pdl(prep_kernel<BPIMD_FP64>, grid, 256, 0, s, w, pos, F, nbead);
-    case BPIMD_MIXED: return launch_pdl(prep_kernel<BPIMD_MIXED>, grid, 256, 0, s, w, pos, F, nbead);
-    default: return launch_pdl(prep_kernel<BPIMD_MIXED32>, grid, 256, 0, s, w, pos, F, nbead);
+    case BPIMD_FP64: return prep_go<BPIMD_FP64>(w, grid, pos, F, nbead, s);
+    case BPIMD_MIXED: return prep_go<BPIMD_MIXED>(w, grid, pos, F, nbead, s);
+    default: return prep_go<BPIMD_MIXED32>(w, grid, pos, F, nbead, s);
   }
 }
 

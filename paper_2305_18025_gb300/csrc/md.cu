@@ -44,14 +44,15 @@ constexpr int MD_THREADS = 256;
 constexpr int ENERGY_THREADS = 1024;  // the one block that adds a call's partial energies
 constexpr int EXT_THREADS = 128;
 constexpr int EXT_WARPS = EXT_THREADS / 32;
-// lanes per particle in the all-pairs force (two particles a thread): float64
-// pairs take ~15 times as long, and the smaller blocks spread them evenly
+// particles a thread and lanes a particle in the all-pairs force: float64 pairs
+// take ~15 times as long, and the smaller blocks spread them evenly
+constexpr int ext_ppt(bool mixed, bool pbc) { return mixed || pbc ? 2 : 1; }
 constexpr int ext_split(bool mixed) { return mixed ? 4 : 8; }
-constexpr int ext_particles(bool mixed) { return 2 * EXT_THREADS / ext_split(mixed); }
+constexpr int ext_particles(bool mixed, bool pbc) { return ext_ppt(mixed, pbc) * EXT_THREADS / ext_split(mixed); }
 constexpr int EXT_CHUNK = 1024;  // positions of one bead index staged per pass
 
-struct alignas(16) Dbl4 {
-  double x, y, z, w;
+struct Dbl3 {
+  double x, y, z;
 };
 
 __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32_t k1) {
@@ -142,7 +143,6 @@ __global__ void __launch_bounds__(MD_THREADS) md_update_kernel(double *__restric
   if (K && blockIdx.x == 0 && threadIdx.x == 0) *step += 1ull;
 }
 
-// Deterministic block sum (fixed shuffle tree, then warps in order); thread 0 gets it.
 // m 2^e of the integer-pipe power of two as a double (e <= 0; the exponent is
 // added with integer instructions; results below the normal range give 0)
 __device__ __forceinline__ double pow2_value(pow2fx::mexp r) {
@@ -177,6 +177,7 @@ __device__ __forceinline__ double f64_of_f32(float x) {
       (long long)(s | ((unsigned long long)(ex - 127 + 1023) << 52) | ((unsigned long long)(b & 0x7fffffu) << 29)));
 }
 
+// Deterministic block sum (fixed shuffle tree, then warps in order); thread 0 gets it.
 __device__ __forceinline__ double block_sum(double v, double *red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -189,83 +190,118 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
   return s;
 }
 
-// ------------------------------------- float64 Gaussian pairs in fixed point
+// --------------------------------- float64 Gaussian pairs on integer mantissas
 // GB300's float64 pipe takes ~75 cycles a warp instruction, and a directed pair
-// needs ten of them beside the integer power of two (720 us a pass at N = 1024,
-// P = 32).  With r' = c r, c^2 = log2(e)/(2 s^2), the Gaussian is 2^(-|d'|^2), so
-// on 64-bit fixed-point r' the whole pair runs on the integer pipe: differences
-// are exact, the three squares sum to the exponent itself (2^-56), and e d' is
-// summed in 96 bits (2^-58 a term; float64 sums round at 2^-53 of their size).
+// in float64 needs ten of them beside the integer power of two.  Here it forms
+// the three differences only.  Every later quantity keeps a mantissa and an
+// exponent of its own, so that a pair is as accurate relative to itself as in
+// float64, however near, far, wide or flat the system is: the squares are summed
+// on the scale of the largest component (2^-56 of d^2), times log2(e)/(2 s^2)
+// they are the argument of the power of two (2^-60), and e d is added to 96-bit
+// sums whose unit lies 62 bits below their largest term.  A pair is ~260
+// instructions, mostly of the integer pipe, beside the float64 pipe's ~57 cycles:
+// 408 us a pass at N = 1024, P = 32 (455 with e d multiplied and summed in float64,
+// ~720 all in float64).  One particle a thread: with two (122 registers for 80)
+// the pass took 460 us.
+struct Acc96 {  // (hi:mid:lo) 2^(B - 94), hi signed
+  unsigned lo, mid, hi;
+  int B;
+};
 struct Sum96 {
   unsigned lo, mid, hi;
 };
-__device__ __forceinline__ void add96(Sum96 &a, long long v) {
-  const unsigned vl = (unsigned)v, vh = (unsigned)((unsigned long long)v >> 32), vs = (unsigned)(v >> 63);
+__device__ __forceinline__ void add_words(unsigned &lo, unsigned &mid, unsigned &hi, unsigned x, unsigned y, unsigned z) {
   asm("add.cc.u32 %0, %0, %3;\n addc.cc.u32 %1, %1, %4;\n addc.u32 %2, %2, %5;"
-      : "+r"(a.lo), "+r"(a.mid), "+r"(a.hi)
-      : "r"(vl), "r"(vh), "r"(vs));
+      : "+r"(lo), "+r"(mid), "+r"(hi)
+      : "r"(x), "r"(y), "r"(z));
 }
-__device__ __forceinline__ double value96(const Sum96 &a) {
-  const long long top = (long long)(((unsigned long long)a.hi << 32) | a.mid);
-  return fma((double)top, 4294967296.0, (double)a.lo);
+// (hi:mid:lo) as a signed integer, rounded to float64
+__device__ __forceinline__ double value96(unsigned lo, unsigned mid, unsigned hi) {
+  const long long top = (long long)(((unsigned long long)hi << 32) | mid);
+  return fma((double)top, 4294967296.0, (double)lo);
+}
+// Room for a term of exponent pe: it is placed 31 bits below the sum's sign,
+// and later ones up to 2^16 times as large need no other move.
+constexpr int ACC_EMPTY = -(1 << 24), ACC_ROOM = 15;  // 2^13 terms a lane stay below 2^(95 - 2)
+__device__ __forceinline__ void acc_raise(Acc96 &a, int pe) {
+  int r = pe + 31 - a.B;
+  a.B = pe + 31;
+  if (r > 96) r = 96;
+  for (; r > 0; r -= 31) {
+    const int t = min(r, 31);
+    a.lo = __funnelshift_r(a.lo, a.mid, t);
+    a.mid = __funnelshift_r(a.mid, a.hi, t);
+    a.hi = (unsigned)((int)a.hi >> t);
+  }
+}
+// a += P 2^(pe - 62), |P| < 2^63, s = a.B - pe >= ACC_ROOM
+__device__ __forceinline__ void acc_add(Acc96 &a, long long P, int s) {
+  const long long top = P >> min(s, 63);
+  const unsigned low = s < 32 ? __funnelshift_r(0u, (unsigned)P, s) : (unsigned)(P >> min(s - 32, 63));
+  add_words(a.lo, a.mid, a.hi, low, (unsigned)top, (unsigned)((unsigned long long)top >> 32));
+}
+__device__ __forceinline__ double acc_value(const Acc96 &a) {
+  const int k = max(a.B - 94, -2044), k1 = k >> 1;  // in two factors: either is a normal number
+  if (k < -1000) return 0.0;                         // zero differences only
+  return value96(a.lo, a.mid, a.hi) * __longlong_as_double((long long)(k1 + 1023) << 52) *
+         __longlong_as_double((long long)(k - k1 + 1023) << 52);
 }
 
-// x c 2^S rounded to an integer; c = cm 2^(ce - 63), cm in [2^63, 2^64); the
-// result is below 2^62 (fixed_scale).
-__device__ __forceinline__ long long to_fixed_scaled(double x, unsigned long long cm, int ce, int S) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7ff);
-  if (ex == 0) return 0;  // zero or subnormal
-  const unsigned long long H = __umul64hi(((b << 11) | (1ull << 63)), cm);  // |x| c = H 2^(ex - 1023 + ce - 62)
-  const int k = 62 - (ex - 1023) - ce - S;                                   // to shift out, >= 1
-  const unsigned long long v = k > 63 ? 0ull : ((H >> (k - 1)) + 1) >> 1;
-  return (long long)b < 0 ? -(long long)v : (long long)v;
-}
-// Fraction bits S <= 60 at which |r'| stays below 2^(62 - S) (so that no
-// difference overflows), for the largest high word of |r|: 60 up to |r'| = 4.
-__device__ __forceinline__ int fixed_scale(int max_hi, int ce) { return min(60, 62 - ((max_hi >> 20) - 1022 + ce + 1)); }
-constexpr int FIXED_MIN_S = 56;  // |r'| < 64; past it (or with a non-finite coordinate) float64 as before
+struct GaussSum {  // sums over a lane's partners
+  Acc96 f[3];      // e d
+  Sum96 u;         // e, 2^-62 (the particle's own e = 1 included)
+  int bad;         // components that met a non-finite difference
+};
 
-// One directed pair: adds e d' (2^-58) and e (2^-62), e = 2^(-|d'|^2).
-__device__ __forceinline__ void gauss_fixed(long long X, long long Y, long long Z, long long x, long long y, long long z,
-                                            int sh, const unsigned long long *T63, Sum96 (&f)[3], Sum96 &u) {
-  long long D[3] = {X - x, Y - y, Z - z};
-  int out = 0;  // |d'| >= 8 along an axis: e < 2^-64, taken as 0
-  unsigned long long q = 0;
-  long long w = 0;
+// One directed pair of difference d: adds e d and e, e = 2^(-g2c |d|^2).
+__device__ __forceinline__ void gauss_pair(const double (&d)[3], unsigned long long gm, int ge,
+                                           const unsigned long long *T63, GaussSum &a) {
+  unsigned long long M[3];  // |d| = M 2^(ef - 1023 - 63), M in [2^63, 2^64); a zero counts as 2^-1023
+  int ef[3], sg[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const int top = (int)(D[c] >> 32);
-    out |= (top >> (31 - sh)) ^ (top >> 31);
-    D[c] = (long long)((unsigned long long)D[c] << sh);  // d' 2^60
-    const int h = (int)(D[c] >> 32), l = (int)((unsigned)D[c] >> 2);
-    q += (unsigned long long)((long long)h * h);  // (h 2^32 + 4 l)^2 = h^2 2^64 + h l 2^35 + ...
-    w += (long long)h * l;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d[c]);
+    const int hi = (int)(b >> 32);
+    sg[c] = hi >> 31;
+    ef[c] = (hi >> 20) & 0x7ff;
+    M[c] = (b << 11) | (1ull << 63);
   }
-  const unsigned long long x2 = q + (unsigned long long)(w >> 29);  // |d'|^2 2^56
-  const unsigned n = (unsigned)(x2 >> 56);
-  const unsigned long long res = pow2fx::pow2neg_frac((unsigned)(x2 >> 24), (unsigned)(x2 << 8), T63);
-  const unsigned long long e = (out != 0 || n > 62) ? 0ull : res >> (n + 1);  // 2^62 at most
-  const int eh = (int)(e >> 32), el = (int)((unsigned)e >> 1);
+  const int em = max(ef[0], max(ef[1], ef[2]));
+  if (em == 0x7ff) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a.bad |= (ef[c] == 0x7ff) << c;
+  }
+  unsigned long long q = 0, w = 0;  // |d|^2 = (q + w 2^-31) 2^(2 (em - 1023) - 58), the low words' squares left out
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const int h = (int)(D[c] >> 32);
-    add96(f[c], (long long)eh * h + (long long)__umulhi((unsigned)eh, (unsigned)D[c]) + 2ll * __mulhi(el, h));
+    const unsigned long long A = M[c] >> (min(em - ef[c], 61) + 2);
+    const unsigned h = (unsigned)(A >> 32), l = (unsigned)A;
+    q += (unsigned long long)h * h;
+    w += (unsigned long long)h * l;
   }
-  add96(u, (long long)e);
+  const unsigned long long Y = pow2fx::mulhi((q + (w >> 31)) << 2, gm);  // g2c |d|^2 = Y 2^-s
+  const int s = 59 - ge - 2 * (em - 1023);
+  const bool far = s < 49;  // Y >= 2^59: e < 2^-1024, as a float64 e would be zero
+  const bool whole = s < 64;
+  const unsigned long long F = whole ? Y << ((64 - s) & 63) : Y >> min(s - 64, 63);
+  const int n = whole ? (int)(Y >> (s & 63)) : 0;
+  const unsigned long long res = far ? 0ull : pow2fx::pow2neg_frac((unsigned)(F >> 32), (unsigned)F, T63);
+  const unsigned long long e = (unsigned)n > 62u ? 0ull : res >> (n + 1);
+  add_words(a.u.lo, a.u.mid, a.u.hi, (unsigned)e, (unsigned)(e >> 32), 0u);
+  if (far) return;
+  const int pe = -1023 - n;
+  if (min(a.f[0].B - ef[0], min(a.f[1].B - ef[1], a.f[2].B - ef[2])) - pe < ACC_ROOM) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (a.f[c].B - ef[c] - pe < ACC_ROOM) acc_raise(a.f[c], ef[c] + pe);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const long long P = (long long)pow2fx::mulhi(res, M[c]);
+    acc_add(a.f[c], (P ^ (long long)sg[c]) - (long long)sg[c], a.f[c].B - ef[c] - pe);
+  }
 }
 
-// -grad U-bar into Fx, per bead index j = blockIdx.y and block of 256 / SPLIT
-// particles (all pairs).  The SPLIT lanes of a thread group take the partners
-// q = sub, sub + SPLIT, ... of each staged chunk for two particles each (half
-// the block apart), so that one load from shared memory serves two pairs (a
-// 16-byte load a pair kept the shared-memory pipe at 79 % of its rate, 23.6
-// instructions a pair), and combine their sums by a fixed shuffle butterfly;
-// U-bar partial sum per block.  The positions of bead j of all particles pass
-// through shared memory in chunks.  Pairs: Gaussian g exp(-r^2/(2 s^2)), or
-// Lennard-Jones 4 eps ((sig/r)^12 - (sig/r)^6) truncated and shifted at rc; in a
-// periodic box (PBC) pair distances by minimum image.  MIXED: pair terms in
-// float32, accumulated per lane in float32.
 // Two float32 numbers in one 64-bit register: one instruction issued for two
 // IEEE operations (rounded as the scalar ones).
 using F2 = unsigned long long;
@@ -291,25 +327,32 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
   return r;
 }
 
-__device__ __forceinline__ int max_high(const double *r) {
-  return max(__double2hiint(r[0]) & 0x7fffffff, max(__double2hiint(r[1]) & 0x7fffffff, __double2hiint(r[2]) & 0x7fffffff));
-}
-
-template <bool MIXED, bool PBC, int SPLIT>
+// -grad U-bar into Fx, per bead index j and block of PPT * 128 / SPLIT particles
+// (all pairs).  The SPLIT lanes of a thread group take the partners q = sub,
+// sub + SPLIT, ... of each staged chunk for PPT particles each, and combine their
+// sums by a fixed shuffle butterfly; U-bar partial sum per block.  Two particles a
+// thread (half the block apart) where a load from shared memory counts: it serves
+// two pairs then (a 16-byte load a pair kept the shared-memory pipe at 79 % of its
+// rate, 23.6 instructions a pair).
+// The positions of bead j of all particles pass through shared memory in chunks.
+// Pairs: Gaussian g exp(-r^2/(2 s^2)), or Lennard-Jones 4 eps ((sig/r)^12 -
+// (sig/r)^6) truncated and shifted at rc; in a periodic box (PBC) pair distances
+// by minimum image.  MIXED: pair terms in float32, accumulated per lane in float32.
+template <bool MIXED, bool PBC, int SPLIT, int PPT>
 __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos, double *__restrict__ Fx, int N,
                                                  int P, const PairParams &pp, int lb, int j,
-                                                 typename std::conditional<MIXED, float4, Dbl4>::type *sr,
-                                                 double *red, unsigned long long *T63s, int *maxhi) {
+                                                 typename std::conditional<MIXED, float4, Dbl3>::type *sr,
+                                                 double *red, unsigned long long *T63s) {
   using R = typename std::conditional<MIXED, float, double>::type;
-  using R4 = typename std::conditional<MIXED, float4, Dbl4>::type;
-  constexpr int HALF = EXT_THREADS / SPLIT;  // particles of a block: 2 HALF
+  using R4 = typename std::conditional<MIXED, float4, Dbl3>::type;
+  constexpr int HALF = EXT_THREADS / SPLIT;  // particles of a block: PPT HALF
   const int sub = threadIdx.x % SPLIT;
-  int l[2];
-  double rd[2][3];
-  R px[2], py[2], pz[2];
+  int l[PPT];
+  double rd[PPT][3];
+  R px[PPT], py[PPT], pz[PPT];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    l[h] = lb * 2 * HALF + h * HALF + threadIdx.x / SPLIT;
+  for (int h = 0; h < PPT; ++h) {
+    l[h] = lb * PPT * HALF + h * HALF + threadIdx.x / SPLIT;
     const double *r = pos + ((size_t)min(l[h], N - 1) * P + j) * 3;
     rd[h][0] = r[0]; rd[h][1] = r[1]; rd[h][2] = r[2];
     // mixed: float32 positions and constants from integer-pipe conversions
@@ -325,57 +368,47 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
     if constexpr (PBC) return d - L * (MIXED ? (R)rintf((float)(d * invL)) : (R)rint((double)(d * invL)));
     else return d;
   };
-  constexpr bool FIXED = !MIXED && !PBC;  // Gaussian pairs in fixed point
-  Sum96 sf[2][3] = {}, su[2] = {};
-  R fx[2] = {0, 0}, fy[2] = {0, 0}, fz[2] = {0, 0}, u[2] = {0, 0};
-  int nin[2] = {0, 0};  // Lennard-Jones pairs inside the cutoff (each carries the shift)
+  constexpr bool INTEGER = !MIXED && !PBC;  // Gaussian pairs on integer mantissas
+  GaussSum gs[PPT];
+  if constexpr (INTEGER) {
+#pragma unroll
+    for (int h = 0; h < PPT; ++h) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) gs[h].f[c] = Acc96{0u, 0u, 0u, ACC_EMPTY};
+      gs[h].u = Sum96{0u, 0u, 0u};
+      gs[h].bad = 0;
+    }
+  }
+  R fx[PPT] = {}, fy[PPT] = {}, fz[PPT] = {}, u[PPT] = {};
+  int nin[PPT] = {};  // Lennard-Jones pairs inside the cutoff (each carries the shift)
   if (pp.pair != BPIMD_PAIR_NONE) {
     for (int base = 0; base < N; base += EXT_CHUNK) {
       const int cnt = min(EXT_CHUNK, N - base);
-      const bool fixed = FIXED && pp.pair == BPIMD_PAIR_GAUSSIAN;
-      int top = 0;  // largest high word of |r| of the chunk and of the block's particles
       __syncthreads();
-      if (fixed && threadIdx.x == 0) *maxhi = 0;
       for (int q = threadIdx.x; q < cnt; q += EXT_THREADS) {
         const double *r = pos + ((size_t)(base + q) * P + j) * 3;
-        if (fixed) top = max(top, max_high(r));
         R4 t;
         if constexpr (MIXED) { t.x = f32_of_f64(r[0]); t.y = f32_of_f64(r[1]); t.z = f32_of_f64(r[2]); }
         else { t.x = r[0]; t.y = r[1]; t.z = r[2]; }
-        t.w = (R)0;
+        if constexpr (MIXED) t.w = 0.0f;
         sr[q] = t;
       }
       __syncthreads();
-      if constexpr (FIXED) {
-        if (fixed) {
-          top = __reduce_max_sync(0xffffffffu, max(top, max(max_high(rd[0]), max_high(rd[1]))));
-          if ((threadIdx.x & 31) == 0) atomicMax(maxhi, top);
-          __syncthreads();
-          const int S = fixed_scale(*maxhi, pp.ce);
-          if (S >= FIXED_MIN_S) {
-            for (int q = threadIdx.x; q < cnt; q += EXT_THREADS) {  // each thread its own entries
-              R4 &t = sr[q];
-              t.x = __longlong_as_double(to_fixed_scaled(t.x, pp.cm, pp.ce, S));
-              t.y = __longlong_as_double(to_fixed_scaled(t.y, pp.cm, pp.ce, S));
-              t.z = __longlong_as_double(to_fixed_scaled(t.z, pp.cm, pp.ce, S));
+      if constexpr (INTEGER) {
+        if (pp.pair == BPIMD_PAIR_GAUSSIAN) {
+#pragma unroll 1
+          for (int q = sub; q < cnt; q += SPLIT) {
+            const R4 t = sr[q];
+#pragma unroll
+            for (int h = 0; h < PPT; ++h) {
+              const double d[3] = {px[h] - t.x, py[h] - t.y, pz[h] - t.z};
+              gauss_pair(d, pp.gm, pp.ge, T63s, gs[h]);
             }
-            long long X[2][3];
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-              for (int c = 0; c < 3; ++c) X[h][c] = to_fixed_scaled(rd[h][c], pp.cm, pp.ce, S);
-            __syncthreads();
-            for (int q = sub; q < cnt; q += SPLIT) {
-              const R4 t = sr[q];
-              const long long x = __double_as_longlong(t.x), y = __double_as_longlong(t.y), z = __double_as_longlong(t.z);
-#pragma unroll
-              for (int h = 0; h < 2; ++h) gauss_fixed(X[h][0], X[h][1], X[h][2], x, y, z, 60 - S, T63s, sf[h], su[h]);
-            }
-            continue;
           }
+          continue;
         }
       }
-      if constexpr (MIXED && !PBC) {
+      if constexpr (MIXED && !PBC && PPT == 2) {
         if (pp.pair == BPIMD_PAIR_GAUSSIAN) {
           // the two particles in the halves of packed float32 instructions
           const F2 X = pack2(px[0], px[1]), Y = pack2(py[0], py[1]), Z = pack2(pz[0], pz[1]), A = pack2(a, a),
@@ -406,7 +439,7 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
         for (int q = sub; q < cnt; q += SPLIT) {
           const R4 t = sr[q];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
+          for (int h = 0; h < PPT; ++h) {
             const R dx = img(px[h] - t.x), dy = img(py[h] - t.y), dz = img(pz[h] - t.z);
             const R d2 = dx * dx + dy * dy + dz * dz;
             R e;
@@ -421,7 +454,7 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
         for (int q = sub; q < cnt; q += SPLIT) {
           const R4 t = sr[q];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
+          for (int h = 0; h < PPT; ++h) {
             const R dx = img(px[h] - t.x), dy = img(py[h] - t.y), dz = img(pz[h] - t.z);
             const R r2 = dx * dx + dy * dy + dz * dz;
             if (r2 > (R)0 && r2 < rc2) {
@@ -436,14 +469,17 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
       }
     }
   }
-  double ub[2];
+  double ub[PPT];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if constexpr (FIXED) {
-      fx[h] = fma(value96(sf[h][0]), pp.ic, fx[h]);
-      fy[h] = fma(value96(sf[h][1]), pp.ic, fy[h]);
-      fz[h] = fma(value96(sf[h][2]), pp.ic, fz[h]);
-      u[h] = fma(value96(su[h]), 2.168404344971009e-19, u[h]);  // 2^-62
+  for (int h = 0; h < PPT; ++h) {
+    if constexpr (INTEGER) {
+      if (pp.pair == BPIMD_PAIR_GAUSSIAN) {
+        const double nan = __longlong_as_double(0x7ff8000000000000LL);
+        fx[h] = gs[h].bad & 1 ? nan : acc_value(gs[h].f[0]);
+        fy[h] = gs[h].bad & 2 ? nan : acc_value(gs[h].f[1]);
+        fz[h] = gs[h].bad & 4 ? nan : acc_value(gs[h].f[2]);
+        u[h] = value96(gs[h].u.lo, gs[h].u.mid, gs[h].u.hi) * 2.168404344971009e-19;  // 2^-62
+      }
     }
 #pragma unroll
     for (int o = 1; o < SPLIT; o <<= 1) {
@@ -487,13 +523,13 @@ __device__ __forceinline__ double ext_force_body(const double *__restrict__ pos,
   }
   // the warps' sums in a fixed order: first halves, then second halves
   if ((threadIdx.x & 31) == 0) {
-    red[threadIdx.x >> 5] = ub[0];
-    red[EXT_WARPS + (threadIdx.x >> 5)] = ub[1];
+#pragma unroll
+    for (int h = 0; h < PPT; ++h) red[h * EXT_WARPS + (threadIdx.x >> 5)] = ub[h];
   }
   __syncthreads();
   double sum = 0.0;
   if (threadIdx.x == 0)
-    for (int q = 0; q < 2 * EXT_WARPS; ++q) sum += red[q];
+    for (int q = 0; q < PPT * EXT_WARPS; ++q) sum += red[q];
   __syncthreads();
   return sum;
 }
@@ -529,13 +565,12 @@ template <bool MIXED, bool PBC>
 __global__ void __launch_bounds__(EXT_THREADS) ext_force_kernel(const double *__restrict__ pos,
                                                                 double *__restrict__ Fx, int N, int P, PairParams pp,
                                                                 double *ubar_part, Kicks kicks) {
-  using R4 = typename std::conditional<MIXED, float4, Dbl4>::type;
+  using R4 = typename std::conditional<MIXED, float4, Dbl3>::type;
   __shared__ R4 sr[EXT_CHUNK];
   __shared__ double red[2 * EXT_WARPS];
   __shared__ unsigned long long T63s[256];  // float64: the table of the integer-pipe power of two
-  __shared__ int maxhi;
   if ((int)blockIdx.y < P) {
-    const double s = ext_force_body<MIXED, PBC, ext_split(MIXED)>(pos, Fx, N, P, pp, blockIdx.x, blockIdx.y, sr, red, T63s, &maxhi);
+    const double s = ext_force_body<MIXED, PBC, ext_split(MIXED), ext_ppt(MIXED, PBC)>(pos, Fx, N, P, pp, blockIdx.x, blockIdx.y, sr, red, T63s);
     if (threadIdx.x == 0) ubar_part[blockIdx.y * gridDim.x + blockIdx.x] = s;
   } else {
     kicks_block<MIXED>(kicks, (blockIdx.y - P) * (long long)gridDim.x + blockIdx.x,
@@ -603,11 +638,10 @@ __global__ void __launch_bounds__(EXT_THREADS) ext_force_batched(const double *_
                                                                  const long long *__restrict__ off,
                                                                  const int4 *__restrict__ tab, int ntab, PairParams pp,
                                                                  double *ubar_part, Kicks kicks, int kick_blocks) {
-  using R4 = typename std::conditional<MIXED, float4, Dbl4>::type;
+  using R4 = typename std::conditional<MIXED, float4, Dbl3>::type;
   __shared__ R4 sr[EXT_CHUNK];
   __shared__ double red[2 * EXT_WARPS];
   __shared__ unsigned long long T63s[256];
-  __shared__ int maxhi;
   if ((int)blockIdx.x < kick_blocks) {
     kicks_block<MIXED>(kicks, blockIdx.x, kick_blocks);
     after_recursions(blockIdx.x == 0);
@@ -620,7 +654,14 @@ __global__ void __launch_bounds__(EXT_THREADS) ext_force_batched(const double *_
     PairParams q = pp;
     q.inv_P = ws[e.x].inv_P;
     q.finv_P = f32_of_f64(q.inv_P);
-    const double s = ext_force_body<MIXED, false, SPLIT>(pos + off[e.x], Fx + off[e.x], N, P, q, e.y, e.z, sr, red, T63s, &maxhi);
+    double s = 0.0;
+    if constexpr (MIXED) {
+      s = ext_force_body<MIXED, false, SPLIT, 2>(pos + off[e.x], Fx + off[e.x], N, P, q, e.y, e.z, sr, red, T63s);
+    } else {  // the tile's halves in turn
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h)
+        s += ext_force_body<MIXED, false, SPLIT, 1>(pos + off[e.x], Fx + off[e.x], N, P, q, 2 * e.y + h, e.z, sr, red, T63s);
+    }
     if (threadIdx.x == 0) ubar_part[k] = s;
     __syncthreads();  // sr is reused by the next entry
   }
@@ -730,14 +771,12 @@ int md_params(const bpimd_config &c, MDParams &p) {
     q.ga = c.pair_a;
     q.inv_s2 = 1.0 / (c.pair_b * c.pair_b);
     q.g2c = 0.5 * q.inv_s2 * 1.4426950408889634;  // log2(e) / (2 s^2)
-    // c = sqrt(g2c) to 64 bits: its float64 root and the residual's correction
-    const double root = std::sqrt(q.g2c), corr = std::fma(-root, root, q.g2c) / (2.0 * root);
-    int ex;
-    const double m = std::frexp(root, &ex);  // root = m 2^ex, m in [0.5, 1)
-    q.ce = ex - 1;
-    q.cm = (uint64_t)std::ldexp(m, 64) + (uint64_t)(int64_t)std::llround(std::ldexp(corr, 64 - ex));
-    if (!(q.cm >> 63)) q.cm = 1ull << 63;  // the correction took it below the power of two
-    q.ic = std::ldexp(1.0 / root, -58);
+    // g2c = gm 2^(ge - 63); where 1/s^2 has left the float64 range e is 0 or 1
+    int ex = 0;
+    const double m = std::frexp(q.g2c, &ex);  // m in [0.5, 1)
+    const bool normal = std::isfinite(q.g2c) && q.g2c >= 2.3e-308;
+    q.gm = normal ? (unsigned long long)std::ldexp(m, 64) : 1ull << 63;
+    q.ge = normal ? ex - 1 : (q.g2c < 1.0 ? -1100 : 1100);
   }
   if (c.pair_type == BPIMD_PAIR_LJ) {
     q.eps = c.pair_a;
@@ -815,7 +854,7 @@ int total_force(bpimd_ctx *ctx, const MDParams &p, const double *pos, KickStep k
     if (cudaStreamWaitEvent(s, md.join, 0) != cudaSuccess) return BPIMD_ERR_CUDA;
     return rc != BPIMD_OK ? rc : re;
   }
-  const int N = ctx->cfg.N, P = ctx->cfg.P, pb = ext_particles(ctx->w.bead32), gx = (N + pb - 1) / pb;
+  const int N = ctx->cfg.N, P = ctx->cfg.P, pb = ext_particles(ctx->w.bead32, p.pp.pbc), gx = (N + pb - 1) / pb;
   const dim3 grid(gx, P + (kick_blocks + gx - 1) / gx);
   return evaluate(ctx, pos, md.VB, md.F, [&] {
     auto go = [&](auto kernel) {
@@ -895,7 +934,7 @@ int md_alloc(bpimd_ctx *ctx, const MDParams &p) {
   }
   const size_t n = (size_t)ctx->cfg.N * ctx->cfg.P * 3;
   md.ext_blocks = p.cell_nc > 0 ? cell_list_partials(ctx->cfg.N, ctx->cfg.P)
-                                 : ((ctx->cfg.N + ext_particles(ctx->w.bead32) - 1) / ext_particles(ctx->w.bead32)) * ctx->cfg.P;
+                                 : ((ctx->cfg.N + ext_particles(ctx->w.bead32, p.pp.pbc) - 1) / ext_particles(ctx->w.bead32, p.pp.pbc)) * ctx->cfg.P;
   md.ke_blocks = grid_for((long long)n, MD_THREADS);
   md.spring_blocks = ctx->w.NB;
   if (cudaMalloc(&md.F, sizeof(double) * n) != cudaSuccess || cudaMalloc(&md.Fx, sizeof(double) * n) != cudaSuccess ||

@@ -11,9 +11,8 @@ struct PairParams {
   double inv_P, kt;      // 1/P, m w0^2 (trap)
   double ga, inv_s2;     // Gaussian g, 1/s^2
   double g2c;            // log2(e) / (2 s^2): the Gaussian is 2^(-g2c d^2)
-  unsigned long long cm; // c = sqrt(g2c) = cm 2^(ce - 63), cm in [2^63, 2^64)
-  int ce;
-  double ic;             // 2^-58 / c
+  unsigned long long gm; // g2c = gm 2^(ge - 63), gm in [2^63, 2^64)
+  int ge;
   double eps, sig2, rc2; // Lennard-Jones eps, sigma^2, cutoff^2
   double ushift;         // LJ energy at the cutoff (subtracted per pair inside it)
   double L, invL;        // periodic box (L = 0: open)

@@ -45,10 +45,12 @@ constexpr int ENERGY_THREADS = 1024;  // the one block that adds a call's partia
 constexpr int EXT_THREADS = 128;
 constexpr int EXT_WARPS = EXT_THREADS / 32;
 // particles a thread and lanes a particle in the all-pairs force: float64 pairs
-// take ~15 times as long, and the smaller blocks spread them evenly
-constexpr int ext_ppt(bool mixed, bool pbc) { return mixed || pbc ? 2 : 1; }
+// take ~15 times as long, and the smaller blocks spread them evenly (in a box,
+// N = 512, P = 32, four steps: Gaussian 2131 us and Lennard-Jones 4217 with one
+// particle and eight lanes; two and eight 2563, 5152; one and four 2520, 5117)
+constexpr int ext_ppt(bool mixed) { return mixed ? 2 : 1; }
 constexpr int ext_split(bool mixed) { return mixed ? 4 : 8; }
-constexpr int ext_particles(bool mixed, bool pbc) { return ext_ppt(mixed, pbc) * EXT_THREADS / ext_split(mixed); }
+constexpr int ext_particles(bool mixed) { return ext_ppt(mixed) * EXT_THREADS / ext_split(mixed); }
 constexpr int EXT_CHUNK = 1024;  // positions of one bead index staged per pass
 
 struct Dbl3 {
@@ -570,7 +572,7 @@ __global__ void __launch_bounds__(EXT_THREADS) ext_force_kernel(const double *__
   __shared__ double red[2 * EXT_WARPS];
   __shared__ unsigned long long T63s[256];  // float64: the table of the integer-pipe power of two
   if ((int)blockIdx.y < P) {
-    const double s = ext_force_body<MIXED, PBC, ext_split(MIXED), ext_ppt(MIXED, PBC)>(pos, Fx, N, P, pp, blockIdx.x, blockIdx.y, sr, red, T63s);
+    const double s = ext_force_body<MIXED, PBC, ext_split(MIXED), ext_ppt(MIXED)>(pos, Fx, N, P, pp, blockIdx.x, blockIdx.y, sr, red, T63s);
     if (threadIdx.x == 0) ubar_part[blockIdx.y * gridDim.x + blockIdx.x] = s;
   } else {
     kicks_block<MIXED>(kicks, (blockIdx.y - P) * (long long)gridDim.x + blockIdx.x,
@@ -854,7 +856,7 @@ int total_force(bpimd_ctx *ctx, const MDParams &p, const double *pos, KickStep k
     if (cudaStreamWaitEvent(s, md.join, 0) != cudaSuccess) return BPIMD_ERR_CUDA;
     return rc != BPIMD_OK ? rc : re;
   }
-  const int N = ctx->cfg.N, P = ctx->cfg.P, pb = ext_particles(ctx->w.bead32, p.pp.pbc), gx = (N + pb - 1) / pb;
+  const int N = ctx->cfg.N, P = ctx->cfg.P, pb = ext_particles(ctx->w.bead32), gx = (N + pb - 1) / pb;
   const dim3 grid(gx, P + (kick_blocks + gx - 1) / gx);
   return evaluate(ctx, pos, md.VB, md.F, [&] {
     auto go = [&](auto kernel) {
@@ -934,7 +936,7 @@ int md_alloc(bpimd_ctx *ctx, const MDParams &p) {
   }
   const size_t n = (size_t)ctx->cfg.N * ctx->cfg.P * 3;
   md.ext_blocks = p.cell_nc > 0 ? cell_list_partials(ctx->cfg.N, ctx->cfg.P)
-                                 : ((ctx->cfg.N + ext_particles(ctx->w.bead32, p.pp.pbc) - 1) / ext_particles(ctx->w.bead32, p.pp.pbc)) * ctx->cfg.P;
+                                 : ((ctx->cfg.N + ext_particles(ctx->w.bead32) - 1) / ext_particles(ctx->w.bead32)) * ctx->cfg.P;
   md.ke_blocks = grid_for((long long)n, MD_THREADS);
   md.spring_blocks = ctx->w.NB;
   if (cudaMalloc(&md.F, sizeof(double) * n) != cudaSuccess || cudaMalloc(&md.Fx, sizeof(double) * n) != cudaSuccess ||

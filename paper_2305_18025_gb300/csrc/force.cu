@@ -69,8 +69,8 @@ __device__ __forceinline__ double img(const Workspace &w, double d) {
 //   Mixed forms: unevaluated float32 pairs (products by FMA, sums by TwoSum:
 //   2^-46 relative) on the float32 pipe; the powers of two of all factors,
 //   the taken-out ones included, scale the pair, so a term is at most 2.
-//   FP64: 64-bit integer mantissas, signed 64-bit sums with one running
-//   exponent a lane (2^-60 of the largest term of a group of four); GB300's
+//   FP64: 64-bit integer mantissas, signed 64-bit sums with a running exponent
+//   a lane and component (2^-57 of the largest term of a group of four); GB300's
 //   float64 pipe retires ~1.7 lanes a clock, so it forms the differences only.
 // The sums of the probabilities themselves are not needed: by the recursions'
 // own equations sum_u Pr[l->u] + Pr[l->l+1] = 1, and so for the columns.
@@ -79,8 +79,8 @@ __device__ __forceinline__ double img(const Workspace &w, double d) {
 // Each pair is formed twice (row and column), which costs less than the
 // transposed reduction, the global partial sums, the fence and the counters
 // of a pass that forms it once.
-struct PSum {  // FP64: sum_c = v[c] 2^(E - 61)
-  long long v[3];
+struct PSum {  // FP64: v 2^(E - 61)
+  long long v;
   int E;
 };
 
@@ -91,12 +91,12 @@ __device__ __forceinline__ unsigned long long mant64(double m) {  // [1, 2) -> [
 // |x| as a mantissa in [2^62, 2^63) (value M 2^(e - 62)) times the term t:
 // the high product, its exponent e, its sign; a zero has the exponent NO_TERM
 constexpr int NO_TERM = -(1 << 30);
-__device__ __forceinline__ unsigned long long diff_term(unsigned long long t, double x, int &e, int &sgn, int &bad) {
+__device__ __forceinline__ unsigned long long diff_term(unsigned long long t, double x, int &e, int &sgn, bool &bad) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int hi = (int)(b >> 32), ex = (hi >> 20) & 0x7ff;
   sgn = hi >> 31;
   e = ex ? ex - 1023 : NO_TERM;
-  bad |= ex == 0x7ff;
+  bad = ex == 0x7ff;
   return pow2fx::mulhi(t, ((b << 10) & 0x3FFFFFFFFFFFFFFFull) | (1ull << 62));
 }
 
@@ -124,20 +124,11 @@ __device__ __forceinline__ long long shift_in(long long v, int k) { return v >> 
 
 // a + b, |b| < 2^62; |a| stays below 2^62
 __device__ __forceinline__ void psum_add(PSum &a, const PSum &b) {
-  const int E = max(a.E, b.E), ka = E - a.E, kb = E - b.E;
-  bool big = false;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    a.v[c] = shift_in(a.v[c], ka) + shift_in(b.v[c], kb);
-    const int h = (int)(a.v[c] >> 32);
-    big |= (h ^ (h >> 31)) >= (1 << 30);
-  }
-  a.E = E;
-  if (big) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) a.v[c] >>= 1;
-    a.E += 1;
-  }
+  const int E = max(a.E, b.E);
+  a.v = shift_in(a.v, E - a.E) + shift_in(b.v, E - b.E);
+  const int h = (int)(a.v >> 32), big = (h ^ (h >> 31)) >> 30;  // 0 or 1
+  a.v >>= big;
+  a.E = E + big;
 }
 
 // Mixed forms: s + c with every rounding error of s in c
@@ -172,7 +163,7 @@ struct SumSlot<false> {
 template <>
 struct SumSlot<true> {
   long long v[3][TILE];
-  int E[TILE], bad[TILE];
+  int E[3][TILE], bad[TILE];
 };
 // Staged partners.  Mixed forms: the endpoint's high and low parts (or, in a
 // box, its fixed-point words) with the weight's mantissa parts in the fourth
@@ -268,8 +259,8 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
   const int gi0 = (int)gbase<GS>(w, r), gstr = gstride<GS>(w);
   const M_t *gm = (const M_t *)(row_item ? w.gm : w.gbm) + gi0;
   const int *ge = (row_item ? w.ge : w.gbe) + gi0;
-  PSum A{{0, 0, 0}, NO_TERM};
-  int bad = 0;
+  PSum A[3] = {{0, NO_TERM}, {0, NO_TERM}, {0, NO_TERM}};
+  int bad = 0;  // components that met a non-finite difference
   float fs[3] = {0.f, 0.f, 0.f}, fc[3] = {0.f, 0.f, 0.f};
   constexpr int G = 4;
   for (int c0 = p0 + rank * ch; c0 < p1; c0 += CL * ch) {
@@ -297,7 +288,7 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
       for (int k = 0; k < G; ++k) { m[k] = gmv[k]; e[k] = gev[k]; }
       if (!RC && q + G < q1) load_g(q + G);
       unsigned long long p[G][3];
-      int pe[G][3], sg[G][3], E = NO_TERM;
+      int pe[G][3], sg[G][3], E[3] = {NO_TERM, NO_TERM, NO_TERM};
 #pragma unroll
       for (int k = 0; k < G; ++k) {
         const int i = min(q + k, p1 - 1) - c0;
@@ -318,15 +309,14 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
         if constexpr (F64) {
           const unsigned long long t = valid ? pow2fx::mulhi(sm.part.m[i], mant64(m[k])) : 0ull;  // value t 2^(et - 63)
           const int et = valid ? sm.part.e[i] + e[k] + 1 : NO_TERM;
-          int nonfinite = 0;
-          p[k][0] = diff_term(t, d.x, pe[k][0], sg[k][0], nonfinite);
-          p[k][1] = diff_term(t, d.y, pe[k][1], sg[k][1], nonfinite);
-          p[k][2] = diff_term(t, d.z, pe[k][2], sg[k][2], nonfinite);
-          bad |= valid ? nonfinite : 0;
+          const double dc[3] = {d.x, d.y, d.z};
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
+            bool nonfinite;
+            p[k][c] = diff_term(t, dc[c], pe[k][c], sg[k][c], nonfinite);
+            bad |= (valid && nonfinite) << c;
             pe[k][c] = max(pe[k][c] + et, NO_TERM);
-            E = max(E, pe[k][c]);
+            E[c] = max(E[c], pe[k][c]);
           }
         } else {
           const float yh = sm.part.h[i].w, yl = sm.part.l[i].w;
@@ -346,32 +336,33 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
         }
       }
       if constexpr (F64) {
-        PSum B{{0, 0, 0}, E + 3};
 #pragma unroll
-        for (int k = 0; k < G; ++k)
+        for (int c = 0; c < 3; ++c) {
+          PSum B{0, E[c] + 3};
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const long long x = (long long)(p[k][c] >> min(E - pe[k][c] + 3, 63));
-            B.v[c] += (x ^ sg[k][c]) - sg[k][c];
+          for (int k = 0; k < G; ++k) {
+            const long long x = (long long)(p[k][c] >> min(E[c] - pe[k][c] + 3, 63));
+            B.v += (x ^ sg[k][c]) - sg[k][c];
           }
-        psum_add(A, B);
+          psum_add(A[c], B);
+        }
       }
     }
   }
   SumSlot<F64> &ws = sm.warp[wp];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    if constexpr (F64) ws.v[c][lane] = A.v[c];
+    if constexpr (F64) { ws.v[c][lane] = A[c].v; ws.E[c][lane] = A[c].E; }
     else { ws.s[c][lane] = fs[c]; ws.c[c][lane] = fc[c]; }
   }
-  if constexpr (F64) { ws.E[lane] = A.E; ws.bad[lane] = bad; }
+  if constexpr (F64) ws.bad[lane] = bad;
   __syncthreads();
   // warp c < 3: component c of the lane's sum over `n` slots, in order
   auto add_slots = [&](const SumSlot<F64> *sl, int n, int c, long long &v, int &E, int &bd, float &s, float &cc) {
     if constexpr (F64) {
       v = 0; E = NO_TERM; bd = 0;
-      for (int k = 0; k < n; ++k) { E = max(E, sl[k].E[lane]); bd |= sl[k].bad[lane]; }
-      for (int k = 0; k < n; ++k) v += shift_in(sl[k].v[c][lane], E - sl[k].E[lane] + 3);
+      for (int k = 0; k < n; ++k) { E = max(E, sl[k].E[c][lane]); bd |= sl[k].bad[lane]; }
+      for (int k = 0; k < n; ++k) v += shift_in(sl[k].v[c][lane], E - sl[k].E[c][lane] + 3);
       E += 3;
     } else {
       s = 0.0f; cc = 0.0f;
@@ -401,7 +392,8 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
       SumSlot<F64> &cs = sm.cta[rank];
       if constexpr (F64) {
         cluster_store(&cs.v[wp][lane], v);
-        if (wp == 0) { cluster_store(&cs.E[lane], E); cluster_store(&cs.bad[lane], bd); }
+        cluster_store(&cs.E[wp][lane], E);
+        if (wp == 0) cluster_store(&cs.bad[lane], bd);
       } else {
         cluster_store(&cs.s[wp][lane], s);
         cluster_store(&cs.c[wp][lane], cc);
@@ -418,7 +410,7 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
     double W;
     if constexpr (F64) {
       W = ((double)v * mz) * pow2_normal(E - 61 + own_e);
-      if (bd) W = __longlong_as_double(0x7ff8000000000000LL);
+      if ((bd >> wp) & 1) W = __longlong_as_double(0x7ff8000000000000LL);
     } else {
       W = ((double)s + (double)cc) * mz;
     }

@@ -154,7 +154,7 @@ __device__ void panel_inverse_body(const Workspace &w, int t, int q, PinvSmem &s
       xi y;
       y.m = __shfl_sync(0xffffffffu, acc.m, s);
       y.e = __shfl_sync(0xffffffffu, acc.e, s);
-      acc = xi_fma<false>(acc, sm.Lk[s][lane], sm.Le[s][lane], y);
+      acc = xi_fma(acc, sm.Lk[s][lane], sm.Le[s][lane], y);
     }
   cg::cluster_group cluster = cg::this_cluster();
   const size_t base = panel_base(w, BWD, t);
@@ -276,28 +276,28 @@ __device__ __forceinline__ xi wire_get(const Wire *p) {
 
 // A row's sum over a warp: two products a lane (kk y, in the K and xi formats)
 // and one more term (p0, pe0) a lane, at most 72 terms in all.  The largest
-// exponent first (one redux), then every term aligned to it with six bits of
-// headroom (72 x 2^57 < 2^64), and the 64-bit sums added exactly in three
-// pieces of 21 and 22 bits by redux: five warp-wide steps where a shuffle tree
-// of extended numbers takes five levels of six.
+// exponent first (one redux), then every term aligned to it with two bits of
+// headroom for the lane's three (2^-59 of the largest), and the 63-bit sums added
+// exactly in three pieces of 21 bits by redux: four warp-wide steps where a
+// shuffle tree of extended numbers takes five levels of six.
 __device__ __forceinline__ xi row_sum(const unsigned long long (&kk)[2], const int (&ke)[2], const xi (&y)[2],
                                       unsigned long long p0, int pe0) {
   unsigned long long p[2];
   int pe[2];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    p[i] = pow2fx::mulhi(kk[i], y[i].m);
+    p[i] = pow2fx::mulhi_centred(kk[i], y[i].m);
     pe[i] = ke[i] + y[i].e + 1;
   }
   const int E = __reduce_max_sync(0xffffffffu, max(pe0, max(pe[0], pe[1])));
   const unsigned long long s =
-      (p0 >> min(E - pe0 + 6, 63)) + (p[0] >> min(E - pe[0] + 6, 63)) + (p[1] >> min(E - pe[1] + 6, 63));
+      (p0 >> min(E - pe0 + 2, 63)) + (p[0] >> min(E - pe[0] + 2, 63)) + (p[1] >> min(E - pe[1] + 2, 63));
   const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)s & 0x1FFFFFu);
   const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(s >> 21) & 0x1FFFFFu);
   const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(s >> 42));
-  xsum t{((unsigned long long)hi << 42) + ((unsigned long long)mid << 21) + lo, E};
-  if (t.s >> 63) t = xsum{t.s >> 1, t.E + 1};
-  return xsum_fin<6>(t);
+  // hi 2^42 + mid 2^21 + lo < 2^68: five bits less of it where it would not fit
+  const int k = hi >> 20 ? 5 : 0;
+  return xsum_fin<2>(xsum{((unsigned long long)hi << (42 - k)) + ((((unsigned long long)mid << 21) + lo) >> k), E + k});
 }
 
 template <int CL>

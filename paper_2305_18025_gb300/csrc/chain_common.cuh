@@ -78,8 +78,9 @@ __device__ __forceinline__ xk mul_mant(xd c, M_t hm, int he) {
 // read its result), while a 64 x 64-bit integer product, shifts and a 64-bit
 // add take a few cycles each.  An extended number is  m * 2^(e - 62)  with an
 // integer mantissa m in [2^62, 2^63) (one bit of headroom for an addition);
-// the extended zero is 2^62 * 2^(XZERO_E - 62).  Products and alignment shifts
-// truncate, at 2^-61 relative: finer than a float64 rounding.
+// the extended zero is 2^62 * 2^(XZERO_E - 62).  Products are within 2^-60,
+// alignment shifts truncate at 2^-61 (sums of many terms: at their headroom,
+// below): finer than a float64 rounding.
 struct xi {
   unsigned long long m;
   int e;
@@ -116,17 +117,9 @@ __device__ __forceinline__ xi xi_mul(xi a, xd c) {
 // acc + K * y with K = kk 2^(ke - 63), kk in [2^63, 2^64): the step of the
 // dependency chain.  The product kk * y.m / 2^64 lies in [2^61, 2^63), the
 // aligned sum in [2^61, 2^64); a K carrying an extended-zero exponent leaves
-// acc unchanged.  MIXED uses the top 32 bits of kk only (two 32 x 32-bit
-// products, relative error below 2^-30: K = c g carries a float32 g there).
-template <bool MIXED>
+// acc unchanged.
 __device__ __forceinline__ xi xi_fma(xi acc, unsigned long long kk, int ke, xi y) {
-  unsigned long long p;
-  if (MIXED) {
-    const unsigned k1 = (unsigned)(kk >> 32);
-    p = (unsigned long long)k1 * (unsigned)(y.m >> 32) + (((unsigned long long)k1 * (unsigned)y.m) >> 32);
-  } else {
-    p = pow2fx::mulhi(kk, y.m);
-  }
+  const unsigned long long p = pow2fx::mulhi_centred(kk, y.m);
   const int pe = ke + y.e + 1;
   const int E = max(acc.e, pe);
   return xi_norm((acc.m >> min(E - acc.e, 63)) + (p >> min(E - pe, 63)), E);
@@ -346,7 +339,7 @@ __device__ __forceinline__ void chain_tile(int N, int t, xi A, xd crow, const un
       ke1 = lds_s32(aKe + (i + 1) * 33 * 4);
     }
     if constexpr (MIXED) acc = xs_fma(acc, km, ke, y);
-    else acc = xi_fma<false>(acc, km, ke, y);
+    else acc = xi_fma(acc, km, ke, y);
     y.m = __shfl_sync(0xffffffffu, acc.m, i);
     y.e = __shfl_sync(0xffffffffu, acc.e, i);
     km = km1;
@@ -428,7 +421,7 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // p = kk y.m / 2^64 in [2^61, 2^63), of value p 2^(pe - 62), pe = ke + y.e + 1;
 // an xi itself is the term (y.m, y.e).  A sum of at most 2^S terms is aligned
 // to the largest exponent E with S bits of headroom: s = sum_i p_i >>
-// (E - pe_i + S) < 2^63, of value s 2^(E + S - 62); each shift truncates below
+// (E - pe_i + S) < 2^63, of value s 2^(E + S - 62); each shift truncates at
 // 2^-(61 - S) of the largest term.  Partial sums of one S combine by xsum_add.
 struct xsum {
   unsigned long long s;
@@ -447,7 +440,7 @@ __device__ __forceinline__ xsum xsum_dot(const unsigned long long *kk, const int
   int E = pe0;
 #pragma unroll
   for (int i = 0; i < K; ++i) {
-    p[i] = pow2fx::mulhi(kk[i], y[i].m);
+    p[i] = pow2fx::mulhi_centred(kk[i], y[i].m);
     pe[i] = ke[i] + y[i].e + 1;
     E = max(E, pe[i]);
   }

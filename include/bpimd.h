@@ -115,7 +115,9 @@ extern "C" {
  * memory: 12 or 8 bytes per pair and copy, ~0.8 GB at N = 8192).  Above it --
  * or at any N when cfg.flags has BPIMD_FLAG_RECOMPUTE -- nothing O(N^2) is
  * stored: the recursions and the exterior forces recompute each g where they
- * use it (the same bits).  Device memory is then O(N + N P). */
+ * use it (the same bits).  Device memory is then O(N + N P).  (BPIMD_FP64 and
+ * BPIMD_MIXED systems of up to 128 particles keep their tables, 240 KB at most,
+ * in either mode.) */
 #define BPIMD_STORE_MAX_N 8192
 #define BPIMD_FLAG_RECOMPUTE 1
 /* Test hook of the error path (bpimd_create only): the forward recursion's

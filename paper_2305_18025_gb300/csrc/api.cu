@@ -205,7 +205,10 @@ int bpimd_create(bpimd_ctx **out, const bpimd_config *cfg, void *cuda_stream) {
   w.k = cfg->m * cfg->omega_P * cfg->omega_P;
   w.half_k = 0.5 * w.k;
   w.cx = w.beta * w.half_k * LOG2E;
-  w.recomp = (cfg->flags & BPIMD_FLAG_RECOMPUTE) || cfg->N > BPIMD_STORE_MAX_N;
+  // Small systems keep their tables (240 KB at N = 128) in either mode: the
+  // one-CTA recursions took twice as long with recomputed factors (N = 100 float64
+  // 73.9 us for ~30) and more than the clusters had (61.4).
+  w.recomp = ((cfg->flags & BPIMD_FLAG_RECOMPUTE) && !small_chain(cfg->N, cfg->precision)) || cfg->N > BPIMD_STORE_MAX_N;
   w.test_timeout = (cfg->flags & BPIMD_FLAG_TEST_TIMEOUT) != 0;
   w.blocks = 1;
   w.gstr = w.N > CHAIN_SMALL_N ? 4 : 32;

@@ -42,6 +42,7 @@ constexpr int CHAIN_SLICES = 4;       // partial sums a row carries between supe
 constexpr int CHAIN_CLUSTER = 8;      // CTAs per recursion (small N)
 constexpr int CHAIN_MAX_N = BPIMD_MAX_N;  // largest N the library accepts
 constexpr int CHAIN_SMALL_N = 128;    // largest single system on one CTA per recursion
+constexpr bool small_chain(int N, int precision) { return N <= CHAIN_SMALL_N && precision != BPIMD_MIXED32; }
 constexpr int BATCH_MAX_N = 4096;     // largest replica of a batch (one CTA per recursion)
 constexpr int BEAD_BLOCK_PARTICLES = 8;  // particles per block of the bead pass
 constexpr int BATCH_BEAD_PARTICLES = 32; // the same in a replica batch

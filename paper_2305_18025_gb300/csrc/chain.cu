@@ -812,7 +812,7 @@ cudaError_t launch_chains(const Workspace &w, double *V_B, cudaStream_t s) {
   // One CTA per recursion with 32-row tiles and no panel inverses, against the
   // panels on clusters: N = 16 16.7 / 20.8 us, N = 64 20.5 / 25.5, N = 128
   // 25.5 / 26.6, N = 192 31.7 / 28.3.
-  if (!w.mixed && !w.test_timeout && w.N <= CHAIN_SMALL_N) return launch_chains_small(w, V_B, s);
+  if (small_chain(w.N, w.mode) && !w.test_timeout) return launch_chains_small(w, V_B, s);
   int dev = 0;
   cudaGetDevice(&dev);
   bool large_ok;

@@ -44,7 +44,6 @@ struct SingleSmem {
   int Kde[2 * BLK];
   int Hoe[2 * BLK];
   int Pe[BATCH_COUPLE][TILE];
-  unsigned long long T63[256];  // recompute mode
   int task[2];  // row tiles of the sums handed out, by parity of t
 };
 
@@ -57,9 +56,9 @@ __host__ __device__ constexpr size_t single_smem_bytes(int N) {
 // warp id -> role index q for warps off warp 0's sub-partition (-1 otherwise)
 __device__ __forceinline__ int role_q(int wid) { return (wid & 3) ? wid - (wid >> 2) - 1 : -1; }
 
-// MODE: BPIMD_MIXED32, or BPIMD_FP64 for both 64-bit forms' stored factors; RC:
-// recompute mode (any form).  ALONE: this CTA has its SM to itself (see above).
-template <int MODE, bool BWD, bool ALONE, bool RC, bool PBC>
+// MODE: BPIMD_MIXED32, or BPIMD_FP64 for both 64-bit forms (stored factors).
+// ALONE: this CTA has its SM to itself (see above).
+template <int MODE, bool BWD, bool ALONE>
 __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *V_B) {
   constexpr bool MIXED = MODE == BPIMD_MIXED32;
   using M_t = typename std::conditional<MIXED, float, double>::type;
@@ -79,8 +78,8 @@ __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *
   if (tid == 0) { Ym[0] = 1.0; Yk[0] = 1ull << 62; Ye[0] = 0; gYm[0] = 1.0; gYe[0] = 0; }
   if (!BWD && tid == 0) w.C[0] = 0.0;
   if (tid < 2) sm.task[tid] = 0;
-  if (q >= 0 && q < 4) stage_diag<MODE, BWD, RC, PBC, 8>(w, 0, 8 * q, sm.Kdm, sm.Kde, sm.T63);
-  if (q == 4 || q == 5) stage_offdiag<MODE, BWD, RC, PBC, 16>(w, 0, 16 * (q - 4), sm.Hom, sm.Hoe, sm.T63);
+  if (q >= 0 && q < 4) stage_diag<MODE, BWD, 8>(w, 0, 8 * q, sm.Kdm, sm.Kde);
+  if (q == 4 || q == 5) stage_offdiag<MODE, BWD, 16>(w, 0, 16 * (q - 4), sm.Hom, sm.Hoe);
   __syncthreads();
 
   xd cnext{1.0, 0};
@@ -111,12 +110,11 @@ __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *
     } else if (q >= 0 || !ALONE) {
       if (q < 0) {
       } else if (q < 4) {
-        if (t + 1 < NT) 
-          stage_diag<MODE, BWD, RC, PBC, 8>(w, t + 1, 8 * q, sm.Kdm + (buf ^ 1) * BLK, sm.Kde + (buf ^ 1) * BLK, sm.T63);
+        if (t + 1 < NT)
+          stage_diag<MODE, BWD, 8>(w, t + 1, 8 * q, sm.Kdm + (buf ^ 1) * BLK, sm.Kde + (buf ^ 1) * BLK);
       } else if (q < 6) {
         if (t + 1 < NT)
-          stage_offdiag<MODE, BWD, RC, PBC, 16>(w, t + 1, 16 * (q - 4), sm.Hom + (buf ^ 1) * BLK,
-                                                sm.Hoe + (buf ^ 1) * BLK, sm.T63);
+          stage_offdiag<MODE, BWD, 16>(w, t + 1, 16 * (q - 4), sm.Hom + (buf ^ 1) * BLK, sm.Hoe + (buf ^ 1) * BLK);
       } else if (q == 6) {
         if (!BWD) prefix_tile(w, t, carry, ncarry);
       }
@@ -129,9 +127,9 @@ __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *
         if (T >= NT) break;
         const int r = T * TILE + lane;
         const int ra = r < N ? r : 0;
-        RowFactors<MODE, BWD, RC, PBC, 32> f;  // rows past N: their tile's padding, or particle 0's (sums not kept)
-        f.load(w, RC ? ra : r);
-        auto load = [&](int src, M_t &m, int &e) { f.h(w, min(src, RC && r >= N ? 0 : src), sm.T63, m, e); };
+        RowFactors<MODE, BWD, false, false, 32> f;  // rows past N: their tile's padding (sums not kept)
+        f.load(w, r);
+        auto load = [&](int src, M_t &m, int &e) { f.h(w, src, nullptr, m, e); };
         if constexpr (MIXED) {
           float sacc = 0.0f;
           int E = XZERO_E;
@@ -224,23 +222,13 @@ __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *
   }
 }
 
-// A single small system: CTA d runs recursion d.
-template <int MODE, bool RC>
+// A single small system of either 64-bit form: CTA d runs recursion d.
 __global__ void __launch_bounds__(BATCH_THREADS) chain_small_kernel(Workspace w, double *V_B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (RC) {
-    pairg::table_init(((SingleSmem *)smem_raw)->T63);
-    __syncthreads();
-  }
   pdl_wait();
-  pdl_trigger();
-  if (RC && w.pbc) {
-    if (blockIdx.x & 1) run_single<MODE, true, true, RC, RC>(w, smem_raw, nullptr);
-    else run_single<MODE, false, true, RC, RC>(w, smem_raw, V_B);
-  } else {
-    if (blockIdx.x & 1) run_single<MODE, true, true, RC, false>(w, smem_raw, nullptr);
-    else run_single<MODE, false, true, RC, false>(w, smem_raw, V_B);
-  }
+  pdl_trigger();  // what runs beside the recursions may start; what needs them waits for this grid
+  if (blockIdx.x & 1) run_single<BPIMD_FP64, true, true>(w, smem_raw, nullptr);
+  else run_single<BPIMD_FP64, false, true>(w, smem_raw, V_B);
 }
 
 // CTA 2k + d runs recursion d (0 forward, 1 backward) of replica order[k].
@@ -254,8 +242,8 @@ __global__ void __launch_bounds__(BATCH_THREADS, 2) chain_batched_kernel(const W
   pdl_wait();
   pdl_trigger();  // what runs beside the recursions may start; what needs them waits for this grid
   const int r = order[blockIdx.x >> 1];
-  if (blockIdx.x & 1) run_single<MIXED ? BPIMD_MIXED32 : BPIMD_FP64, true, false, false, false>(ws[r], smem_raw, nullptr);
-  else run_single<MIXED ? BPIMD_MIXED32 : BPIMD_FP64, false, false, false, false>(ws[r], smem_raw, V_B ? V_B + r : nullptr);
+  if (blockIdx.x & 1) run_single<MIXED ? BPIMD_MIXED32 : BPIMD_FP64, true, false>(ws[r], smem_raw, nullptr);
+  else run_single<MIXED ? BPIMD_MIXED32 : BPIMD_FP64, false, false>(ws[r], smem_raw, V_B ? V_B + r : nullptr);
 }
 
 static_assert(single_smem_bytes(BATCH_MAX_N) <= 227 * 1024, "batched recursion state must fit in shared memory");
@@ -264,21 +252,14 @@ static_assert(BATCH_THREADS / 32 == 16, "role table assumes 16 warps");
 }  // namespace
 
 cudaError_t prepare_chains_small() {
-  const int bytes = (int)single_smem_bytes(CHAIN_SMALL_N);
-  cudaError_t e = cudaSuccess;
-  for (auto k : {chain_small_kernel<BPIMD_FP64, false>, chain_small_kernel<BPIMD_FP64, true>,
-                 chain_small_kernel<BPIMD_MIXED, true>})
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  return e;
+  return cudaFuncSetAttribute(chain_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)single_smem_bytes(CHAIN_SMALL_N));
 }
 
 // BPIMD_FP64 and BPIMD_MIXED (BPIMD_MIXED32's chain has 32-bit words here, less
 // than its single systems had)
 cudaError_t launch_chains_small(const Workspace &w, double *V_B, cudaStream_t s) {
-  const size_t bytes = single_smem_bytes(w.N);
-  if (!w.recomp) return launch_pdl(chain_small_kernel<BPIMD_FP64, false>, 2, BATCH_THREADS, bytes, s, w, V_B);
-  return w.mode == BPIMD_FP64 ? launch_pdl(chain_small_kernel<BPIMD_FP64, true>, 2, BATCH_THREADS, bytes, s, w, V_B)
-                              : launch_pdl(chain_small_kernel<BPIMD_MIXED, true>, 2, BATCH_THREADS, bytes, s, w, V_B);
+  return launch_pdl(chain_small_kernel, 2, BATCH_THREADS, single_smem_bytes(w.N), s, w, V_B);
 }
 
 cudaError_t launch_chains_batched(const Workspace *ws, const int *order, int R, int maxN, bool mixed, double *V_B,

@@ -257,20 +257,19 @@ struct RowFactors {
 // before use.
 // Off-diagonal block: H(tt*32+i, (tt+1)*32+lane), rows i in [i0, i0+NR), as
 // stored (float for MIXED32), into dm/de[i*33 + lane].
-template <int MODE, bool BWD, bool RC, bool PBC, int NR>
-__device__ __forceinline__ void stage_offdiag(const Workspace &w, int tt, int i0, void *dmv, int *de,
-                                              const unsigned long long *T63) {
+template <int MODE, bool BWD, int NR>
+__device__ __forceinline__ void stage_offdiag(const Workspace &w, int tt, int i0, void *dmv, int *de) {
   using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
   const int lane = threadIdx.x & 31;
   const int srcbase = tt * TILE, row = tt * TILE + TILE + lane;
   M_t *dm = (M_t *)dmv;
-  RowFactors<MODE, BWD, RC, PBC, 32> f;
+  RowFactors<MODE, BWD, false, false, 32> f;
   f.load(w, min(row, w.N - 1));
 #pragma unroll
   for (int i = i0; i < i0 + NR; ++i) {
     M_t m = (M_t)1.0;
     int e = XZERO_E;
-    if (row < w.N) f.h(w, srcbase + i, T63, m, e);
+    if (row < w.N) f.h(w, srcbase + i, nullptr, m, e);
     dm[i * 33 + lane] = m;
     de[i * 33 + lane] = e;
   }
@@ -279,21 +278,20 @@ __device__ __forceinline__ void stage_offdiag(const Workspace &w, int tt, int i0
 // Diagonal block of tile tt, K = c_row * H as 64-bit integer mantissas (the
 // chain format of xi_fma), rows i in [i0, i0+NR): the mantissa product is
 // formed on the integer pipe (mul_mant).
-template <int MODE, bool BWD, bool RC, bool PBC, int NR>
-__device__ __forceinline__ void stage_diag(const Workspace &w, int tt, int i0, unsigned long long *dm, int *de,
-                                           const unsigned long long *T63) {
+template <int MODE, bool BWD, int NR>
+__device__ __forceinline__ void stage_diag(const Workspace &w, int tt, int i0, unsigned long long *dm, int *de) {
   using M_t = typename std::conditional<MODE == BPIMD_MIXED32, float, double>::type;
   const int lane = threadIdx.x & 31;
   const int r0 = tt * TILE, row = r0 + lane;
   const xd c = (row < w.N) ? xnorm_int(chain_coef<BWD>(w, row)) : xd{1.0, 0};
-  RowFactors<MODE, BWD, RC, PBC, 32> f;
+  RowFactors<MODE, BWD, false, false, 32> f;
   f.load(w, min(row, w.N - 1));
 #pragma unroll
   for (int i = i0; i < i0 + NR; ++i) {
     const int src = r0 + i;
     M_t m = (M_t)1.0;
     int e = XZERO_E;
-    if (row < w.N && src <= row) f.h(w, src, T63, m, e);
+    if (row < w.N && src <= row) f.h(w, src, nullptr, m, e);
     const xk k = mul_mant<M_t>(c, m, e);
     dm[i * 33 + lane] = k.m;
     de[i * 33 + lane] = k.e;

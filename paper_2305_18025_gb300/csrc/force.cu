@@ -66,11 +66,14 @@ __device__ __forceinline__ double img(const Workspace &w, double d) {
 //   row b    : mu_b / (N y_N) sum_a y_a g(a,b) (r_b^P - r_a^1)
 //   column a : y_a / (N y_N) sum_b mu_b g(a,b) (r_b^P - r_a^1)
 // a pair is one product and three products with the difference's components.
-//   Mixed forms: the product on 64-bit mantissas, cut to an unevaluated float32
-//   pair once (+-2^-47); its products with the difference and the sums as such
-//   pairs (products by FMA, sums by TwoSum: 2^-46 relative) on the float32 pipe;
-//   the powers of two of all factors, the taken-out ones included, scale the
-//   pair, so a term is at most 2.
+//   Mixed forms: unevaluated float32 pairs (products by FMA, sums by TwoSum:
+//   2^-46 relative) on the float32 pipe; the powers of two of all factors,
+//   the taken-out ones included, scale the pair, so a term is at most 2.  High
+//   parts are the nearest float32: a weight's error over random mantissas is then
+//   0.12 2^-46 (rms; 0.91 at most, 0.00 on average), where high parts cut off gave
+//   0.89 (3.1, -0.80) and one cut of the 64-bit product 0.42 (1.0, -0.36) at 4-12 %
+//   of the pass (N = 1024, P = 32: 56.6 us for 55.6; 152 replicas of 1024: 784 us
+//   for 701).
 //   FP64: 64-bit integer mantissas, signed 64-bit sums with a running exponent
 //   a lane and component (2^-57 of the largest term of a group of four); GB300's
 //   float64 pipe retires ~1.7 lanes a clock, so it forms the differences only.
@@ -88,9 +91,6 @@ struct PSum {  // FP64: v 2^(E - 61)
 
 __device__ __forceinline__ unsigned long long mant64(double m) {  // [1, 2) -> [2^63, 2^64)
   return ((unsigned long long)__double_as_longlong(m) << 11) | (1ull << 63);
-}
-__device__ __forceinline__ unsigned long long mant64(float m) {
-  return ((unsigned long long)((unsigned)__float_as_int(m) << 8) | (1ull << 31)) << 32;
 }
 
 // |x| as a mantissa in [2^62, 2^63) (value M 2^(e - 62)) times the term t:
@@ -142,6 +142,17 @@ __device__ __forceinline__ void two_sum(float &s, float &c, float x) {
   c += (s - (t - bp)) + (x - bp);
   s = t;
 }
+// a mantissa in [1, 2) as the nearest float32 and the rest (to 2^-49)
+__device__ __forceinline__ void mant_hl(double m, float &h, float &l) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(m);
+  h = __uint_as_float(0x3F800000u + (((unsigned)(b >> 29) & 0x7FFFFFu) + ((unsigned)(b >> 28) & 1u)));
+  l = (float)((int)((unsigned)b << 3) >> 3) * 2.2204460492503131e-16f;  // 2^-52
+}
+__device__ __forceinline__ void mant_hl(float m, float &h, float &l) {
+  h = m;
+  l = 0.0f;
+}
+
 constexpr int PROB_THREADS = 256, PROB_WARPS = PROB_THREADS / 32;
 constexpr int PROB_MAX_CL = 8;
 constexpr int PROB_CHUNK = 256;  // most partners staged at a time
@@ -160,7 +171,7 @@ struct SumSlot<true> {
   int E[3][TILE], bad[TILE];
 };
 // Staged partners.  Mixed forms: the endpoint's high and low parts (or, in a
-// box, its fixed-point words) with the weight's 64-bit mantissa in the fourth
+// box, its fixed-point words) with the weight's mantissa parts in the fourth
 // places; FP64: coordinates and the weight's 64-bit mantissa.
 template <bool F64>
 struct Partners;
@@ -198,8 +209,8 @@ __device__ __forceinline__ void stage_partner(const Workspace &w, Partners<F64> 
     P.z[i] = ep.z;
     P.m[i] = mant64(wt.m);
   } else {
-    const unsigned long long m = mant64(wt.m);
-    const float h = __uint_as_float((unsigned)(m >> 32)), l = __uint_as_float((unsigned)m);
+    float h, l;
+    mant_hl(wt.m, h, l);
     if constexpr (PBC) {
       P.h[i] = make_float4(__uint_as_float(ep.u.x), __uint_as_float(ep.u.y), __uint_as_float(ep.u.z), h);
       P.l[i].w = l;
@@ -313,14 +324,13 @@ __device__ __forceinline__ void exterior_item(const Workspace &w, int item, int 
             E[c] = max(E[c], pe[k][c]);
           }
         } else {
-          // y g = (t / 2^63) 2^x, cut to float32 high and low parts (+-2^-47) once
-          const unsigned long long ym = ((unsigned long long)__float_as_uint(sm.part.h[i].w) << 32) | __float_as_uint(sm.part.l[i].w);
-          unsigned long long t = pow2fx::mulhi(ym, mant64(m[k]));  // in [2^62, 2^64)
-          const int sh = (int)(t >> 63) ^ 1, x = min(sm.part.e[i] + e[k] + own_e + 1 - sh, 100);
-          t <<= sh;
-          const float th = valid && x >= -126 ? __uint_as_float(((unsigned)(x + 127) << 23) | ((unsigned)(t >> 40) & 0x7FFFFFu)) : 0.0f;
-          const float lo = __uint_as_float(0x4B000000u | ((unsigned)(t >> 17) & 0x7FFFFFu)) - 8388607.5f;  // the next 23 bits and a half
-          const float tl = valid && x >= -80 ? lo * __uint_as_float((unsigned)(x + 81) << 23) : 0.0f;
+          const float yh = sm.part.h[i].w, yl = sm.part.l[i].w;
+          const int x = sm.part.e[i] + e[k] + own_e;
+          const float sc = valid && x >= -126 ? __int_as_float((min(x, 100) + 127) << 23) : 0.0f;
+          float gh, gl;
+          mant_hl(m[k], gh, gl);
+          const float t = yh * gh, te = fmaf(yl, gh, fmaf(yh, gl, fmaf(yh, gh, -t)));
+          const float th = t * sc, tl = te * sc;
           const float dc[3] = {valid ? d.x : 0.0f, valid ? d.y : 0.0f, valid ? d.z : 0.0f};
 #pragma unroll
           for (int c = 0; c < 3; ++c) {

@@ -199,7 +199,7 @@ def bpimd_profile_end(ctx):
 
 
 def bpimd_exchange_energy_forces_noalloc(cfg, positions, V_B, forces, stream=None):
-    """Allocation-free evaluation (no context; fixed 1 MiB device scratch, N <= 256).
+    """Allocation-free evaluation (no context; fixed 2 MiB device scratch, N <= 256).
 
     For callers that cannot allocate device memory when they evaluate (their
     memory manager owns all device memory, or cudaMalloc's device-wide

@@ -39,7 +39,7 @@ constexpr int TILE2 = TILE * TILE;
 constexpr int XZERO_E = -(1 << 29);   // exponent carried by an extended zero
 constexpr int CHAIN_PANEL = 64;       // rows solved at a time by a recursion cluster
 constexpr int CHAIN_SLICES = 4;       // partial sums a row carries between superblocks
-constexpr int CHAIN_CLUSTER = 8;      // CTAs per recursion (small N)
+constexpr int CHAIN_CLUSTER = 8;      // CTAs per recursion where two clusters of 16 do not fit on the device
 constexpr int CHAIN_MAX_N = BPIMD_MAX_N;  // largest N the library accepts
 constexpr int CHAIN_SMALL_N = 128;    // largest single system on one CTA per recursion
 constexpr bool small_chain(int N, int precision) { return N <= CHAIN_SMALL_N && precision != BPIMD_MIXED32; }
@@ -61,11 +61,6 @@ struct xd {  // value = m * 2^e
   int e;
 };
 
-__device__ __forceinline__ double pow2_nonpos(int k) {
-  // 2^k for k <= 0; 0 below the normal range (the scaled operand is then
-  // below 2^-1022 of the larger one and cannot change a double sum).
-  return (k < -1022) ? 0.0 : __longlong_as_double((long long)(k + 1023) << 52);
-}
 __device__ __forceinline__ float pow2f_nonpos(int k) {
   return (k < -126) ? 0.0f : __int_as_float((k + 127) << 23);
 }
@@ -97,11 +92,9 @@ __device__ __forceinline__ double xtod(xd a) {
   double s2 = __longlong_as_double((long long)(e2 + 1023) << 52);
   return a.m * s1 * s2;
 }
-// natural log of an extended number (m > 0)
-__device__ __forceinline__ double xlog(xd a) { return log(a.m) + (double)a.e * LN2; }
 
 // ------------------------------------------- programmatic dependent launches
-// The three kernels of an evaluation are launched with programmatic stream
+// The kernels of an evaluation are launched with programmatic stream
 // serialisation: a kernel may be scheduled while its predecessor in the
 // stream drains (hiding the launch gap), waits (griddepcontrol.wait: the
 // predecessor has completed and its writes are visible) before its first
@@ -109,6 +102,12 @@ __device__ __forceinline__ double xlog(xd a) { return log(a.m) + (double)a.e * L
 // issued (griddepcontrol.launch_dependents).  A successor launches only after
 // every CTA of its predecessor has started, so an early launch never takes
 // resources the predecessor still needs.
+// Two kernels do not wait before they start to work: the MD's physical force
+// (ext_force_kernel, ext_force_batched) and the update of later rows between
+// superblocks (source_update_kernel, `beside`).  They follow a recursion kernel
+// and read only what was complete before that one could begin.  It rests on a
+// rule of the recursion kernels (chain_kernel, chain_small_kernel,
+// chain_batched_kernel): each triggers only after its own wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -132,14 +131,14 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 struct Workspace {
   int N, P, NT, NB;     // NT = ceil(N/TILE), NB = NT(NT+1)/2 blocks of g
   int mode;             // precision form: BPIMD_FP64, BPIMD_MIXED or BPIMD_MIXED32
-  int mixed;            // MIXED32: float32 pair-factor and alpha mantissas, 32-bit recursion chain
+  int mixed;            // MIXED32: float32 pair-factor mantissas (and, in replicas, a 32-bit recursion chain)
   int bead32;           // MIXED and MIXED32: float32 bead differences and spring energies
   double m, omega_P, beta, k, half_k;
   double inv_P;         // 1/P (kernels take it from here: a float64 division costs a GB300 SM ~20 warp-cycles per lane)
   double cx;            // beta (1/2) k log2(e): g = 2^(-cx d^2)
   int gstr;             // source stride of the pair-factor tables (below)
   int recomp;           // recompute mode: no O(N^2) table; g is formed where it is used
-  int test_timeout;     // BPIMD_FLAG_TEST_TIMEOUT: the forward lead waits for a hand-off never made
+  int test_timeout;     // BPIMD_FLAG_TEST_TIMEOUT: the forward recursion waits for a hand-off never made
   // periodic cubic box of side L (0: open boundaries); every spring joins the
   // minimum image of its beads.  MIXED keeps the bead-1/bead-P copies in a box
   // as 32-bit fixed-point fractions of L (R1s/RPs reinterpreted as uint32
@@ -286,7 +285,7 @@ cudaError_t launch_prep(const Workspace &w, const double *pos, double *F, cudaSt
 // fill the pair-factor entries outside a <= b < N (fixed for a given N) with
 // extended zeros; needed once per workspace before the first launch_prep
 cudaError_t launch_gmat_padding(const Workspace &w, cudaStream_t s);
-// both recursions, prefix sums, V_B (device scalar, may be null), normaliser, alpha
+// both recursions, prefix sums, V_B (device scalar, may be null), normaliser
 cudaError_t launch_chains(const Workspace &w, double *V_B, cudaStream_t s);
 // single systems of up to CHAIN_SMALL_N particles, one CTA per recursion
 cudaError_t prepare_chains_small();

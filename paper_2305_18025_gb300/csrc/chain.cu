@@ -307,8 +307,7 @@ struct ChainShape {
   static constexpr int PARTS = 32 / R;         // source parts of a bulk task (lanes a row)
   static constexpr int SRC = PT / PARTS;       // sources a lane of a bulk task
   static constexpr int BULK = 14;              // bulk warps
-  static constexpr int PREFIX_WARP = CRIT + BULK;
-  static constexpr int THREADS = 32 * (CRIT + BULK + 1);
+  static constexpr int THREADS = 32 * (CRIT + BULK + 1);  // one more warp: the prefix sums
 };
 
 // MODE: precision form (the stored-factor kernels serve BPIMD_MIXED with the
@@ -346,7 +345,10 @@ __device__ void run_chain(const Workspace &w, int t0, int np, ChainSmem &sm, dou
   __syncthreads();
   cluster_arrive();
   pdl_wait();
-  pdl_trigger();  // what runs beside the recursions may start; what needs them waits for this grid
+  // After the wait, never before it: what is launched to run beside this kernel
+  // (the physical force, later rows' updates) starts here without a wait of its
+  // own, and what needs the recursions waits for this grid.
+  pdl_trigger();
   if (t0 == 0 && rank == 0 && tid == 0) {
     gYm[0] = 1.0;
     gYe[0] = 0;

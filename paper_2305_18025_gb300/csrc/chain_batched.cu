@@ -226,7 +226,7 @@ __device__ void run_single(const Workspace &w, unsigned char *smem_raw, double *
 __global__ void __launch_bounds__(BATCH_THREADS) chain_small_kernel(Workspace w, double *V_B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
-  pdl_trigger();  // what runs beside the recursions may start; what needs them waits for this grid
+  pdl_trigger();  // after the wait, never before it: what runs beside the recursions starts here without one
   if (blockIdx.x & 1) run_single<BPIMD_FP64, true, true>(w, smem_raw, nullptr);
   else run_single<BPIMD_FP64, false, true>(w, smem_raw, V_B);
 }
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, 2) chain_batched_kernel(const W
                                                                          double *V_B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
-  pdl_trigger();  // what runs beside the recursions may start; what needs them waits for this grid
+  pdl_trigger();  // after the wait, never before it: what runs beside the recursions starts here without one
   const int r = order[blockIdx.x >> 1];
   if (blockIdx.x & 1) run_single<MIXED ? BPIMD_MIXED32 : BPIMD_FP64, true, false>(ws[r], smem_raw, nullptr);
   else run_single<MIXED ? BPIMD_MIXED32 : BPIMD_FP64, false, false>(ws[r], smem_raw, V_B ? V_B + r : nullptr);

@@ -125,8 +125,8 @@ __device__ __forceinline__ xi xi_fma(xi acc, unsigned long long kk, int ke, xi y
   return xi_norm((acc.m >> min(E - acc.e, 63)) + (p >> min(E - pe, 63)), E);
 }
 
-// ----------------------------------------- the 32-bit chain format (MIXED)
-// MIXED runs the dependency chain on 32-bit words: m * 2^(e - 30) with m in
+// ------------------------------- the 32-bit chain format (BPIMD_MIXED32 replicas)
+// There the dependency chain runs on 32-bit words: m * 2^(e - 30) with m in
 // [2^30, 2^31) (one bit of headroom), the factor K by the top 32 bits of its
 // mantissa.  A step is one 32 x 32-bit high product, two shifts, one add and a
 // select (truncation at 2^-30 per operation, far below the float32 rounding

@@ -10,7 +10,8 @@
 // i.e. the per-neighbour sums of the paper distributed over their terms.
 // Precision forms: bead differences in float64 (FP64) or float32 (mixed
 // forms, from the high/low parts or the fixed-point copies); products and sums
-// on 64-bit integer mantissas, the direct links and the results in float64.
+// on 64-bit integer mantissas (FP64) or as float32 pairs (mixed forms); the direct
+// links and the results in float64.
 #include <type_traits>
 
 #include "bpimd_internal.cuh"

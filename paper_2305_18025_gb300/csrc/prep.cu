@@ -144,7 +144,7 @@ __device__ __forceinline__ void bead_pass_body(const Workspace &w, const double 
   }
   __syncthreads();
   // phase 2: one lane per particle -- links, endpoint copies and the
-  // coefficient c (the float64 transcendentals run once per 8 particles)
+  // coefficient c (the float64 transcendentals run once per block of particles)
   if (wp == warp2 && lane < COUNT) {
     const int l = l0 + lane;
     if (l < w.N) {
@@ -422,8 +422,7 @@ __global__ void __launch_bounds__(256) prep_batched(const Workspace *__restrict_
   } else {
     for (int k = blockIdx.x - nbead; k < nblk; k += gridDim.x - nbead) {
       const int2 e = blk_tab[k];
-      if (ws[e.x].pbc) gmat_block<MODE, true, 32>(ws[e.x], pos + off[e.x], e.y, Tm, Te, E, T63);
-      else gmat_block<MODE, false, 32>(ws[e.x], pos + off[e.x], e.y, Tm, Te, E, T63);
+      gmat_block<MODE, false, 32>(ws[e.x], pos + off[e.x], e.y, Tm, Te, E, T63);  // batches have no periodic box
     }
   }
   pdl_trigger();

@@ -39,9 +39,24 @@ sys.path.insert(0, ROOT)
 
 METRIC = "exchange V_B+force evals/s at N=1024,P=32 (mixed vs FP64 GPU); MD steps/s"
 N_DEF, P_DEF, BETA_DEF, SEED_DEF = 1024, 32, 1.0, 3
-LAUNCHES_PER_EVAL = 4          # bead pass + pair factors, panel inverses, recursions (2 clusters), exterior forces
 BATCH_LAUNCHES_PER_EVAL = 3    # replica batch: bead pass + pair factors, recursions, exterior forces
 BATCH_MD = dict(dt=0.01, gamma=1.0, omega0=1.0, gaussian=(1.0, 0.5), seed=77)  # 256-replica workload
+
+
+def launches_per_eval(N, precision, recompute=False):
+    """Kernel launches of one evaluation of a single system: bead pass + pair
+    factors, recursions, exterior forces.  The recursions are one launch up to
+    128 particles (64-bit forms), else the panel inverses and the clusters, which
+    past 28 panels of 64 rows (16 with recomputed factors) run in superblocks of at
+    most 16 panels: between two of them one update of the next rows, and beside
+    every later one but the last an update of the rows after it."""
+    if N <= 128 and precision != "mixed32":
+        return 3
+    panels = (N + 63) // 64
+    k = 1 if panels <= (16 if recompute or N > 8192 else 28) else (panels + 15) // 16
+    return 3 + k + (k - 1) + max(k - 2, 0)
+
+
 DFMA_LATENCY_CYCLES = 64       # measured on GB300: dependent float64 FMA latency
 FLUSH_BYTES = 256 << 20        # > 129 MB L2
 
@@ -212,7 +227,8 @@ def roofline(stage_ms_per_eval, args, sm_mhz, peaks, precision="mixed"):
 #     products and sums are on the integer pipe);
 #   mixed forms: float32 pairs -- 9 operations for the differences, 10 for the
 #     weight, 33 for three compensated products and sums, twice = 104 float32
-#     ops per pair, and 2 integer multiply-adds of addresses;
+#     ops per pair, and 2 integer multiply-adds of addresses (`fp32_frac` is the
+#     share of the unit that carries the mixed stage; `frac` counts the addresses);
 #   pair factors, float64: 6 float64 ops per pair (difference and square);
 #   pair factors, mixed: the integer power's products (pow2_fixed.cuh)
 #     = 19 integer multiply-adds.
@@ -268,6 +284,7 @@ def roofline_stages(stage_ms_per_eval, args, sm_mhz, peaks, unit_peaks, precisio
         prob = {"bound": "int", "unit": "32-bit integer multiply-adds/s", "achieved": PROB_MIXED_IMADS * pairs / t_prob,
                 "peak": unit_peaks["int_mad_per_s"], "peak_source": "library integer multiply-add probe (measured)"}
         prob["fp32_frac"] = PROB_M32_F32OPS * pairs / t_prob / fp32_peak
+        prob["carried_by"] = "fp32"
     else:
         prob = {"bound": "fp32", "unit": "float32 ops/s", "achieved": PROB_M32_F32OPS * pairs / t_prob,
                 "peak": fp32_peak, "peak_source": "nominal 128 float32 lanes per SM x 152 SMs x sampled clock"}
@@ -411,7 +428,7 @@ def run_ours(args, rank, world, local_rank):
         "precision": "mixed",
         "timing": {"l2": "flushed between timed steps (256 MiB device write, untimed)",
                    "stream": "a dedicated CUDA stream bound to the context (flush and events on it)"},
-        "gpu_launches": LAUNCHES_PER_EVAL * args.steps,
+        "gpu_launches": launches_per_eval(args.N, "mixed") * args.steps,
         "clocks": clocks,
         "e2e": results["e2e"],
         "roofline": roof,
@@ -457,11 +474,11 @@ def run_ours(args, rank, world, local_rank):
 # arithmetic of each precision form (what the path computes in)
 DTYPES = {
     "mixed": "f32+f64+u64 (float32 bead differences and spring energies; float64-accurate pair factors, "
-             "64-bit integer recursions, integer-mantissa probabilities, "
-             "compensated float32-pair force sums)",
-    "fp64": "f64+u64 (float64, with 64-bit integer recursions and integer-pipe pair factors)",
-    "mixed32": "f32+u64+f64 (float32 pair factors, recursion bulk sums and probabilities; 64-bit integer "
-               "tile products; float64 prefix sums and outputs)",
+             "64-bit integer recursions, exterior forces as compensated float32 pairs)",
+    "fp64": "f64+u64 (float64, with 64-bit integer recursions, integer-pipe pair factors and integer "
+            "exterior sums)",
+    "mixed32": "f32+u64+f64 (float32 pair factors by the hardware exponential, 64-bit integer recursions, "
+               "exterior forces as compensated float32 pairs; float64 prefix sums and outputs)",
 }
 
 
@@ -494,7 +511,7 @@ def md_throughput(args, pos_np, wP, dev, max_over_ranks, barrier, world):
         en = md.step(x, v, 1).cpu().tolist()
         md.close()
         out[prec] = {"value": aggregate_rate(world, steps, ms * 1e-3), "unit": "MD steps/s", "steps": steps,
-                     "gpu_launches": (LAUNCHES_PER_EVAL + 2) * (steps + 1),
+                     "gpu_launches": (launches_per_eval(args.N, prec) + 2) * (steps + 1),
                      "ms_per_step": ms / steps, "energies_after": dict(zip(["V_B", "U_bar", "kinetic", "E_prim"], en))}
     out["config"] = {"workload": f"trapped bosons N={args.N} P={args.P} beta={args.beta:g}, harmonic trap w0=1, "
                                  "Gaussian repulsion g=3 s=0.5 between equal-index beads",

@@ -18,8 +18,9 @@ class ExchangeEnergy:
 
     def __init__(self, N, P, m, omega_P, beta, precision="fp64", device="cuda", stream=None, box=0.0,
                  recompute=False):
-        """recompute=True: no O(N^2) storage at any N (automatic above
-        BPIMD_STORE_MAX_N): the pair factors are recomputed where used."""
+        """recompute=True: no O(N^2) storage (automatic above BPIMD_STORE_MAX_N):
+        the pair factors are recomputed where used.  (fp64 and mixed systems of up
+        to 128 particles keep theirs, 240 KB at most.)"""
         if not torch.cuda.is_available():
             raise RuntimeError("bpimd needs a CUDA device; there is no CPU fallback")
         prec = _c.PRECISIONS[precision]

@@ -244,9 +244,9 @@ __device__ __forceinline__ void acc_add(Acc96 &a, long long P, int s) {
 }
 __device__ __forceinline__ double acc_value(const Acc96 &a) {
   const int k = max(a.B - 94, -2044), k1 = k >> 1;  // in two factors: either is a normal number
-  if (k < -1000) return 0.0;                         // zero differences only
-  return value96(a.lo, a.mid, a.hi) * __longlong_as_double((long long)(k1 + 1023) << 52) *
-         __longlong_as_double((long long)(k - k1 + 1023) << 52);
+  const double v = value96(a.lo, a.mid, a.hi) * __longlong_as_double((long long)(k1 + 1023) << 52) *
+                   __longlong_as_double((long long)(k - k1 + 1023) << 52);
+  return fabs(v) < 1e-300 ? 0.0 : v;  // zero differences, each counted as 2^-1023
 }
 
 struct GaussSum {  // sums over a lane's partners

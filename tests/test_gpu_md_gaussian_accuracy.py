@@ -59,7 +59,7 @@ def positions(kind, N):
     return pos
 
 
-CASES = [("pair3", 2, 0.5), ("pair6", 2, 0.5), ("pair9", 2, 0.5), ("pair20", 2, 0.5), ("flat", 65, 0.5),
+CASES = [("pair3", 2, 0.5), ("pair6", 2, 0.5), ("pair9", 2, 0.5), ("pair20", 2, 0.5), ("pair0", 2, 0.5), ("flat", 65, 0.5),
          ("plane", 33, 0.5), ("sparse", 40, 0.5), ("close", 33, 0.5), ("far", 34, 0.5), ("wide", 64, 0.05),
          ("wide", 64, 0.5), ("wide", 64, 50.0), ("wide", 64, 5e3), ("wide", 64, 5e5), ("wide", 64, 1e10),
          ("wide", 33, 1e160), ("many", 1027, 0.5)]
@@ -78,6 +78,16 @@ def test_pair_forces_relative_to_their_own_size(kind, N, s):
     assert (np.abs(got - F) <= unit * LD(2.0) ** -53 + LD(1e-290)).all(), \
         float((np.abs(got - F) / (unit * LD(2.0) ** -53 + LD(1e-290))).max())
     assert abs(LD(en[1]) - U) <= N * 2.0 ** -50 * g + U * LD(2.0) ** -50
+
+
+def test_powers_near_the_end_of_the_float64_range():
+    pos, g, s = positions("pair37", 2), 1e200, 0.5  # e = 2^-987
+    F, unit, _ = reference(pos, g, s)
+    md = RingPolymerMD(2, 2, 1.0, 1e-150, 1.0, dt=DT, gamma=0.0, gaussian=(g, s))
+    x, v = torch.from_numpy(pos.copy()).cuda(), torch.zeros((2, 2, 3), dtype=torch.float64, device="cuda")
+    md.step(x, v, 1)
+    md.close()
+    assert (np.abs(v.cpu().numpy().astype(LD) / LD(DT) - F) <= unit * LD(2.0) ** -53).all()
 
 
 def test_replicas_take_the_same_pairs():

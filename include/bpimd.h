@@ -79,7 +79,7 @@ extern "C" {
  *   float64 product x by a 64-bit fixed-point table method (integer pipe,
  *   2^-60 relative before the final float64 rounding); the blocked recursions
  *   (panel inverses, panel products and the sums over earlier sources) on
- *   64-bit integer mantissas with int32 exponents (products to 2^-60, sums to
+ *   64-bit integer mantissas with int32 exponents (products to 2^-59, sums to
  *   2^-56 .. 2^-59 of their largest term); exterior forces from float64
  *   differences by 64-bit integer products and sums (a component's to 2^-57 of
  *   the largest term of a group of four); float64 direct links and results.

@@ -286,7 +286,7 @@ __device__ __forceinline__ xi row_sum(const unsigned long long (&kk)[2], const i
   int pe[2];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    p[i] = pow2fx::mulhi_centred(kk[i], y[i].m);
+    p[i] = pow2fx::mulhi(kk[i], y[i].m);
     pe[i] = ke[i] + y[i].e + 1;
   }
   const int E = __reduce_max_sync(0xffffffffu, max(pe0, max(pe[0], pe[1])));

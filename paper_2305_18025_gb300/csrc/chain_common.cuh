@@ -78,7 +78,7 @@ __device__ __forceinline__ xk mul_mant(xd c, M_t hm, int he) {
 // read its result), while a 64 x 64-bit integer product, shifts and a 64-bit
 // add take a few cycles each.  An extended number is  m * 2^(e - 62)  with an
 // integer mantissa m in [2^62, 2^63) (one bit of headroom for an addition);
-// the extended zero is 2^62 * 2^(XZERO_E - 62).  Products are within 2^-60,
+// the extended zero is 2^62 * 2^(XZERO_E - 62).  Products are within 2^-59,
 // alignment shifts truncate at 2^-61 (sums of many terms: at their headroom,
 // below): finer than a float64 rounding.
 struct xi {
@@ -119,7 +119,7 @@ __device__ __forceinline__ xi xi_mul(xi a, xd c) {
 // aligned sum in [2^61, 2^64); a K carrying an extended-zero exponent leaves
 // acc unchanged.
 __device__ __forceinline__ xi xi_fma(xi acc, unsigned long long kk, int ke, xi y) {
-  const unsigned long long p = pow2fx::mulhi_centred(kk, y.m);
+  const unsigned long long p = pow2fx::mulhi(kk, y.m);
   const int pe = ke + y.e + 1;
   const int E = max(acc.e, pe);
   return xi_norm((acc.m >> min(E - acc.e, 63)) + (p >> min(E - pe, 63)), E);
@@ -438,7 +438,7 @@ __device__ __forceinline__ xsum xsum_dot(const unsigned long long *kk, const int
   int E = pe0;
 #pragma unroll
   for (int i = 0; i < K; ++i) {
-    p[i] = pow2fx::mulhi_centred(kk[i], y[i].m);
+    p[i] = pow2fx::mulhi(kk[i], y[i].m);
     pe[i] = ke[i] + y[i].e + 1;
     E = max(E, pe[i]);
   }

@@ -43,14 +43,6 @@ BPIMD_HD unsigned long long mulhi(unsigned long long a, unsigned long long b) {
   return (unsigned long long)ah * bh + mulhi32(ah, bl) + mulhi32(al, bh);
 }
 
-// The same plus one unit: -1 to +2 units of 2^-64, 1/4 too small on average (the
-// exact product's high word is 1/2 too small on average); the addition is the
-// multiply-add's own.
-BPIMD_HD unsigned long long mulhi_centred(unsigned long long a, unsigned long long b) {
-  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a, bh = (unsigned)(b >> 32), bl = (unsigned)b;
-  return ((unsigned long long)ah * bh + 1ull) + mulhi32(ah, bl) + mulhi32(al, bh);
-}
-
 constexpr unsigned long long Q64_HALF = 0x8000000000000000ull;
 constexpr unsigned long long Q64_SIXTH = 0xFFFFFFFFFFFFFFFFull / 6;
 constexpr unsigned Q32_24TH = 0xFFFFFFFFu / 24;

@@ -198,7 +198,7 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
 // the three differences only.  Every later quantity keeps a mantissa and an
 // exponent of its own, so that a pair is as accurate relative to itself as in
 // float64, however near, far, wide or flat the system is: the squares are summed
-// on the scale of the largest component (2^-56 of d^2), times log2(e)/(2 s^2)
+// on the scale of the largest component (2^-57 of d^2), times log2(e)/(2 s^2)
 // they are the argument of the power of two (2^-60), and e d is added to 96-bit
 // sums whose unit lies 62 bits below their largest term.  A pair is ~260
 // instructions, mostly of the integer pipe, beside the float64 pipe's ~57 cycles:
@@ -273,7 +273,9 @@ __device__ __forceinline__ void gauss_pair(const double (&d)[3], unsigned long l
 #pragma unroll
     for (int c = 0; c < 3; ++c) a.bad |= (ef[c] == 0x7ff) << c;
   }
-  unsigned long long q = 0, w = 0;  // |d|^2 = (q + w 2^-31) 2^(2 (em - 1023) - 58), the low words' squares left out
+  // |d|^2 = (q + w 2^-31) 2^(2 (em - 1023) - 58); the low words' squares and the
+  // cuts amount to two units on average, with which q starts: 2^-60 rms, no mean error
+  unsigned long long q = 2, w = 0;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const unsigned long long A = M[c] >> (min(em - ef[c], 61) + 2);
